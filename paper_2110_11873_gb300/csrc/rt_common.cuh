@@ -68,7 +68,8 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 constexpr int kBlockVec = 512;          // threads per block of the vector kernels
 constexpr int kMaxPartials = 2048;      // upper bound on reduction partials per column
 constexpr int kMaxRestart = 160;         // longest GMRES cycle (the paper runs GMRES unrestarted, up to 134 steps)
-constexpr int kGramB = 4;                // basis vectors per block pass of the GMRES Arnoldi step
+constexpr int kGramB = 4;                // basis vectors per block pass of rt_arnoldi_bmgs and of the batch
+constexpr int kGramMax = 8;              // basis vectors per block pass inside the single-instance GMRES
 
 // device-side state of a GMRES cycle (lives in device memory).  The scalars
 // come first: the host reads only that header (kGmresHeader bytes) after a
@@ -87,7 +88,7 @@ struct GmresDev {
   double cs[kMaxRestart], sn[kMaxRestart];
   double g[kMaxRestart + 1];
   double y[kMaxRestart];
-  double gram[(kMaxRestart + 1) * kGramB];   // gram[i*kGramB + d] = <v_i, v_{i-d}>, d = 1..kGramB-1
+  double gram[(kMaxRestart + 1) * kGramMax];  // gram[i*B + d] = <v_i, v_{i-d}>, d = 1..B-1, B the block size
 };
 constexpr size_t kGmresHeader = offsetof(GmresDev, H);
 
@@ -100,13 +101,15 @@ constexpr size_t kGmresHeader = offsetof(GmresDev, H);
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// launch as a programmatic dependent of the stream's previous kernel
+// launch as a programmatic dependent of the stream's previous kernel, with
+// dynamic shared memory
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t st, Args... args) {
+inline cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
+                                   Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -116,12 +119,28 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cud
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// sum of G partials in a fixed order (lane-strided, then a fixed shuffle
-// tree); every lane of the calling warp gets the result
+// the same without dynamic shared memory
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t st, Args... args) {
+  return launch_pdl_smem(kernel, grid, block, 0, st, args...);
+}
+
+// sum of G partials in a fixed order (lane-strided trees, then a fixed
+// shuffle tree); every lane of the calling warp gets the result
 __device__ __forceinline__ double partials_sum_warp(const double* __restrict__ part, int G) {
   const int lane = threadIdx.x & 31;
+  constexpr int U = 8;   // loads in flight per lane, added as a tree
   double s = 0.0;
-  for (int i = lane; i < G; i += 32) s += part[i];
+  for (int i0 = lane; i0 < G; i0 += 32 * U) {
+    double v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = i0 + 32 * u < G ? part[i0 + 32 * u] : 0.0;
+#pragma unroll
+    for (int o = U / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < o; ++u) v[u] += v[u + o];
+    s += v[0];
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s;
@@ -160,13 +179,14 @@ __device__ inline void givens_step(GmresDev* gm, int m, int j, double* hist, int
 
 // End of Arnoldi step j from the last block pass's partials (Gp per set; set
 // 0: ||w||^2, set 1+k: <w, v_{i0+k}>, k < ng): h_{j+1,j} = ||w|| to
-// hcol[j+1], the Gram row j+1 (<v_{j+1}, v_{j+1-d}>, d = ng - k), and with
+// hcol[j+1], the Gram row j+1 (<v_{j+1}, v_{j+1-d}>, d = ng - k; rows of gb
+// entries), and with
 // gm set the Givens rotations of column j.  One CTA of at least 32*(1+ng)
 // threads; thread 0 does the scalar work.
 __device__ inline void arnoldi_fold(const double* __restrict__ part, int Gp, int ng, double* __restrict__ hcol,
-                                    double* __restrict__ gram, GmresDev* gm, int m, int j, double* hist,
+                                    double* __restrict__ gram, int gb, GmresDev* gm, int m, int j, double* hist,
                                     int hist_cap) {
-  __shared__ double sets[kGramB];
+  __shared__ double sets[kGramMax];
   const int warp = threadIdx.x >> 5;
   if (warp <= ng) {
     const double s = partials_sum_warp(part + (size_t)warp * Gp, Gp);
@@ -177,7 +197,7 @@ __device__ inline void arnoldi_fold(const double* __restrict__ part, int Gp, int
     const double hn = sqrt(sets[0]);
     const double inv = hn > 0.0 ? 1.0 / hn : 0.0;
     hcol[j + 1] = hn;
-    for (int d = 1; d <= ng; ++d) gram[(j + 1) * kGramB + d] = sets[1 + ng - d] * inv;
+    for (int d = 1; d <= ng; ++d) gram[(j + 1) * gb + d] = sets[1 + ng - d] * inv;
     if (gm) givens_step(gm, m, j, hist, hist_cap);
   }
 }
@@ -317,7 +337,7 @@ struct Problem {
   double* dinv = nullptr;     // N, Jacobi inverse diagonal
   float* work32 = nullptr;    // 2 vectors of N (FP32 operator)
   double* partials = nullptr; // 2 x kMaxPartials x 8
-  double* bpart = nullptr;    // 3 x kGramB x kMaxPartials: block-pass partials (two ping-pong buffers, Gram)
+  double* bpart = nullptr;    // 2 x kGramMax x kMaxPartials: block-pass partials (two ping-pong buffers, Gram)
   GmresDev* gm = nullptr;
   BicgDev* bc = nullptr;
   double* hist = nullptr;     // device history
@@ -356,6 +376,7 @@ struct NormIn {
   int Gp, ng;
   double* hcol;         // column jprev of the Hessenberg matrix
   double* gram;
+  int gb;               // entries per Gram row (the block size)
   GmresDev* gm;
   int m, jprev;
   double* hist;

@@ -27,10 +27,11 @@
 #include <memory>
 #include <mutex>
 #include <tuple>
+#include <utility>
 
 #include <cuda.h>
 
-#include "rt_common.cuh"
+#include "rt_pass.cuh"
 
 namespace rt {
 
@@ -421,6 +422,96 @@ __global__ void __launch_bounds__(kMgsThreads, kMgsCtasPerSm) k_bmgs(double* __r
   block_sum4_out(s, nn ? nn : 1 + ng, part_out);
 }
 
+// The same passes with the dots on the integer pipe and the operands streamed
+// through shared memory (rt_pass.cuh), in blocks of B basis vectors: 4 for
+// rt_arnoldi_bmgs (its Gram rows), 8 inside GMRES, where half the passes
+// re-read w half as often (sweep atmosphere with N_s = 500: 162 ms a solve
+// with blocks of 4, 153 ms with 8).  Each CTA owns a contiguous range of
+// tiles.  NB = 0 is the first kernel of a step (the dots with the first
+// block).  Bound: bytes to the SMs -- a middle pass moves 9 or 17 vectors in and
+// w out at 6 TB/s of the 7.6 TB/s that a plain read of L2-resident data
+// reaches here -- and, in a last block with no look-ahead, the FP64 updates
+// (83% of the pipe's cycles).
+template <int B, int NB, int NN>
+__global__ void __launch_bounds__(kPassThreads, 2) k_pass(double* __restrict__ w, const double* __restrict__ V,
+                                                          int64_t N, int i0, const double* __restrict__ part_in,
+                                                          double* __restrict__ part_out, double* __restrict__ hcol,
+                                                          const double* __restrict__ gram, int j, int rev,
+                                                          const int* kstop, int* err) {
+  using S = PassShape<B, NB, NN>;
+  static_assert(kPassWarps >= B && kPassTile >= B * B, "one warp per set of partials");
+  if (kstop && j >= *kstop) return;
+  pdl_launch_dependents();
+  extern __shared__ unsigned char pass_dyn[];
+  __shared__ uint64_t bars[2 * kPassMaxStages];
+  __shared__ int dead;
+  __shared__ double hs[B], gs[B][B];
+  PassRing R;
+  pass_ring_init(R, pass_dyn, bars, &dead, S::NST);
+  const int G = gridDim.x;
+  const int64_t tiles = (N + kPassTile - 1) / kPassTile;
+  const int64_t lo = tiles * blockIdx.x / G * kPassTile;
+  const int64_t hi = min(N, tiles * (blockIdx.x + 1) / G * kPassTile);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp == kPassWarps) {   // producer
+    const PassSrc src = pass_src<B, NB, NN>(w, V + (size_t)i0 * N, V + (size_t)(i0 + NB) * N, N);
+    const int nt = pass_tiles(lo, hi);
+    // the basis vectors do not depend on the previous pass: their first
+    // tiles are copied while it drains
+    const int early = NB > 0 ? min(S::NST, nt) : 0;
+    for (int part = NB > 0 ? 0 : 1; part < 2; ++part) {
+      if (part == 1) {
+        pdl_wait();
+        asm volatile("fence.proxy.async;" ::: "memory");   // the previous kernels' stores, before the copies
+      }
+      for (int q = 0; q < early; ++q) {
+        int64_t e0;
+        int cnt;
+        pass_tile(lo, hi, q, nt, rev, e0, cnt);
+        pass_issue<B, NB, NN>(R, q, src, e0, cnt, part == 0, part == 1);
+      }
+    }
+    pass_produce<B, NB, NN>(R, src, lo, hi, rev, early);
+    return;
+  }
+  if (NB > 0 && threadIdx.x < B * B) {   // the block's Gram entries <v_{i0+k-d}, v_{i0+k}>
+    const int k = threadIdx.x / B, d = threadIdx.x % B;
+    gs[k][d] = k < NB && d >= 1 && d <= k ? gram[(i0 + k) * B + d] : 0.0;
+  }
+  pdl_wait();
+  if (NB > 0) {
+    if (warp < NB) {
+      const double r = partials_sum_warp(part_in + (size_t)warp * G, G);
+      if (lane == 0) hs[warp] = r;
+    }
+    pass_sync();
+    if (warp == 0) {   // h_k = r_k - sum_{l<k} h_l <v_l, v_k>, lane k, l in increasing order
+      const int k = lane < NB ? lane : NB - 1;
+      double r = hs[k];
+#pragma unroll
+      for (int l = 0; l + 1 < NB; ++l) {
+        const double hl = __shfl_sync(0xffffffffu, r, l);
+        if (k > l) r = fma(-hl, gs[k][k - l], r);
+      }
+      __syncwarp();
+      if (lane < NB) {
+        hs[lane] = r;
+        if (blockIdx.x == 0) hcol[i0 + lane] = r;
+      }
+    }
+    pass_sync();
+  }
+  double h[NB > 0 ? NB : 1];
+#pragma unroll
+  for (int k = 0; k < NB; ++k) h[k] = hs[k];
+  FixDot<S::ND, S::NF> D;
+  D.init();
+  pass_consume<B, NB, NN>(R, w, lo, hi, rev, h, D);
+  const double s = pass_block_dots(D.finish(), S::ND);
+  if ((int)threadIdx.x < S::ND) part_out[(size_t)threadIdx.x * G + blockIdx.x] = s;
+  if (threadIdx.x == 0 && dead) atomicExch(err, 1);
+}
+
 // v_{j+1} = w / ||w|| by blocks 1..gridDim.x-1 (||w||^2 is set 0 of the last
 // pass's partials, over Gp blocks).  Block 0, scheduled first, writes
 // h_{j+1} = ||w|| to hcol[j+1] and the Gram row j+1: <v_{j+1}, v_{j+1-d}> =
@@ -432,12 +523,12 @@ constexpr int kScaleU = 4;
 __global__ void __launch_bounds__(kVecThreads, 3) k_bscale(const double* __restrict__ w, double* __restrict__ V,
                                                            int64_t N, const double* __restrict__ part_in, int Gp,
                                                            int ng, double* __restrict__ hcol, double* __restrict__ gram,
-                                                           GmresDev* gm, int m, int j, double* hist, int hist_cap,
-                                                           int rev, const int* kstop) {
+                                                           int gb, GmresDev* gm, int m, int j, double* hist,
+                                                           int hist_cap, int rev, const int* kstop) {
   if (kstop && j >= *kstop) return;
   pdl_wait();
   if (blockIdx.x == 0) {
-    arnoldi_fold(part_in, Gp, ng, hcol, gram, gm, m, j, hist, hist_cap);
+    arnoldi_fold(part_in, Gp, ng, hcol, gram, gb, gm, m, j, hist, hist_cap);
     return;
   }
   double* __restrict__ vo = V + (size_t)(j + 1) * N;
@@ -465,10 +556,10 @@ __global__ void __launch_bounds__(kVecThreads, 3) k_bscale(const double* __restr
 // the end of the last Arnoldi step of a cycle whose normalisations are done
 // by the next step's apply (NormIn): the fold and the Givens rotations only
 __global__ void k_arnoldi_tail(const double* __restrict__ part, int Gp, int ng, double* __restrict__ hcol,
-                               double* __restrict__ gram, GmresDev* gm, int m, int j, double* hist, int hist_cap,
-                               const int* kstop) {
+                               double* __restrict__ gram, int gb, GmresDev* gm, int m, int j, double* hist,
+                               int hist_cap, const int* kstop) {
   if (kstop && j >= *kstop) return;
-  arnoldi_fold(part, Gp, ng, hcol, gram, gm, m, j, hist, hist_cap);
+  arnoldi_fold(part, Gp, ng, hcol, gram, gb, gm, m, j, hist, hist_cap);
 }
 
 // the grid of the block-MGS passes: one CTA per resident slot
@@ -476,6 +567,26 @@ inline int mgs_grid(const Problem* P) {
   int64_t g = (P->Nop + kMgsThreads - 1) / kMgsThreads;
   const int cap = std::min(kMgsCtasPerSm * P->num_sms, kMaxPartials);
   return (int)(g < 1 ? 1 : (g > cap ? cap : g));
+}
+
+// How the block passes run on the basis V and the vector w: k_pass (fixed), or
+// k_bdot / k_bmgs where a bulk copy cannot start on a vector (a caller's V or w
+// that is not 16-byte aligned; vector lengths are even), and the grid, which is
+// also the number of partials per reduction.  k_pass is the faster one at
+// every size measured: a step at j = 29 took 273.8 us with k_bdot / k_bmgs and
+// 213.2 us with k_pass at N = 1,939,200, 87.6 and 68.5 us at N = 195,200, 64.0
+// and 52.8 us at N = 69,440 (blocks of 4).
+struct MgsPlan {
+  bool fixed;
+  int grid;
+};
+constexpr int kPassCtasPerSm = 2;   // resident at once (the ring's size): 1 per SM took 1.25 times as long
+inline MgsPlan mgs_plan(const Problem* P, const double* V, const double* w) {
+  const int64_t N = P->Nop;
+  if ((N & 1) || !P->dev_err || (reinterpret_cast<uintptr_t>(V) & 15) || (reinterpret_cast<uintptr_t>(w) & 15))
+    return {false, mgs_grid(P)};
+  const int64_t tiles = (N + kPassTile - 1) / kPassTile;
+  return {true, (int)std::min<int64_t>(tiles, std::min(kPassCtasPerSm * P->num_sms, kMaxPartials))};
 }
 
 // back substitution H(0:k,0:k) y = g(0:k) in the textbook order: row k-1
@@ -884,14 +995,40 @@ struct Workspace {
   double* part[2];  // ping-pong partial buffers
 };
 
+using PassFn = void (*)(double*, const double*, int64_t, int, const double*, double*, double*, const double*, int, int,
+                        const int*, int*);
+// the passes of blocks of B vectors: first dots with n + 1 vectors, a full
+// block with n + 1 look-ahead dots, a last block of n + 1 vectors
+template <int B>
+struct PassTable {
+  PassFn dot[B], mid[B], last[B];
+  template <int... n>
+  constexpr explicit PassTable(std::integer_sequence<int, n...>)
+      : dot{k_pass<B, 0, n + 1>...}, mid{k_pass<B, B, n + 1>...}, last{k_pass<B, n + 1, 0>...} {}
+  PassTable() : PassTable(std::make_integer_sequence<int, B>()) {}
+};
+static const PassTable<kGramB> g_pass4;      // rt_arnoldi_bmgs (RT_GRAM_BLOCK)
+static const PassTable<kGramMax> g_pass8;    // GMRES
+
+template <int B>
+static cudaError_t pass_smem_attr(const PassTable<B>& T) {
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < B; ++i)
+    for (PassFn f : {T.dot[i], T.mid[i], T.last[i]})
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassDynSmem);
+  return e;
+}
+
 static rt_status ensure_workspace(Problem* P, int restart, cudaStream_t st) {
   {
-    // k_lsq's shared triangle of the longest cycle (103 KB) needs the opt-in;
-    // set here, outside any stream capture
+    // k_lsq's shared triangle of the longest cycle (103 KB) and the rings of
+    // the block passes need the opt-in; set here, outside any stream capture
     static std::once_flag lsq_attr;
     static cudaError_t lsq_err = cudaSuccess;
     std::call_once(lsq_attr, [] {
       lsq_err = cudaFuncSetAttribute(k_lsq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsq_smem(kMaxRestart));
+      if (lsq_err == cudaSuccess) lsq_err = pass_smem_attr(g_pass4);
+      if (lsq_err == cudaSuccess) lsq_err = pass_smem_attr(g_pass8);
     });
     RT_TRY_CUDA(lsq_err);
   }
@@ -904,7 +1041,7 @@ static rt_status ensure_workspace(Problem* P, int restart, cudaStream_t st) {
   if (!P->work) RT_TRY_CUDA(dev_alloc(P, (void**)&P->work, (size_t)kWorkVecs * P->Nop * sizeof(double)));
   if (!P->dinv) RT_TRY_CUDA(dev_alloc(P, (void**)&P->dinv, (size_t)P->Nop * sizeof(double)));
   if (!P->partials) RT_TRY_CUDA(dev_alloc(P, (void**)&P->partials, (size_t)2 * 2 * kMaxPartials * sizeof(double)));
-  if (!P->bpart) RT_TRY_CUDA(dev_alloc(P, (void**)&P->bpart, (size_t)3 * kGramB * kMaxPartials * sizeof(double)));
+  if (!P->bpart) RT_TRY_CUDA(dev_alloc(P, (void**)&P->bpart, (size_t)2 * kGramMax * kMaxPartials * sizeof(double)));
   if (!P->gm) RT_TRY_CUDA(dev_alloc(P, (void**)&P->gm, sizeof(GmresDev)));
   if (!P->bc) RT_TRY_CUDA(dev_alloc(P, (void**)&P->bc, sizeof(BicgDev)));
   if (restart > P->ws_restart) {
@@ -921,8 +1058,8 @@ static rt_status ensure_workspace(Problem* P, int restart, cudaStream_t st) {
 
 static inline double* wk(Problem* P, int i) { return P->work + (size_t)i * P->Nop; }
 static inline double* partb(Problem* P, int i) { return P->partials + (size_t)i * 2 * kMaxPartials; }
-// block-pass partials: buffers 0 and 1 ping-pong, 2 holds the Gram partials
-static inline double* bpartb(Problem* P, int i) { return P->bpart + (size_t)i * kGramB * kMaxPartials; }
+// block-pass partials: two buffers that the passes alternate between
+static inline double* bpartb(Problem* P, int i) { return P->bpart + (size_t)i * kGramMax * kMaxPartials; }
 
 // the dense sigma-form SOR / SSOR preconditioners, and the left ones
 static inline bool prec_dense(int pc) {
@@ -989,31 +1126,63 @@ static rt_status add_precond(Problem* P, double* x, double* t, int precond, doub
 // scale == false: the normalisation and the fold are left to the next apply
 // (NormIn); *pb_out and *ng_out then name the last pass's partial buffer and
 // Gram-set count.
-static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* hcol, double* gram, GmresDev* gm,
-                              int m, double* hist, int hcap, const int* kstop, cudaStream_t st, bool scale = true,
-                              int* pb_out = nullptr, int* ng_out = nullptr) {
-  const int Gm = mgs_grid(P);
+// the passes of one step in blocks of B vectors (k_pass); *pb: the buffer of
+// the last pass's partials, *ng its Gram sets, *rev the last sweep direction
+template <int B>
+static rt_status enqueue_passes(Problem* P, const PassTable<B>& T, const double* V, double* w, int Gm, int j,
+                                double* hcol, const double* gram, const int* kstop, cudaStream_t st, int* pb, int* ng,
+                                int* rev) {
   const int64_t N = P->Nop;
-  using BdotFn = void (*)(const double*, const double*, int64_t, double*, int, int, const int*);
-  using BmgsFn = void (*)(double*, const double*, int64_t, int, const double*, double*, double*, const double*, int,
-                          int, const int*);
-  static const BdotFn bdot[kGramB] = {k_bdot<1>, k_bdot<2>, k_bdot<3>, k_bdot<4>};
-  static const BmgsFn pass[kGramB] = {k_bmgs<4, 1>, k_bmgs<4, 2>, k_bmgs<4, 3>, k_bmgs<4, 4>};
-  static const BmgsFn last[kGramB] = {k_bmgs<1, 0>, k_bmgs<2, 0>, k_bmgs<3, 0>, k_bmgs<4, 0>};
-  static_assert(kGramB == 4, "kernel tables");
-  int pb = 0, rev = 0;
-  RT_TRY_CUDA(launch_pdl(bdot[std::min(kGramB, j + 1) - 1], Gm, kMgsThreads, st, (const double*)w, (const double*)V, N,
-                         bpartb(P, 0), j, rev, kstop)); RT_COUNT(1);
-  int ng = 0;
-  for (int i0 = 0; i0 <= j; i0 += kGramB) {
-    const int nb = std::min(kGramB, j + 1 - i0);
-    const int nn = std::max(0, std::min(kGramB, j + 1 - (i0 + nb)));
-    if (nn == 0) ng = nb < kGramB ? nb : 0;
-    rev ^= 1;
-    RT_TRY_CUDA(launch_pdl(nn ? pass[nn - 1] : last[nb - 1], Gm, kMgsThreads, st, w, (const double*)V, N, i0,
-                           (const double*)bpartb(P, pb), bpartb(P, pb ^ 1), hcol, (const double*)gram, j, rev,
-                           kstop)); RT_COUNT(1);
-    pb ^= 1;
+  RT_TRY_CUDA(launch_pdl_smem(T.dot[std::min(B, j + 1) - 1], Gm, kPassThreads, kPassDynSmem, st, w, V, N, 0,
+                              (const double*)nullptr, bpartb(P, 0), (double*)nullptr, (const double*)nullptr, j, *rev,
+                              kstop, P->dev_err)); RT_COUNT(1);
+  for (int i0 = 0; i0 <= j; i0 += B) {
+    const int nb = std::min(B, j + 1 - i0);
+    const int nn = std::max(0, std::min(B, j + 1 - (i0 + nb)));
+    if (nn == 0) *ng = nb < B ? nb : 0;
+    *rev ^= 1;
+    RT_TRY_CUDA(launch_pdl_smem(nn ? T.mid[nn - 1] : T.last[nb - 1], Gm, kPassThreads, kPassDynSmem, st, w, V, N, i0,
+                                (const double*)bpartb(P, *pb), bpartb(P, *pb ^ 1), hcol, gram, j, *rev, kstop,
+                                P->dev_err)); RT_COUNT(1);
+    *pb ^= 1;
+  }
+  return RT_OK;
+}
+
+static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* hcol, double* gram, int gb,
+                              GmresDev* gm, int m, double* hist, int hcap, const int* kstop, cudaStream_t st, bool scale = true,
+                              int* pb_out = nullptr, int* ng_out = nullptr) {
+  const MgsPlan plan = mgs_plan(P, V, w);
+  const int Gm = plan.grid;
+  const int64_t N = P->Nop;
+  int pb = 0, rev = 0, ng = 0;
+  if (plan.fixed) {
+    if (gb == kGramB) RT_TRY(enqueue_passes(P, g_pass4, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev));
+    else RT_TRY(enqueue_passes(P, g_pass8, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev));
+  } else {
+    using BdotFn = void (*)(const double*, const double*, int64_t, double*, int, int, const int*);
+    using BmgsFn = void (*)(double*, const double*, int64_t, int, const double*, double*, double*, const double*, int,
+                            int, const int*);
+    static const BdotFn bdot[kGramB] = {k_bdot<1>, k_bdot<2>, k_bdot<3>, k_bdot<4>};
+    static const BmgsFn pass[kGramB] = {k_bmgs<4, 1>, k_bmgs<4, 2>, k_bmgs<4, 3>, k_bmgs<4, 4>};
+    static const BmgsFn last[kGramB] = {k_bmgs<1, 0>, k_bmgs<2, 0>, k_bmgs<3, 0>, k_bmgs<4, 0>};
+    static_assert(kGramB == 4, "kernel tables");
+    if (gb != kGramB) {
+      set_error("internal: these block passes take blocks of %d vectors", kGramB);
+      return RT_EINVAL;
+    }
+    RT_TRY_CUDA(launch_pdl(bdot[std::min(kGramB, j + 1) - 1], Gm, kMgsThreads, st, (const double*)w, (const double*)V,
+                           N, bpartb(P, 0), j, rev, kstop)); RT_COUNT(1);
+    for (int i0 = 0; i0 <= j; i0 += kGramB) {
+      const int nb = std::min(kGramB, j + 1 - i0);
+      const int nn = std::max(0, std::min(kGramB, j + 1 - (i0 + nb)));
+      if (nn == 0) ng = nb < kGramB ? nb : 0;
+      rev ^= 1;
+      RT_TRY_CUDA(launch_pdl(nn ? pass[nn - 1] : last[nb - 1], Gm, kMgsThreads, st, w, (const double*)V, N, i0,
+                             (const double*)bpartb(P, pb), bpartb(P, pb ^ 1), hcol, (const double*)gram, j, rev,
+                             kstop)); RT_COUNT(1);
+      pb ^= 1;
+    }
   }
   if (pb_out) *pb_out = pb;
   if (ng_out) *ng_out = ng;
@@ -1022,8 +1191,8 @@ static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* h
     return RT_OK;
   }
   rev ^= 1;
-  RT_TRY_CUDA(launch_pdl(k_bscale, std::min(Gm, 2 * P->num_sms) + 1, kVecThreads, st, (const double*)w, V, N, (const double*)bpartb(P, pb), Gm, ng,
-                         hcol, gram, gm, m, j, hist, hcap, rev, kstop)); RT_COUNT(1);
+  RT_TRY_CUDA(launch_pdl(k_bscale, std::min(mgs_grid(P), 2 * P->num_sms) + 1, kVecThreads, st, (const double*)w, V, N, (const double*)bpartb(P, pb), Gm, ng,
+                         hcol, gram, gb, gm, m, j, hist, hcap, rev, kstop)); RT_COUNT(1);
   RT_TRY_CUDA(cudaGetLastError());
   return RT_OK;
 }
@@ -1111,11 +1280,14 @@ static rt_status enqueue_cycle(Problem* P, int m, int precond, int fp32, cudaStr
   const int amode = precond == RT_PREC_JACOBI ? AM_JACOBI : precond == RT_PREC_LOCAL_LAMBDA ? AM_LOCAL_LAMBDA : AM_PLAIN;
   const bool fuse = P->form == RT_FORM_I && !prec_dense(precond) &&
                     (!fp32 || (!prec_left(precond) && staged_f64io_ok(P, amode, P->V, w)));
+  const MgsPlan plan = mgs_plan(P, P->V, w);
+  const int Gm = plan.grid;                          // partials per reduction of the block passes
+  const int gb = plan.fixed ? kGramMax : kGramB;     // their block size
   int pb = 0, ng = 0;
   for (int j = 0; j < m; ++j) {
     double* vj = P->V + (size_t)j * N;
     if (fuse && j > 0) {
-      const NormIn nin{w, bpartb(P, pb), mgs_grid(P), ng, &gm->H[(j - 1) * (m + 1)], gm->gram, gm, m, j - 1, hist,
+      const NormIn nin{w, bpartb(P, pb), Gm, ng, &gm->H[(j - 1) * (m + 1)], gm->gram, gb, gm, m, j - 1, hist,
                        hcap, kstop};
       RT_TRY(apply_prec(P, vj, w, precond, fp32, st, kstop, j, &nin));
     } else {
@@ -1124,12 +1296,12 @@ static rt_status enqueue_cycle(Problem* P, int m, int precond, int fp32, cudaStr
     // block MGS: dots with the first block, one pass per block of kGramB
     // basis vectors (the last with ||w|| and the Gram dots of v_{j+1}), then
     // (unless fused) the normalisation with the Givens rotations of column j
-    RT_TRY(enqueue_bmgs(P, P->V, w, j, &gm->H[j * (m + 1)], gm->gram, gm, m, hist, hcap, kstop, st, !fuse, &pb,
+    RT_TRY(enqueue_bmgs(P, P->V, w, j, &gm->H[j * (m + 1)], gm->gram, gb, gm, m, hist, hcap, kstop, st, !fuse, &pb,
                         &ng));
   }
   if (fuse) {
-    k_arnoldi_tail<<<1, 32 * kGramB, 0, st>>>(bpartb(P, pb), mgs_grid(P), ng, &gm->H[(m - 1) * (m + 1)], gm->gram,
-                                              gm, m, m - 1, hist, hcap, kstop); RT_COUNT(1);
+    k_arnoldi_tail<<<1, 32 * kGramMax, 0, st>>>(bpartb(P, pb), Gm, ng, &gm->H[(m - 1) * (m + 1)], gm->gram, gb,
+                                                gm, m, m - 1, hist, hcap, kstop); RT_COUNT(1);
   }
   RT_TRY_CUDA(cudaGetLastError());
   k_lsq<<<1, 32, lsq_smem(m), st>>>(gm, m); RT_COUNT(1);
@@ -1470,8 +1642,8 @@ static rt_status solve_gmres(Problem* P, const rt_solver_opts* o, const double* 
     if (hl) RT_TRY_CUDA(cudaMemcpyAsync(o->resid_hist, P->hist, hl * sizeof(double), cudaMemcpyDeviceToHost, st));
   }
   RT_TRY_CUDA(cudaStreamSynchronize(st));
-  if (o->precision == RT_PRECISION_FP32_REFINE) {
-    const rt_status f = check_device_flag(P, st);
+  {
+    const rt_status f = check_device_flag(P, st);   // the bounded waits of the copies into shared memory
     if (f != RT_OK) s = f;
   }
   if (info) {
@@ -1874,7 +2046,7 @@ rt_status rt_arnoldi_bmgs(rt_problem* prob, double* V_dev, int32_t j, double* w_
   int* always = reinterpret_cast<int*>(&P->gm->kstop);   // a gate that never stops the kernels
   const int big = 1 << 30;
   RT_TRY_CUDA(cudaMemcpyAsync(always, &big, sizeof(int), cudaMemcpyHostToDevice, st));
-  return enqueue_bmgs(P, V_dev, w_dev, j, h_dev, gram_dev, nullptr, 0, nullptr, 0, always, st);
+  return enqueue_bmgs(P, V_dev, w_dev, j, h_dev, gram_dev, kGramB, nullptr, 0, nullptr, 0, always, st);
 }
 
 rt_status rt_solve_gmres(rt_problem* prob, const rt_solver_opts* opts, const double* b_dev, double* x_dev,

@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kMom64Threads) k_moments64_norm(
   if (nin.kstop && nin.jprev >= *nin.kstop) return;
   pdl_wait();   // the last block pass's w and partials
   if (blockIdx.x == 0) {
-    arnoldi_fold(nin.part, nin.Gp, nin.ng, nin.hcol, nin.gram, nin.gm, nin.m, nin.jprev, nin.hist, nin.hist_cap);
+    arnoldi_fold(nin.part, nin.Gp, nin.ng, nin.hcol, nin.gram, nin.gb, nin.gm, nin.m, nin.jprev, nin.hist, nin.hist_cap);
     return;
   }
   const double inv = arnoldi_inv_norm(nin.part, nin.Gp);

@@ -53,6 +53,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "rt_async.cuh"
 #include "rt_device.cuh"
 
 namespace rt {
@@ -79,7 +80,6 @@ constexpr int kNST = RT_STAGED_NST;            // stages per warp
 constexpr int kRS = RT_STAGED_RS;              // prefetch distance of the node operands (steps)
 constexpr int kMaxT = RT_STAGED_MAXT;          // warps per CTA (depth tiles of a ray group)
 constexpr int kTabPad = 2 * kRS;               // table entries past the last node (prefetch reads them)
-constexpr unsigned long long kWaitNs = 1000000000ull;   // bound of one wait
 constexpr int kQuadThreads = 256;
 constexpr int kQuadMaxHeights = 64;            // heights per CTA of k_quad
 constexpr int kQuadBatch = 2;                  // heights per batch of loads (two batches in flight)
@@ -105,46 +105,6 @@ constexpr size_t smem_bytes(int warp_bytes, int ntile) { return 128 + (size_t)nt
 static_assert(smem_bytes(Cfg<double, KM_JACOBI>::WARP, kMaxT) <= 227 * 1024, "a CTA fits the shared memory");
 
 // ------------------------------------------------------------ PTX helpers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ unsigned long long gtimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n"
-      " .reg .pred p;\n"
-      " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// wait for the phase of `parity` to complete; false after kWaitNs
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = gtimer();
-  while (!mbar_try_wait(bar, parity))
-    if (gtimer() - t0 > kWaitNs) return false;
-  return true;
-}
-
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2,
                                             uint64_t* bar) {
   asm volatile(
@@ -449,7 +409,7 @@ __global__ void __launch_bounds__(kQuadThreads) k_quad_norm(double* __restrict__
   pdl_launch_dependents();
   if (blockIdx.y == 0) {
     if (blockIdx.x == 0)
-      arnoldi_fold(nin.part, nin.Gp, nin.ng, nin.hcol, nin.gram, nin.gm, nin.m, nin.jprev, nin.hist, nin.hist_cap);
+      arnoldi_fold(nin.part, nin.Gp, nin.ng, nin.hcol, nin.gram, nin.gb, nin.gm, nin.m, nin.jprev, nin.hist, nin.hist_cap);
     return;
   }
   const double inv = arnoldi_inv_norm(nin.part, nin.Gp);

@@ -1,0 +1,122 @@
+"""The streamed block passes of the Arnoldi step (dots in fixed point on the
+integer pipe) against the MGS loop in numpy.
+
+Vector lengths around the passes' tile (256 elements) and grid edges, every
+last-block size, values that force new fixed-point scales (magnitudes growing
+along the vector, isolated large entries, zeros), operands that no bulk copy
+can start on (8-byte aligned: the register kernels), infinities and NaN, and
+the 8-vector blocks of GMRES over a long cycle.
+
+Tolerance of the coefficients: MGS in FP64 gives each h_i to within a few
+rounding errors of |w| |v_i| = |w|; both sides accumulate at most N of them in
+trees or chains of length < 1000, so 1e-12 |w| holds with margin, and w and
+v_{j+1} likewise to 1e-11 (division by the norm of what is left of w)."""
+import numpy as np
+import pytest
+import torch
+
+import rt_workloads as W
+from gpu_util import problem, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def _mgs(Q, w):
+    h = []
+    for v in Q:
+        h.append(np.dot(w, v))
+        w = w - h[-1] * v
+    h.append(np.linalg.norm(w))
+    return np.array(h), w
+
+
+def _values(kind, N, rng):
+    w = rng.standard_normal(N)
+    if kind == "growing":
+        w *= np.exp(np.linspace(-30.0, 10.0, N))
+    elif kind == "spikes":
+        w[rng.integers(0, N, 5)] *= 1e9
+    elif kind == "zeros":
+        w[: N // 2] = 0.0
+        w[N // 2:: 3] = 0.0
+    elif kind == "tiny":
+        w *= 1e-290
+    return w
+
+
+def _step(P, N, j, kind, offset=0, seed=0):
+    rng = np.random.default_rng(seed)
+    Q = []
+    for i in range(j + 1):
+        v = _values("growing" if kind == "growing" and i % 2 else "normal", N, rng)
+        for _ in range(2):
+            for u in Q:
+                v = v - np.dot(u, v) * u
+        Q.append(v / np.linalg.norm(v))
+    w0 = _values(kind, N, rng)
+    gram = np.zeros((j + 2, 4))
+    for i in range(1, j + 1):
+        for d in range(1, min(i, 3) + 1):
+            gram[i, d] = Q[i] @ Q[i - d]
+    buf = torch.zeros((j + 2) * N + 2, dtype=torch.float64, device="cuda")
+    Vd = buf[offset: offset + (j + 2) * N]
+    Vd[: (j + 1) * N] = to_dev(np.concatenate(Q))
+    wbuf = torch.zeros(N + 2, dtype=torch.float64, device="cuda")
+    wd = wbuf[offset: offset + N]
+    wd.copy_(to_dev(w0))
+    h = to_host(P.arnoldi_bmgs(Vd, j, wd, to_dev(gram.reshape(-1))))
+    P.check()
+    href, w = _mgs(Q, w0)
+    s = np.abs(w0).max() * np.linalg.norm(w0 / np.abs(w0).max())   # |w0| without underflow of its square
+    np.testing.assert_allclose(h, href, rtol=0, atol=1e-12 * s)
+    np.testing.assert_allclose(to_host(wd), w, rtol=0, atol=1e-11 * s)
+    if href[-1] > 0.0:   # (the square of the norm underflows for the tiny values, on both sides)
+        np.testing.assert_allclose(to_host(Vd)[(j + 1) * N:], w / href[-1], rtol=0, atol=1e-11 * s / href[-1])
+
+
+# N = 2 Ns Nmu Nnu: below, at and just past one tile; several tiles; more tiles than CTAs
+@pytest.mark.parametrize("Ns,Nmu,Nnu", [(2, 2, 2), (21, 2, 3), (32, 2, 2), (43, 2, 3), (37, 6, 33), (100, 16, 61)])
+@pytest.mark.parametrize("j", [0, 3, 4, 6, 13])
+def test_pass_sizes(Ns, Nmu, Nnu, j):
+    P = problem(W.slab(Ns, Nmu, Nnu, 1e-4, 1e6, 6.0))
+    if j + 2 > P.N:
+        j = P.N - 3
+    _step(P, P.N, j, "normal", seed=j)
+
+
+@pytest.mark.parametrize("kind", ["growing", "spikes", "zeros", "tiny"])
+@pytest.mark.parametrize("offset", [0, 1])   # 1: 8-byte aligned operands
+def test_pass_values(kind, offset):
+    P = problem(W.slab(100, 8, 41, 1e-4, 1e6, 6.0))
+    _step(P, P.N, 9, kind, offset, seed=3)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_pass_not_finite(bad):
+    """A non-finite w gives non-finite coefficients, as the FP64 products do."""
+    P = problem(W.slab(37, 6, 33, 1e-4, 1e6, 6.0))
+    N, j = P.N, 5
+    rng = np.random.default_rng(0)
+    V = torch.zeros((j + 2) * N, dtype=torch.float64, device="cuda")
+    V[: (j + 1) * N] = to_dev(rng.standard_normal((j + 1) * N) / np.sqrt(N))
+    w0 = rng.standard_normal(N)
+    w0[N // 3] = bad
+    v0 = to_host(V)[N // 3]
+    h = to_host(P.arnoldi_bmgs(V, j, to_dev(w0), torch.zeros((j + 2) * 4, dtype=torch.float64, device="cuda")))
+    assert (np.isnan(h[0]) if np.isnan(bad) else h[0] == bad * np.sign(v0)), h
+    assert not np.isfinite(h).any()
+
+
+@pytest.mark.parametrize("form", ["I", "sigma"])
+def test_gmres_blocks_of_eight(form):
+    """One long GMRES cycle (every block of 8 and each last-block size before
+    it) gives the least-squares residual of the Krylov space: the estimate it
+    stops on and the true residual agree."""
+    at = W.paper(60, 8, 11, freq_norm=0)
+    P = problem(at) if form == "I" else __import__("paper_2110_11873_gb300").Problem(at, form="sigma")
+    b = P.rhs()
+    for m in (1, 7, 8, 9, 16, 23, 40):
+        x, info = P.solve(b, "gmres", restart=m, maxit=m, precond="none", rtol=1e-13)
+        r = b - P.apply(x)
+        rel = float(torch.linalg.vector_norm(r) / torch.linalg.vector_norm(b))
+        assert abs(rel - info.err_est) <= 1e-11 + 1e-8 * info.err_est, (m, rel, info)
