@@ -569,6 +569,8 @@ inline int mgs_grid(const Problem* P) {
   return (int)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
+inline int cdiv(int a, int b) { return (a + b - 1) / b; }
+
 // How the block passes run on the basis V and the vector w: k_pass (fixed), or
 // k_bdot / k_bmgs where a bulk copy cannot start on a vector (a caller's V or w
 // that is not 16-byte aligned; vector lengths are even), and the grid, which is
@@ -1198,10 +1200,20 @@ static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* h
 }
 
 // --------------------------------------------------------------- GMRES
+// A restart cycle is launched as graphs of kSegSteps Arnoldi steps and a last
+// one with the end of the cycle.  One graph of the whole cycle (as the cycle
+// was launched before) ran its kernels past convergence as gated launches,
+// about 1.3 us each: an unrestarted sigma-form run of 41 steps spent two thirds
+// of its time in them, and the launch queued ahead of the host's check cost a
+// cycle of 30 steps 5%.
+constexpr int kSegSteps = 8;
+inline int cycle_segments(int m) { return (m + kSegSteps - 1) / kSegSteps; }
+
+// seg: steps seg * kSegSteps .. of the cycle, or cycle_segments(m) for its end
 struct GmresGraphKey {
-  int m, precond, fp32;
+  int m, precond, fp32, seg;
   bool operator<(const GmresGraphKey& o) const {
-    return std::tie(m, precond, fp32) < std::tie(o.m, o.precond, o.fp32);
+    return std::tie(m, precond, fp32, seg) < std::tie(o.m, o.precond, o.fp32, o.seg);
   }
 };
 
@@ -1261,10 +1273,11 @@ void release_graphs(Problem* P) {
   }
 }
 
-// Enqueue one restart cycle: steps 0..m-1, least squares, x update, true
-// residual and the start of the next cycle.  Vectors: x = wk(0), b = wk(1),
-// r = wk(2), w = wk(3), t = wk(4), Ax = wk(5), tmp = wk(6).
-static rt_status enqueue_cycle(Problem* P, int m, int precond, int fp32, cudaStream_t st) {
+// Enqueue segment seg of a restart cycle: Arnoldi steps of 0..m-1 or, for seg
+// = cycle_segments(m), the least squares, x update, true residual and the
+// start of the next cycle.  Vectors: x = wk(0), b = wk(1), r = wk(2), w =
+// wk(3), t = wk(4), Ax = wk(5), tmp = wk(6).
+static rt_status enqueue_cycle(Problem* P, int m, int precond, int fp32, int seg, cudaStream_t st) {
   const int G = P->vec_grid;
   const int64_t N = P->Nop;
   GmresDev* gm = P->gm;
@@ -1283,8 +1296,15 @@ static rt_status enqueue_cycle(Problem* P, int m, int precond, int fp32, cudaStr
   const MgsPlan plan = mgs_plan(P, P->V, w);
   const int Gm = plan.grid;                          // partials per reduction of the block passes
   const int gb = plan.fixed ? kGramMax : kGramB;     // their block size
+  const bool end = seg == cycle_segments(m);
+  const int j0 = end ? m : seg * kSegSteps, j1 = end ? m : std::min(m, j0 + kSegSteps);
+  // where the step before the segment left its last partials (enqueue_bmgs)
   int pb = 0, ng = 0;
-  for (int j = 0; j < m; ++j) {
+  if (j0 > 0) {
+    pb = cdiv(j0, gb) & 1;
+    ng = j0 % gb;
+  }
+  for (int j = j0; j < j1; ++j) {
     double* vj = P->V + (size_t)j * N;
     if (fuse && j > 0) {
       const NormIn nin{w, bpartb(P, pb), Gm, ng, &gm->H[(j - 1) * (m + 1)], gm->gram, gb, gm, m, j - 1, hist,
@@ -1298,6 +1318,10 @@ static rt_status enqueue_cycle(Problem* P, int m, int precond, int fp32, cudaStr
     // (unless fused) the normalisation with the Givens rotations of column j
     RT_TRY(enqueue_bmgs(P, P->V, w, j, &gm->H[j * (m + 1)], gm->gram, gb, gm, m, hist, hcap, kstop, st, !fuse, &pb,
                         &ng));
+  }
+  if (!end) {
+    RT_TRY_CUDA(cudaGetLastError());
+    return RT_OK;
   }
   if (fuse) {
     k_arnoldi_tail<<<1, 32 * kGramMax, 0, st>>>(bpartb(P, pb), Gm, ng, &gm->H[(m - 1) * (m + 1)], gm->gram, gb,
@@ -1372,6 +1396,39 @@ static rt_status launch_graph(GraphCache* gc, cudaGraphExec_t ex, cudaStream_t s
   return RT_OK;
 }
 
+// Two pinned host copies of a solver's state header, written behind graph
+// launches: the host reads one launch's copy while the next launch runs.
+template <typename Hdr>
+struct HeaderQueue {
+  GraphCache* gc;
+  const Hdr* dev;
+  size_t bytes;
+  cudaStream_t st;
+  rt_status init() {
+    if (bytes > kHdrBytes) {
+      set_error("internal: solver header larger than its host copy");
+      return RT_EINVAL;
+    }
+    if (!gc->hdr) {
+      RT_TRY_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&gc->hdr), 2 * kHdrBytes, cudaHostAllocDefault));
+      for (cudaEvent_t& e : gc->hev) RT_TRY_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
+    return RT_OK;
+  }
+  // launch ex, then copy the header into the slot
+  rt_status launch(cudaGraphExec_t ex, int slot) {
+    RT_TRY(launch_graph(gc, ex, st));
+    RT_TRY_CUDA(cudaMemcpyAsync(gc->hdr + slot * kHdrBytes, dev, bytes, cudaMemcpyDeviceToHost, st));
+    RT_TRY_CUDA(cudaEventRecord(gc->hev[slot], st));
+    return RT_OK;
+  }
+  rt_status read(int slot, Hdr* out) {
+    RT_TRY_CUDA(cudaEventSynchronize(gc->hev[slot]));
+    memcpy(static_cast<void*>(out), gc->hdr + slot * kHdrBytes, bytes);
+    return RT_OK;
+  }
+};
+
 // Launches `ex` until `stop(header)` holds, one launch ahead of the host:
 // launch k+1 and the copy of its state header are queued before the host
 // waits for launch k's copy, so the device does not idle while the host
@@ -1384,30 +1441,17 @@ static rt_status launch_graph(GraphCache* gc, cudaGraphExec_t ex, cudaStream_t s
 template <typename Hdr, typename Stop>
 static rt_status launch_until(GraphCache* gc, cudaGraphExec_t ex, const Hdr* dev, Hdr* out, size_t bytes,
                               cudaStream_t st, int* launches, Stop&& stop) {
-  if (bytes > kHdrBytes) {
-    set_error("internal: solver header larger than its host copy");
-    return RT_EINVAL;
-  }
-  if (!gc->hdr) {
-    RT_TRY_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&gc->hdr), 2 * kHdrBytes, cudaHostAllocDefault));
-    for (cudaEvent_t& e : gc->hev) RT_TRY_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  }
-  auto enqueue = [&](int slot) -> rt_status {
-    RT_TRY(launch_graph(gc, ex, st));
-    RT_TRY_CUDA(cudaMemcpyAsync(gc->hdr + slot * kHdrBytes, dev, bytes, cudaMemcpyDeviceToHost, st));
-    RT_TRY_CUDA(cudaEventRecord(gc->hev[slot], st));
-    return RT_OK;
-  };
+  HeaderQueue<Hdr> Q{gc, dev, bytes, st};
+  RT_TRY(Q.init());
   *launches = 0;
-  RT_TRY(enqueue(0));
+  RT_TRY(Q.launch(ex, 0));
   for (int k = 0;; ++k) {
-    const rt_status s = enqueue((k + 1) & 1);   // one ahead
+    const rt_status s = Q.launch(ex, (k + 1) & 1);   // one ahead
     if (s != RT_OK) {
       cudaStreamSynchronize(st);
       return s;
     }
-    RT_TRY_CUDA(cudaEventSynchronize(gc->hev[k & 1]));
-    memcpy(static_cast<void*>(out), gc->hdr + (k & 1) * kHdrBytes, bytes);
+    RT_TRY(Q.read(k & 1, out));
     *launches += 1;
     if (stop(*out)) break;
   }
@@ -1415,15 +1459,15 @@ static rt_status launch_until(GraphCache* gc, cudaGraphExec_t ex, const Hdr* dev
   return RT_OK;
 }
 
-static rt_status get_graph(Problem* P, GraphCache* gc, int m, int precond, int fp32, cudaGraphExec_t* out) {
-  GmresGraphKey key{m, precond, fp32};
+static rt_status get_graph(Problem* P, GraphCache* gc, int m, int precond, int fp32, int seg, cudaGraphExec_t* out) {
+  GmresGraphKey key{m, precond, fp32, seg};
   auto it = gc->gmres.find(key);
   if (it != gc->gmres.end()) {
     *out = it->second;
     return RT_OK;
   }
   cudaGraphExec_t ex = nullptr;
-  RT_TRY(capture_graph(gc, [&](cudaStream_t cs) { return enqueue_cycle(P, m, precond, fp32, cs); }, &ex));
+  RT_TRY(capture_graph(gc, [&](cudaStream_t cs) { return enqueue_cycle(P, m, precond, fp32, seg, cs); }, &ex));
   gc->gmres[key] = ex;
   *out = ex;
   return RT_OK;
@@ -1478,17 +1522,47 @@ static rt_status gmres_core(Problem* P, const rt_solver_opts* o, int fp32, doubl
   *cycles = 0;
   if (hs->bnorm == 0.0 || !(hs->rel >= tol) || hs->rel != hs->rel) return RT_OK;
   GraphCache* gc = cache_of(P);
-  cudaGraphExec_t ex;
-  RT_TRY(get_graph(P, gc, m, o->precond, fp32, &ex));
   // A cycle that runs after one of these stops changes nothing: k_cycle_start
   // of the stopping cycle set kstop = 0 (converged, NaN, no steps left), so
   // every step is gated off and the update and residual repeat exactly; or
   // the first step broke down, which the next cycle repeats with the same
   // result (no step done, x unchanged).
   RT_NVTX("GMRES restart cycles (graphs)");
-  RT_TRY(launch_until(gc, ex, P->gm, hs, kGmresHeader, st, cycles, [&](const GmresDev& h) {
-    return h.rel != h.rel || !(h.rel >= tol) || h.iters >= maxit || (h.breakdown && h.kdone == 0) || h.kstop == 0;
-  }));
+  // The cycle's segments, one launch ahead of the host: segment `cur` is
+  // waited for while `next` is queued behind it.  Once the steps left are all
+  // gated off (kstop below the end of `cur`: the last step done is folded by
+  // the first kernel after it, so a stop at that end still needs the next
+  // segment), the end of the cycle comes next.
+  const int nseg = cycle_segments(m);
+  HeaderQueue<GmresDev> Q{gc, P->gm, kGmresHeader, st};
+  RT_TRY(Q.init());
+  auto launch = [&](int seg, int slot) -> rt_status {
+    cudaGraphExec_t ex;
+    RT_TRY(get_graph(P, gc, m, o->precond, fp32, seg, &ex));
+    return Q.launch(ex, slot);
+  };
+  int cur = 0, next = 1, slot = 0;
+  rt_status s = launch(cur, slot);
+  while (s == RT_OK) {
+    s = launch(next, slot ^ 1);
+    if (s == RT_OK) s = Q.read(slot, hs);
+    if (s != RT_OK) break;
+    int after = next == nseg ? 0 : next + 1;
+    if (cur == nseg) {
+      *cycles += 1;
+      const GmresDev& h = *hs;
+      if (h.rel != h.rel || !(h.rel >= tol) || h.iters >= maxit || (h.breakdown && h.kdone == 0) || h.kstop == 0)
+        break;
+    } else if (next != nseg && hs->kstop < std::min(m, (cur + 1) * kSegSteps)) {
+      after = nseg;
+    }
+    cur = next;
+    next = after;
+    slot ^= 1;
+  }
+  const cudaError_t e = cudaStreamSynchronize(st);   // the launch queued ahead (no effect)
+  RT_TRY(s);
+  RT_TRY_CUDA(e);
   return RT_OK;
 }
 
