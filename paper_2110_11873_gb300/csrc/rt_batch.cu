@@ -38,8 +38,10 @@
 #include <memory>
 #include <mutex>
 #include <thread>
+#include <utility>
 
 #include "rt_device.cuh"
+#include "rt_pass.cuh"
 
 namespace rt {
 
@@ -48,6 +50,7 @@ namespace {
 constexpr int kBT = 512;          // threads of the batched vector kernels
 constexpr int kFormalWarps = 4;   // warps per CTA of the batched formal solver
 constexpr int kInstThreads = 128; // threads of the per-instance scalar kernels
+constexpr int kBatchB = kGramMax; // basis vectors per block pass
 enum VecId { VX = 100, VB, VR, VW, VT, VTMP };
 
 struct InstDev {
@@ -62,12 +65,13 @@ struct InstDev {
   float* S32;
   double *V, *x, *b, *r, *w, *t, *tmp, *dinv, *part;
   GmresDev* gm;
+  int* err;          // set when a bounded wait of a block pass gave up
 };
 
 struct InstStatus {
   double rel;
   double est;   // |g_{j+1}| / ||b|| of the instance's last Arnoldi step (rel before any)
-  int iters, kstop, kdone, breakdown;
+  int iters, kstop, kdone, breakdown, err;
 };
 
 struct Counts {
@@ -104,11 +108,10 @@ __device__ __forceinline__ double bsum(double v) {
   return s;
 }
 
-// an instance's partials: three buffers of kGramB sets of nchunks values
-// (buffers 0 and 1 ping-pong between Arnoldi passes, buffer 2 holds the
-// Gram dots of the newest basis vector)
+// an instance's partials: two buffers of kBatchB sets of nchunks values that
+// the Arnoldi passes alternate between
 __device__ __forceinline__ double* pset(const InstDev& I, int buf, int k) {
-  return I.part + ((size_t)buf * kGramB + k) * I.nchunks;
+  return I.part + ((size_t)buf * kBatchB + k) * I.nchunks;
 }
 
 // sqrt of the sum of an instance's chunk partials (set 0 of buffer pb, in a
@@ -117,9 +120,7 @@ __device__ __forceinline__ double* pset(const InstDev& I, int buf, int k) {
 __device__ __forceinline__ double inst_norm_inv(const InstDev& I, int pb, double* hn_out) {
   __shared__ double nb[2];
   if (threadIdx.x < 32) {
-    double s = 0.0;
-    for (int c = threadIdx.x; c < I.nchunks; c += 32) s += pset(I, pb, 0)[c];
-    s = warp_sum(s);
+    const double s = partials_sum_warp(pset(I, pb, 0), I.nchunks);
     if (threadIdx.x == 0) {
       const double h = sqrt(s);
       nb[0] = h;
@@ -240,168 +241,115 @@ __global__ void __launch_bounds__(32 * kFormalWarps) kb_formal(const InstDev* __
   }
 
 // Block MGS (the single-instance GMRES's Arnoldi step, per instance): passes
-// of kGramB basis vectors, the MGS coefficients of a block from the dots r_k
+// of kBatchB basis vectors, the MGS coefficients of a block from the dots r_k
 // taken before it and the Gram entries, h_k = r_k - sum_{l<k} h_l <v_l, v_k>.
-
-// warps k < n each sum set k of buffer buf into out[k] (fixed order)
-__device__ __forceinline__ void inst_sets(const InstDev& I, int buf, int n, double* out) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp < n) {
-    const double* p = pset(I, buf, warp);
-    double s = 0.0;
-    for (int c = lane; c < I.nchunks; c += 32) s += p[c];
-    s = warp_sum(s);
-    if (lane == 0) out[warp] = s;
-  }
-  __syncthreads();
-}
-
-// block sums of s[0..kGramB-1] (fixed order) for one chunk: sum k < n goes
-// to set k of the instance's buffer buf, entry chunk
-__device__ __forceinline__ void chunk_sum4(const double* s, int n, const InstDev& I, int buf, int chunk) {
-  constexpr int NW = kBT / 32;
-  static_assert(kGramB == 4 && kGramB * NW <= 64 && (NW & (NW - 1)) == 0, "reduction layout");
-  __shared__ double red[kGramB][NW];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const double t = warp_sum4(s);
-  if ((lane & 7) == 0) red[lane >> 3][warp] = t;
-  __syncthreads();
-  if (threadIdx.x < kGramB * NW) {
-    const int k = threadIdx.x / NW, src = threadIdx.x % NW;
-    double x = red[k][src];
-#pragma unroll
-    for (int o = NW / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (src == 0 && k < n) pset(I, buf, k)[chunk] = x;
-  }
-  __syncthreads();
-}
-
-// The block sizes are template parameters: a DFMA under a false predicate
-// still takes its FP64-pipe slot.
-
-// first kernel of Arnoldi step j: partial dots <w, v_k>, k < NK, into buffer 0
-template <int NK>
-__global__ void __launch_bounds__(kBT) kb_bdot(const InstDev* __restrict__ insts, const int2* __restrict__ wl,
-                                               const Counts* cnt, int j) {
-  constexpr int nk = NK;
-  for (int w = blockIdx.x; w < cnt->nc; w += gridDim.x) {
-    const int2 it = wl[w];
-    const InstDev& I = insts[it.x];
-    if (step_gated(I, j)) continue;
-    double s[kGramB] = {0.0, 0.0, 0.0, 0.0};
-    CHUNK_LOOP(const double wi = I.w[n_]; double vv[kGramB]; _Pragma("unroll")
-               for (int k = 0; k < kGramB; ++k) if (k < nk) vv[k] = I.V[(int64_t)k * I.N + n_]; _Pragma("unroll")
-               for (int k = 0; k < kGramB; ++k) if (k < nk) s[k] = fma(wi, vv[k], s[k]);)
-    chunk_sum4(s, nk, I, 0, it.y);
-  }
-}
-
-// one block pass over v_{i0} .. v_{i0+NB-1} into buffer pb ^ 1: the dots with
-// the next NN vectors, or, for the last block (NN == 0), ||w||^2 (set 0) and
-// the Gram dots <w, v_{i0+k}>, k < ng (set 1+k; ng = NB when v_{j+1} shares
-// the block, else 0)
+// One block pass of Arnoldi step j over v_{i0} .. v_{i0+NB-1} of every
+// instance, chunk by chunk (rt_pass.cuh), partials into buffer pb ^ 1: the
+// dots with the next NN vectors, or, for the last block (NN == 0), ||w||^2
+// (set 0) and the Gram dots <w, v_{i0+k}> (set 1+k) while v_{j+1} shares the
+// block.  NB == 0: the step's first dots <w, v_k>, k < NN, into buffer 0.
+// A CTA takes consecutive chunks, so it forms the coefficients once per
+// instance it meets, and its producer warp runs ahead across chunks.
 template <int NB, int NN>
-__global__ void __launch_bounds__(kBT) kb_bmgs(const InstDev* __restrict__ insts, const int2* __restrict__ wl,
-                                               const Counts* cnt, int j, int i0, int pb) {
-  static_assert(NB >= 1 && NB <= kGramB && NN >= 0 && NN <= kGramB && (NN == 0 || NB == kGramB), "block shape");
-  constexpr int nb = NB, nn = NN, ng = NN == 0 && NB < kGramB ? NB : 0;
-  __shared__ double rs[kGramB], hs[kGramB];
-  for (int w = blockIdx.x; w < cnt->nc; w += gridDim.x) {
-    const int2 it = wl[w];
-    const InstDev& I = insts[it.x];
-    if (step_gated(I, j)) continue;
-    inst_sets(I, pb, nb, rs);
-    if (threadIdx.x == 0) {
-      for (int k = 0; k < nb; ++k) {
-        double h = rs[k];
-        for (int l = 0; l < k; ++l) h -= hs[l] * I.gm->gram[(i0 + k) * kGramB + (k - l)];
-        hs[k] = h;
-        if (it.y == 0) I.gm->H[j * (I.m + 1) + i0 + k] = h;
-      }
+__global__ void __launch_bounds__(kPassThreads, 2) kb_pass(const InstDev* __restrict__ insts,
+                                                           const int2* __restrict__ wl, const Counts* cnt, int j,
+                                                           int i0, int pb) {
+  constexpr int B = kBatchB;
+  using S = PassShape<B, NB, NN>;
+  static_assert(kPassWarps >= B && kPassTile >= B * B, "one warp per set of partials");
+  extern __shared__ unsigned char pass_dyn[];
+  __shared__ uint64_t bars[2 * kPassMaxStages];
+  __shared__ int dead;
+  __shared__ double hs[B], gs[B][B];
+  PassRing R;
+  pass_ring_init(R, pass_dyn, bars, &dead, S::NST);
+  const int64_t n = cnt->nc;
+  const int w0 = (int)(n * blockIdx.x / gridDim.x), w1 = (int)(n * (blockIdx.x + 1) / gridDim.x);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp == kPassWarps) {   // producer
+    asm volatile("fence.proxy.async;" ::: "memory");   // the previous kernels' stores, before the copies
+    for (int q = w0; q < w1; ++q) {
+      const int2 it = wl[q];
+      const InstDev& I = insts[it.x];
+      if (step_gated(I, j)) continue;
+      const PassSrc src = pass_src<B, NB, NN>(I.w, I.V + (int64_t)i0 * I.N, I.V + (int64_t)(i0 + NB) * I.N, I.N);
+      const int64_t lo = (int64_t)it.y * I.chunk;
+      pass_produce<B, NB, NN>(R, src, lo, min(I.N, lo + I.chunk), 0, 0);
     }
-    __syncthreads();
-    double h[kGramB];
-#pragma unroll
-    for (int k = 0; k < kGramB; ++k) h[k] = k < nb ? hs[k] : 0.0;
-    __syncthreads();
-    const double* vb = I.V + (int64_t)i0 * I.N;
-    const double* vn = I.V + (int64_t)(i0 + nb) * I.N;
-    double s[kGramB] = {0.0, 0.0, 0.0, 0.0};
-    CHUNK_LOOP(double wi = I.w[n_]; double bv[kGramB]; _Pragma("unroll")
-               for (int k = 0; k < kGramB; ++k) if (k < nb) bv[k] = vb[(int64_t)k * I.N + n_]; _Pragma("unroll")
-               for (int k = 0; k < kGramB; ++k) if (k < nb) wi = fma(-h[k], bv[k], wi);
-               I.w[n_] = wi;
-               if constexpr (nn > 0) { _Pragma("unroll")
-                 for (int k = 0; k < kGramB; ++k) if (k < nn) s[k] = fma(wi, vn[(int64_t)k * I.N + n_], s[k]);
-               } else {
-                 s[0] = fma(wi, wi, s[0]); _Pragma("unroll")
-                 for (int k = 0; k < kGramB - 1; ++k) if (k < ng) s[1 + k] = fma(wi, bv[k], s[1 + k]);
-               })
-    chunk_sum4(s, nn ? nn : 1 + ng, I, pb ^ 1, it.y);
-  }
-}
-
-// per instance: h_{j+1,j} = ||w|| and the Gram row j+1 of v_{j+1} from the
-// last pass's partials (buffer pb, ng Gram sets), then the Givens rotations
-// of column j and the residual estimate
-__global__ void kb_givens(const InstDev* __restrict__ insts, const int* __restrict__ wi, const Counts* cnt, int j,
-                          int pb, int ng) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= cnt->ni) return;
-  const InstDev& I = insts[wi[q]];
-  GmresDev* gm = I.gm;
-  if (j >= gm->kstop) return;
-  const int m = I.m;
-  double* Hc = gm->H + j * (m + 1);
-  double sets[kGramB] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-  for (int k = 0; k < kGramB; ++k) {
-    if (k <= ng) {
-      const double* p = pset(I, pb, k);
-      double t = 0.0;
-      for (int c = 0; c < I.nchunks; ++c) t += p[c];
-      sets[k] = t;
-    }
-  }
-  const double hj = sqrt(sets[0]);
-  const double inv = hj > 0.0 ? 1.0 / hj : 0.0;
-  Hc[j + 1] = hj;
-  gm->vscale = inv;
-#pragma unroll
-  for (int k = 0; k < kGramB - 1; ++k)   // set 1+k: <w, v_{j+1-d}> with d = ng - k
-    if (k < ng) gm->gram[(j + 1) * kGramB + (ng - k)] = sets[1 + k] * inv;
-  for (int i = 0; i < j; ++i) {
-    const double t = gm->cs[i] * Hc[i] + gm->sn[i] * Hc[i + 1];
-    Hc[i + 1] = -gm->sn[i] * Hc[i] + gm->cs[i] * Hc[i + 1];
-    Hc[i] = t;
-  }
-  const double a = Hc[j], b = Hc[j + 1];
-  const double hn = hypot(a, b);
-  if (hn == 0.0) {
-    gm->breakdown = 1;
-    gm->kstop = j;
     return;
   }
-  const double c = a / hn, s = b / hn;
-  gm->cs[j] = c;
-  gm->sn[j] = s;
-  Hc[j] = hn;
-  Hc[j + 1] = 0.0;
-  gm->g[j + 1] = -s * gm->g[j];
-  gm->g[j] = c * gm->g[j];
-  gm->iters += 1;
-  gm->kdone = j + 1;
-  const double est = fabs(gm->g[j + 1]) / gm->bnorm;
-  gm->est = est;
-  if (!(est >= gm->tol) || gm->iters >= gm->maxit || b == 0.0) gm->kstop = j + 1;
+  int have = -1;
+  for (int q = w0; q < w1; ++q) {
+    const int2 it = wl[q];
+    const InstDev& I = insts[it.x];
+    if (step_gated(I, j)) continue;
+    if (NB > 0 && (it.x != have || it.y == 0)) {
+      have = it.x;
+      pass_sync();   // the last instance's coefficients are in registers
+      if (threadIdx.x < B * B) {
+        const int k = threadIdx.x / B, d = threadIdx.x % B;
+        gs[k][d] = k < NB && d >= 1 && d <= k ? I.gm->gram[(i0 + k) * B + d] : 0.0;
+      }
+      if (warp < NB) {
+        const double r = partials_sum_warp(pset(I, pb, warp), I.nchunks);
+        if (lane == 0) hs[warp] = r;
+      }
+      pass_sync();
+      if (warp == 0) {   // lane k, l in increasing order
+        const int k = lane < NB ? lane : NB - 1;
+        double r = hs[k];
+#pragma unroll
+        for (int l = 0; l + 1 < NB; ++l) {
+          const double hl = __shfl_sync(0xffffffffu, r, l);
+          if (k > l) r = fma(-hl, gs[k][k - l], r);
+        }
+        __syncwarp();
+        if (lane < NB) {
+          hs[lane] = r;
+          if (it.y == 0) I.gm->H[j * (I.m + 1) + i0 + lane] = r;
+        }
+      }
+      pass_sync();
+    }
+    double h[NB > 0 ? NB : 1];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) h[k] = hs[k];
+    const int64_t lo = (int64_t)it.y * I.chunk;
+    FixDot<S::ND, S::NF> D;
+    D.init();
+    pass_consume<B, NB, NN>(R, I.w, lo, min(I.N, lo + I.chunk), 0, h, D);
+    const double s = pass_block_dots(D.finish(), S::ND);
+    if ((int)threadIdx.x < S::ND) pset(I, NB > 0 ? pb ^ 1 : 0, threadIdx.x)[it.y] = s;
+    if (threadIdx.x == 0 && *R.dead) atomicExch(I.err, 1);
+  }
 }
 
-using KbBdotFn = void (*)(const InstDev*, const int2*, const Counts*, int);
-using KbBmgsFn = void (*)(const InstDev*, const int2*, const Counts*, int, int, int);
-static_assert(kGramB == 4, "kernel tables");
-const KbBdotFn kb_bdot_fn[kGramB] = {kb_bdot<1>, kb_bdot<2>, kb_bdot<3>, kb_bdot<4>};
-const KbBmgsFn kb_pass_fn[kGramB] = {kb_bmgs<4, 1>, kb_bmgs<4, 2>, kb_bmgs<4, 3>, kb_bmgs<4, 4>};
-const KbBmgsFn kb_last_fn[kGramB] = {kb_bmgs<1, 0>, kb_bmgs<2, 0>, kb_bmgs<3, 0>, kb_bmgs<4, 0>};
+// one CTA per instance: h_{j+1,j} = ||w||, the Gram row j+1 of v_{j+1} and
+// 1 / ||w|| from the last pass's partials (buffer pb, ng Gram sets), then the
+// Givens rotations of column j and the residual estimate
+__global__ void __launch_bounds__(32 * kBatchB) kb_givens(const InstDev* __restrict__ insts,
+                                                         const int* __restrict__ wi, const Counts* cnt, int j, int pb,
+                                                         int ng) {
+  for (int q = blockIdx.x; q < cnt->ni; q += gridDim.x) {
+    const InstDev& I = insts[wi[q]];
+    if (j < I.gm->kstop)
+      arnoldi_fold(pset(I, pb, 0), I.nchunks, ng, I.gm->H + j * (I.m + 1), I.gm->gram, kBatchB, I.gm, I.m, j, nullptr,
+                   0);
+    __syncthreads();
+  }
+}
+
+using KbPassFn = void (*)(const InstDev*, const int2*, const Counts*, int, int, int);
+// first dots with n + 1 vectors, a full block with n + 1 look-ahead dots, a
+// last block of n + 1 vectors
+struct KbPassTable {
+  KbPassFn dot[kBatchB], mid[kBatchB], last[kBatchB];
+  template <int... n>
+  explicit KbPassTable(std::integer_sequence<int, n...>)
+      : dot{kb_pass<0, n + 1>...}, mid{kb_pass<kBatchB, n + 1>...}, last{kb_pass<n + 1, 0>...} {}
+  KbPassTable() : KbPassTable(std::make_integer_sequence<int, kBatchB>()) {}
+};
+const KbPassTable kb_passes;
 
 __global__ void kb_lsq(const InstDev* __restrict__ insts, const int* __restrict__ wi, const Counts* cnt) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -461,12 +409,11 @@ __global__ void __launch_bounds__(kBT) kb_residual(const InstDev* __restrict__ i
 }
 
 __global__ void kb_set_bnorm(const InstDev* __restrict__ insts, const int* __restrict__ wi, const Counts* cnt) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= cnt->ni) return;
-  const InstDev& I = insts[wi[q]];
-  double s = 0.0;
-  for (int c = 0; c < I.nchunks; ++c) s += I.part[c];
-  I.gm->bnorm = sqrt(s);
+  for (int q = blockIdx.x; q < cnt->ni; q += gridDim.x) {   // one warp per instance
+    const InstDev& I = insts[wi[q]];
+    const double s = partials_sum_warp(I.part, I.nchunks);
+    if (threadIdx.x == 0) I.gm->bnorm = sqrt(s);
+  }
 }
 
 // start of a cycle: beta = ||r||, v_0 = r / beta, g = beta e_1, step budget
@@ -495,6 +442,7 @@ __global__ void __launch_bounds__(kBT) kb_cycle_start(const InstDev* __restrict_
       st.kstop = gm->kstop;
       st.kdone = gm->kdone;
       st.breakdown = gm->breakdown;
+      st.err = *I.err;
       status[it.x] = st;
     }
   }
@@ -691,14 +639,16 @@ rt_status grow(Server* S, T** p, size_t* cap, size_t need) {
 // the Jacobi inverse diagonal, partials, GMRES state
 size_t solver_bytes(int64_t N, int m, int nchunks) {
   auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  return al((size_t)(m + 1) * N * 8) + 7 * al((size_t)N * 8) + al((size_t)3 * kGramB * nchunks * 8) +
+  return al((size_t)(m + 1) * N * 8) + 7 * al((size_t)N * 8) + al((size_t)2 * kBatchB * nchunks * 8) +
          al(sizeof(GmresDev));
 }
 
-int64_t chunk_for(int64_t N) {
-  (void)N;
-  return 65536;
-}
+// Elements per work item of the vector kernels (a multiple of the block
+// passes' tile).  64 K elements left most SMs idle on a few instances and
+// rounded the items per CTA up badly on many; 8 K elements are 32 tiles, next to
+// which an item's reduction is a few per cent.
+constexpr int64_t kChunk = 8192;
+static_assert(kChunk % kPassTile == 0, "a chunk starts on a tile");
 
 template <int MODE>
 void formal32(Server* S, cudaStream_t st, int src, int dst, int step) {
@@ -815,15 +765,10 @@ rt_status autotune_grids(Server* S, int resident) {
   auto apply = [&] { enqueue_apply(S, st, 0, VW, mode, fp32, 0); RT_COUNT(fp32 ? 4 : 2); };
   tune(&S->grid_g, gs, apply);
   tune(&S->grid_h, hs, apply);
-  // the vector grid on the kernel that dominates the cycle: a full block
-  // pass (4 updates, 4 look-ahead dots) of Arnoldi step 7; it writes only
-  // w, one partial buffer and rows 0-3 of Hessenberg column 7, all of which
-  // step 7 of the cycle recomputes before reading them
+  // the vector grid on the residual pass; it writes only r and one buffer of
+  // partials, which the cycle recomputes before reading them
   tune(&S->grid_v, vs, [&] {
-    if (S->opts.restart >= 2 * kGramB)
-      kb_pass_fn[kGramB - 1]<<<S->grid_v, kBT, 0, st>>>(S->d_insts, S->d_wl_c, S->d_counts, 2 * kGramB - 1, 0, 0);
-    else
-      kb_bdot<1><<<S->grid_v, kBT, 0, st>>>(S->d_insts, S->d_wl_c, S->d_counts, 0);
+    kb_residual<<<S->grid_v, kBT, 0, st>>>(S->d_insts, S->d_wl_c, S->d_counts);
     RT_COUNT(1);
   });
   cudaEventDestroy(e0);
@@ -846,18 +791,20 @@ rt_status enqueue_batch_cycle(Server* S, cudaStream_t st) {
     // steps after the first normalise v_j = w / ||w|| inside the quadrature
     enqueue_apply(S, st, j, VW, mode, fp32, j, j > 0);
     int pb = 0;
-    kb_bdot_fn[std::min(kGramB, j + 1) - 1]<<<S->grid_v, kBT, 0, st>>>(I, S->d_wl_c, C, j); RT_COUNT(1);
-    for (int i0 = 0; i0 <= j; i0 += kGramB) {
-      const int nb = std::min(kGramB, j + 1 - i0);
-      const int nn = std::max(0, std::min(kGramB, j + 1 - (i0 + nb)));
-      (nn ? kb_pass_fn[nn - 1] : kb_last_fn[nb - 1])<<<S->grid_v, kBT, 0, st>>>(I, S->d_wl_c, C, j, i0, pb); RT_COUNT(1);
+    const int gp = 2 * S->sms;   // the passes' resident CTAs
+    kb_passes.dot[std::min(kBatchB, j + 1) - 1]<<<gp, kPassThreads, kPassDynSmem, st>>>(I, S->d_wl_c, C, j, 0, 0); RT_COUNT(1);
+    for (int i0 = 0; i0 <= j; i0 += kBatchB) {
+      const int nb = std::min(kBatchB, j + 1 - i0);
+      const int nn = std::max(0, std::min(kBatchB, j + 1 - (i0 + nb)));
+      (nn ? kb_passes.mid[nn - 1] : kb_passes.last[nb - 1])<<<gp, kPassThreads, kPassDynSmem, st>>>(I, S->d_wl_c, C, j,
+                                                                                                    i0, pb); RT_COUNT(1);
       pb ^= 1;
     }
     // h_{j+1,j}, the Gram row, the rotations and the inverse norm that the
     // next step's quadrature scales w by; an instance that stops at step j
     // never forms v_{j+1}, which no later kernel of the cycle reads
-    const int ng = (j + 1) % kGramB;
-    kb_givens<<<S->grid_i, kInstThreads, 0, st>>>(I, S->d_wl_i, C, j, pb, ng); RT_COUNT(1);
+    const int ng = (j + 1) % kBatchB;
+    kb_givens<<<std::min(S->opts.max_slots, 4 * S->sms), 32 * kBatchB, 0, st>>>(I, S->d_wl_i, C, j, pb, ng); RT_COUNT(1);
   }
   kb_lsq<<<S->grid_i, kInstThreads, 0, st>>>(I, S->d_wl_i, C); RT_COUNT(1);
   if (mode == KM_LOCAL_LAMBDA) {
@@ -979,7 +926,7 @@ rt_status make_instance(Server* S, Request* rq, Instance* in, int slot) {
   RT_TRY(setup_device_tables(&P, S->st));
   const int m = S->opts.restart;
   const int64_t N = P.N;
-  const int64_t chunk = chunk_for(N);
+  const int64_t chunk = kChunk;
   const int nchunks = (int)((N + chunk - 1) / chunk);
   const size_t bytes = solver_bytes(N, m, nchunks);
   void* blk = nullptr;
@@ -999,8 +946,9 @@ rt_status make_instance(Server* S, Request* rq, Instance* in, int slot) {
     p += al((size_t)N * 8);
   }
   D.part = reinterpret_cast<double*>(p);
-  p += al((size_t)3 * kGramB * nchunks * 8);
+  p += al((size_t)2 * kBatchB * nchunks * 8);
   D.gm = reinterpret_cast<GmresDev*>(p);
+  D.err = P.dev_err;
   D.Ns = P.Ns;
   D.Nmu = P.Nmu;
   D.Nnu = P.Nnu;
@@ -1069,7 +1017,7 @@ rt_status start_instances(Server* S, const std::vector<Instance*>& fresh) {
   Counts cn{0, 0, (int)c.size(), (int)wi.size(), {0, 0, 0}, {0, 0, 0}};
   RT_TRY_CUDA(cudaMemcpyAsync(S->d_new_counts, &cn, sizeof cn, cudaMemcpyHostToDevice, S->st));
   kb_residual<<<S->grid_v, kBT, 0, S->st>>>(S->d_insts, S->d_wl_new_c, S->d_new_counts); RT_COUNT(1);
-  kb_set_bnorm<<<(int)((wi.size() + kInstThreads - 1) / kInstThreads), kInstThreads, 0, S->st>>>(
+  kb_set_bnorm<<<(int)std::min<size_t>(wi.size(), 4 * S->sms), 32, 0, S->st>>>(
       S->d_insts, S->d_wl_new_i, S->d_new_counts); RT_COUNT(1);
   kb_cycle_start<<<S->grid_v, kBT, 0, S->st>>>(S->d_insts, S->d_wl_new_c, S->d_new_counts, S->d_status); RT_COUNT(1);
   RT_TRY_CUDA(cudaGetLastError());
@@ -1244,7 +1192,8 @@ void worker_main(Server* S) {
       in->cycles += 1;
       const InstStatus& st = hs[q];
       rt_status fin = RT_EPENDING;
-      if (st.rel != st.rel) fin = RT_ENUMERIC;
+      if (st.err) fin = RT_ETIMEOUT;
+      else if (st.rel != st.rel) fin = RT_ENUMERIC;
       else if (st.rel < in->req->rtol) fin = RT_OK;
       else if (st.iters >= in->req->maxit) fin = RT_ENOTCONV;
       else if (st.breakdown && st.kdone == 0) fin = RT_EBREAKDOWN;
@@ -1318,8 +1267,11 @@ static rt_status create_server(const rt_server_opts* opts, const rt_allocator* h
   }
   e = cudaStreamCreateWithFlags(&S->st, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S->cap, cudaStreamNonBlocking);
+  for (int i = 0; i < kBatchB; ++i)
+    for (KbPassFn f : {kb_passes.dot[i], kb_passes.mid[i], kb_passes.last[i]})
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassDynSmem);
   if (e != cudaSuccess) {
-    set_error("server stream creation failed: %s", cudaGetErrorString(e));
+    set_error("server set-up failed: %s", cudaGetErrorString(e));
     rt_server_destroy(srv);
     return RT_ECUDA;
   }

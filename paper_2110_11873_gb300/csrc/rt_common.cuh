@@ -68,8 +68,8 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 constexpr int kBlockVec = 512;          // threads per block of the vector kernels
 constexpr int kMaxPartials = 2048;      // upper bound on reduction partials per column
 constexpr int kMaxRestart = 160;         // longest GMRES cycle (the paper runs GMRES unrestarted, up to 134 steps)
-constexpr int kGramB = 4;                // basis vectors per block pass of rt_arnoldi_bmgs and of the batch
-constexpr int kGramMax = 8;              // basis vectors per block pass inside the single-instance GMRES
+constexpr int kGramB = 4;                // basis vectors per block pass of rt_arnoldi_bmgs
+constexpr int kGramMax = 8;              // basis vectors per block pass inside GMRES
 
 // device-side state of a GMRES cycle (lives in device memory).  The scalars
 // come first: the host reads only that header (kGmresHeader bytes) after a
@@ -198,7 +198,10 @@ __device__ inline void arnoldi_fold(const double* __restrict__ part, int Gp, int
     const double inv = hn > 0.0 ? 1.0 / hn : 0.0;
     hcol[j + 1] = hn;
     for (int d = 1; d <= ng; ++d) gram[(j + 1) * gb + d] = sets[1 + ng - d] * inv;
-    if (gm) givens_step(gm, m, j, hist, hist_cap);
+    if (gm) {
+      gm->vscale = inv;
+      givens_step(gm, m, j, hist, hist_cap);
+    }
   }
 }
 
