@@ -125,21 +125,20 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cud
   return launch_pdl_smem(kernel, grid, block, 0, st, args...);
 }
 
-// sum of G partials in a fixed order (lane-strided trees, then a fixed
-// shuffle tree); every lane of the calling warp gets the result
+// sum of G partials in a fixed order (lane-strided, then a fixed shuffle
+// tree); every lane of the calling warp gets the result
 __device__ __forceinline__ double partials_sum_warp(const double* __restrict__ part, int G) {
   const int lane = threadIdx.x & 31;
-  constexpr int U = 8;   // loads in flight per lane, added as a tree
+  constexpr int U = 8;   // loads in flight per lane
   double s = 0.0;
   for (int i0 = lane; i0 < G; i0 += 32 * U) {
     double v[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = i0 + 32 * u < G ? part[i0 + 32 * u] : 0.0;
+    for (int u = 0; u < U; ++u)
+      if (i0 + 32 * u < G) v[u] = part[i0 + 32 * u];
 #pragma unroll
-    for (int o = U / 2; o > 0; o >>= 1)
-#pragma unroll
-      for (int u = 0; u < o; ++u) v[u] += v[u + o];
-    s += v[0];
+    for (int u = 0; u < U; ++u)
+      if (i0 + 32 * u < G) s += v[u];
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -248,16 +247,30 @@ struct BicgDev {
 };
 
 // Column of the FP64 step-coefficient tables for ray r = m*Nnu + p.  Without
-// a downwind term the coefficients of a step depend on |mu| only, so the
-// tables hold one column per (|mu|, p) that both directions share (shared =
-// 1, nray/2 columns): m < Nh (mu < 0) reads column (Nh-1-m)*Nnu + p, m >= Nh
-// column (m-Nh)*Nnu + p.  DELO-parabolic's coefficients include the downwind
-// interval, which differs between the directions: one column per ray.
+// a downwind term the coefficients of a step depend on |mu| and on the
+// profile at p only.
+//   CS_RAY    one column per ray (DELO-parabolic: its coefficients include the
+//             downwind interval, which differs between the directions)
+//   CS_MU     one column per (|mu|, p) that both directions share: m < Nh
+//             (mu < 0) reads column (Nh-1-m)*Nnu + p, m >= Nh (m-Nh)*Nnu + p
+//   CS_PAIR   the same for a profile that is symmetric on the grid: one
+//             column per |mu| and pair of frequencies p, Nnu-1-p
+enum CoefShare { CS_RAY = 0, CS_MU = 1, CS_PAIR = 2 };
+// Vector length from which a symmetric profile takes the paired FP64 kernels
+// (k_psweep, moments_pair64).  Above it the FP64 pipe bounds the apply and
+// sharing the work of a pair pays (N = 51.5 million: 621 -> 446 us with the
+// paired sweep alone); below, the quarter of the units is bound by latency
+// (N = 47,040: 17.5 -> 18.2 us; N = 1.9 million: 38.9 -> 35.5 us, not worth
+// another rounding of the operator, which BiCGSTAB and CGS amplify).
+constexpr int64_t kPairMinN = (int64_t)4 << 20;
+__host__ __device__ __forceinline__ int pair_count(int Nnu) { return (Nnu + 1) / 2; }
 __host__ __device__ __forceinline__ int64_t coef_col(int64_t r, int Nh, int Nnu, int shared) {
-  if (!shared) return r;
+  if (shared == CS_RAY) return r;
   const int m = (int)(r / Nnu);
-  const int64_t p = r - (int64_t)m * Nnu;
-  return (int64_t)(m < Nh ? Nh - 1 - m : m - Nh) * Nnu + p;
+  const int p = (int)(r - (int64_t)m * Nnu);
+  const int64_t mm = m < Nh ? Nh - 1 - m : m - Nh;
+  if (shared == CS_PAIR) return mm * pair_count(Nnu) + (p < Nnu - 1 - p ? p : Nnu - 1 - p);
+  return mm * Nnu + p;
 }
 
 // Device memory source of a problem: NULL means cudaMalloc/cudaFree; the
@@ -297,21 +310,25 @@ struct Problem {
   int ngroups = 0;
   int ntile64 = 1, ntile32 = 1;   // depth tiles per ray group (FP64 / FP32 kernels)
   // FP64 device tables
-  int cshare = 0;          // 1: the FP64 tables hold one column per (|mu|, p), shared by both directions
-  int64_t cstride = 0;     // columns of the FP64 tables: nray/2 (shared) or nray (DELO-parabolic)
+  int cshare = 0;          // CoefShare: which rays share a column of the FP64 tables
+  int64_t cstride = 0;     // columns of the FP64 tables
+  // FP64 formal solver, CS_PAIR: one lane per direction and frequency pair
+  // (npair = 2 Nh (Nnu+1)/2 of them, the downward half first); else 0
+  int64_t npair = 0;
+  int ngroups64 = 0;       // groups of 32 lanes of the FP64 formal solver (rays, or pairs)
   double* ce = nullptr;    // [(Ns-1)][cstride] step factor e of the interval (i, i+1), column coef_col(r)
   double* ca = nullptr;    // ... alpha (coefficient of the upwind S)
   double* cb = nullptr;    // ... beta  (coefficient of S at the new node)
   double* cg = nullptr;    // ... gamma (DELO-parabolic only: coefficient of S at the downwind node)
-  double* Etile = nullptr; // [ntile64-1][nray] FP64 formal solver: slope of each depth tile's map
+  double* Etile = nullptr; // [ntile64-1][nray or npair] FP64 formal solver: slope of each depth tile's map
   // sigma-form SOR / SSOR: the assembled matrix A (row-major n x n, n = Nop),
   // the dense P^-1 (row-major), a triangular-inverse scratch and a vector
   double *Asig = nullptr, *Mpre = nullptr, *Mtri = nullptr, *Mscr = nullptr;
   int asig_ready = 0;        // Asig holds the assembled matrix
   int mpre_kind = 0;         // RT_PREC_SOR / RT_PREC_SSOR that Mpre holds (0: none)
   double mpre_omega = 0.0;
-  double* Bmap = nullptr;  // [2*ngroups][ntile64-1][32] FP64 formal solver: offsets of the tile maps
-  double* Kmap = nullptr;  // [ntile64-1][L+2][nray] weights of the map offsets in the node source values
+  double* Bmap = nullptr;  // [2*ngroups64][ntile64-1][32] FP64 formal solver: offsets of the tile maps
+  double* Kmap = nullptr;  // [ntile64-1][L+2][nray or npair] weights of the map offsets in the node source values
   double* wray = nullptr;  // [3][nray] hat-w_m * hat-w_p, the same times T201_m, times T202_m
   double* wjac = nullptr;  // [3][Ns][nray] wray times the Jacobi inverse diagonal (I, I, Q), once a solver set it
   double* wI2 = nullptr;   // [Nnu] spectral weights hat-w_p

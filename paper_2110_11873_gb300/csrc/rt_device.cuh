@@ -10,7 +10,8 @@ namespace {
 
 constexpr int kMomThreads = 256;
 constexpr int kMaxTiles = 8;     // FP32 kernel: up to 256 threads per CTA (255 registers a lane)
-constexpr int kMaxTiles64 = 16;  // FP64 formal solver: depth tiles per ray group (one warp each)
+constexpr int kMaxTilesRay = 16; // FP64 formal solver on rays: depth tiles per ray group (one warp each)
+constexpr int kMaxTiles64 = 32;  // FP64 formal solver on pairs of rays: the same
 constexpr int kRing = 8;         // prefetch depth of the FP64 formal-solver kernel (steps)
 constexpr int kRing32 = 16;      // prefetch depth of the FP32 kernel (one lane carries I and Q)
 
@@ -134,6 +135,48 @@ __device__ __forceinline__ void moments_height(
   }
 }
 
+// the end of the FP64 quadrature of height k: the CTA's sums of a0 (J00) and
+// a1 (J20) in a fixed order, then sigma and S
+template <int MODE>
+__device__ __forceinline__ void moments_finish64(double a0, double a1, const double* __restrict__ t201,
+                                                 const double* __restrict__ t202, const double* __restrict__ Minv,
+                                                 int Ns, int Nmu, double xi, double xiW2, double* __restrict__ S,
+                                                 int k) {
+  // transposed warp sum: lanes 0-15 get the sum of a0, lanes 16-31 of a1
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool h16 = lane & 16;
+  double t = (h16 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h16 ? a0 : a1, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  __shared__ double red[2][32];
+  __shared__ double sig[2];
+  if ((lane & 15) == 0) red[lane >> 4][warp] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int nw = blockDim.x >> 5;
+    double j00 = 0.0, j20 = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      j00 += red[0][w];
+      j20 += red[1][w];
+    }
+    double s0 = xi * j00, s2 = xiW2 * j20;
+    if (MODE == KM_LOCAL_LAMBDA) {
+      const double* Mi = Minv + 4 * k;
+      const double u0 = Mi[0] * s0 + Mi[1] * s2;
+      const double u2 = Mi[2] * s0 + Mi[3] * s2;
+      s0 = u0;
+      s2 = u2;
+    }
+    sig[0] = s0;
+    sig[1] = s2;
+  }
+  __syncthreads();
+  for (int m = threadIdx.x; m < Nmu; m += blockDim.x) {
+    S[(int64_t)k * Nmu + m] = sig[0] + t201[m] * sig[1];
+    S[((int64_t)Ns + k) * Nmu + m] = t202[m] * sig[1];
+  }
+}
+
 // FP64 quadrature of height k as flat dot products over its rays (the CTA's
 // threads stride over r): with the per-ray weights w0 = hat-w_m hat-w_p,
 // w1 = w0 T201_m, w2 = w0 T202_m (wray, [3][nray]),
@@ -178,40 +221,50 @@ __device__ __forceinline__ void moments_flat64(const double* __restrict__ x, con
     a1 = fma(w1[r], vI, a1);
     a2 = fma(w2[r], vQ, a2);
   }
-  a1 += a2;
-  // transposed warp sum: lanes 0-15 get the sum of a0, lanes 16-31 of a1
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool h16 = lane & 16;
-  double t = (h16 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h16 ? a0 : a1, 16);
+  moments_finish64<MODE>(a0, a1 + a2, t201, t202, Minv, Ns, Nmu, xi, xiW2, S, k);
+}
+
+// moments_flat64 for a profile symmetric on the frequency grid, modes PLAIN
+// and LOCAL_LAMBDA: the rays (+-mu, p) and (+-mu, Nnu-1-p) have the same
+// weights, so the four values are added first: 9 operations for 8 elements
+// (I and Q) instead of 12.  The FP64 pipe bounds it on large problems.
+template <int MODE, bool NORM = false>
+__device__ __forceinline__ void moments_pair64(const double* __restrict__ x, const double* __restrict__ wray,
+                                               const double* __restrict__ t201, const double* __restrict__ t202,
+                                               const double* __restrict__ Minv, int Ns, int Nmu, int64_t nray,
+                                               double xi, double xiW2, double* __restrict__ S, int k,
+                                               double inv = 1.0, double* __restrict__ xout = nullptr) {
+  const int Nh = Nmu / 2, Nnu = (int)(nray / Nmu), np = pair_count(Nnu);
+  const int64_t oI = (int64_t)k * nray, oQ = ((int64_t)Ns + k) * nray;
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+  for (int q = threadIdx.x; q < Nh * np; q += blockDim.x) {
+    const int mm = q / np, p = q - mm * np, p2 = Nnu - 1 - p;
+    const int up = (Nh + mm) * Nnu, dn = (Nh - 1 - mm) * Nnu;
+    const int r[4] = {up + p, dn + p, up + p2, dn + p2};
+    const int n = p == p2 ? 2 : 4;   // the middle frequency is its own mirror
+    double vI[4], vQ[4];
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  __shared__ double red[2][32];
-  __shared__ double sig[2];
-  if ((lane & 15) == 0) red[lane >> 4][warp] = t;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = blockDim.x >> 5;
-    double j00 = 0.0, j20 = 0.0;
-    for (int w = 0; w < nw; ++w) {
-      j00 += red[0][w];
-      j20 += red[1][w];
+    for (int i = 0; i < 4; ++i) {
+      vI[i] = i < n ? x[oI + r[i]] : 0.0;
+      vQ[i] = i < n ? x[oQ + r[i]] : 0.0;
     }
-    double s0 = xi * j00, s2 = xiW2 * j20;
-    if (MODE == KM_LOCAL_LAMBDA) {
-      const double* Mi = Minv + 4 * k;
-      const double u0 = Mi[0] * s0 + Mi[1] * s2;
-      const double u2 = Mi[2] * s0 + Mi[3] * s2;
-      s0 = u0;
-      s2 = u2;
+    if (NORM) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        vI[i] *= inv;
+        vQ[i] *= inv;
+        if (i < n) {
+          xout[oI + r[i]] = vI[i];
+          xout[oQ + r[i]] = vQ[i];
+        }
+      }
     }
-    sig[0] = s0;
-    sig[1] = s2;
+    const double sI = (vI[0] + vI[1]) + (vI[2] + vI[3]), sQ = (vQ[0] + vQ[1]) + (vQ[2] + vQ[3]);
+    a0 = fma(wray[r[0]], sI, a0);
+    a1 = fma(wray[nray + r[0]], sI, a1);
+    a2 = fma(wray[2 * nray + r[0]], sQ, a2);
   }
-  __syncthreads();
-  for (int m = threadIdx.x; m < Nmu; m += blockDim.x) {
-    S[(int64_t)k * Nmu + m] = sig[0] + t201[m] * sig[1];
-    S[((int64_t)Ns + k) * Nmu + m] = t202[m] * sig[1];
-  }
+  moments_finish64<MODE>(a0, a1 + a2, t201, t202, Minv, Ns, Nmu, xi, xiW2, S, k);
 }
 
 // --------------------------------------------------------------- K2: Lambda
@@ -258,7 +311,8 @@ struct FormalArgs {
   const double* cb;
   const double* cg;       // DELO-parabolic: downwind coefficient table (else NULL)
   int64_t cstride;        // columns of the FP64 tables (coef_col)
-  int cshare;             // 1: one column per (|mu|, p) shared by both directions
+  int cshare;             // CoefShare
+  int64_t npair;          // FP64, CS_PAIR: lanes (direction, frequency pair); else 0
   const float* dtau32;    // FP32: interval optical depths
   const float* r32;       // FP32: per-ray scale phi_hat/|mu|
   const void* S;          // source functions (TC) [2][Ns][Nmu]

@@ -13,6 +13,8 @@
 //              CTA each, so they spread evenly over the SMs -- chain the maps
 //              of the tiles before their own (the slopes E are a setup
 //              table) and sweep their tile with the output.
+//   k_psweep   the same units where the profile is symmetric on the frequency
+//              grid: a lane marches the rays p and Nnu-1-p together.
 //   k_formal   formal solver Lambda (Eq. 9-10) along every ray, writing
 //              y_k = z_k - I_k on the fly.  A CTA owns one group of 32 rays of
 //              the same direction sign (so the 32 lanes of a warp read one
@@ -59,7 +61,8 @@ __global__ void k_coeffs64(const double* __restrict__ dtau, const double* __rest
     const int64_t c = t % cstride;
     const int i = (int)(t / cstride);
     // the ray this column stands for (shared columns: the upward ray of that |mu| and p)
-    const int64_t r = shared ? ((int64_t)Nh + c / Nnu) * Nnu + c % Nnu : c;
+    const int np = shared == CS_PAIR ? pair_count(Nnu) : Nnu;
+    const int64_t r = shared ? ((int64_t)Nh + c / np) * Nnu + c % np : c;
     const double D = dtau[i] * rscale[r];
     double e, al, be;
     if (fs == RT_FS_DELO_LINEAR || fs == RT_FS_DELO_PARABOLIC) {
@@ -231,21 +234,23 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(
 }
 
 // FP64 quadrature, one CTA per height (flat over the rays); WJ: Jacobi mode
-// with the per-element weights of k_jacobi_weights in place of wray
+// with the per-element weights of k_jacobi_weights in place of wray; PAIR:
+// symmetric profile (moments_pair64)
 constexpr int kMom64Threads = 512;
-template <int MODE, bool WJ = false>
+template <int MODE, bool WJ = false, bool PAIR = false>
 __global__ void __launch_bounds__(kMom64Threads) k_moments64(
     const double* __restrict__ x, const double* __restrict__ dinv, const double* __restrict__ wray,
     const double* __restrict__ t201, const double* __restrict__ t202, const double* __restrict__ Minv, int Ns,
     int Nmu, int64_t nray, double xi, double xiW2, double* __restrict__ S, const int* kstop, int step) {
   if (kstop && step >= *kstop) return;
-  moments_flat64<MODE, WJ>(x, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
+  if (PAIR) moments_pair64<MODE>(x, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
+  else moments_flat64<MODE, WJ>(x, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
 }
 
 // GMRES (NormIn): block 0 ends Arnoldi step nin.jprev (fold and Givens
 // rotations, Sect. 2.1); blocks 1..Ns normalise u into x = u / ||u|| while
 // forming the quadrature of x (Eq. 11-14) for height blockIdx.x - 1
-template <int MODE, bool WJ>
+template <int MODE, bool WJ, bool PAIR>
 __global__ void __launch_bounds__(kMom64Threads) k_moments64_norm(
     double* __restrict__ x, const double* __restrict__ dinv, const double* __restrict__ wray,
     const double* __restrict__ t201, const double* __restrict__ t202, const double* __restrict__ Minv, int Ns,
@@ -257,8 +262,11 @@ __global__ void __launch_bounds__(kMom64Threads) k_moments64_norm(
     return;
   }
   const double inv = arnoldi_inv_norm(nin.part, nin.Gp);
-  moments_flat64<MODE, WJ, true>(nin.u, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x - 1,
-                                 inv, x);
+  if (PAIR)
+    moments_pair64<MODE, true>(nin.u, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x - 1, inv, x);
+  else
+    moments_flat64<MODE, WJ, true>(nin.u, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x - 1,
+                                   inv, x);
 }
 
 // wjac[q][k][r] = wray[q][r] * D^-1 of element (k, r): Stokes I for q = 0, 1
@@ -429,24 +437,36 @@ static rt_status upload(Problem* P, T** dst, const std::vector<T>& src, cudaStre
   return RT_OK;
 }
 
-// Depth tiles per ray group.  FP64: the formal solver's warp units spread
+// Depth tiles per lane group.  FP64, rays (k_fsweep): the warp units spread
 // evenly over the SMs, so an SM carries ceil(units / SMs) of them.  A step
 // costs a sweep unit 4 FP64 operations; an SM retires one FP64 warp
 // operation in about kFp64OpCycles, while one warp alone needs about
 // kFp64StepCycles per step (the dependent chain through I; both measured on
 // GB300), and the sweep takes the longer of the two.  The map offsets cost 2
 // independent FMAs per tile node and ray (pipe time only).  T minimises the
-// sum.  FP32: tiles are cheap, so aim
+// sum.  FP64, pairs (k_psweep): as many units as are resident at once
+// (kPairResident per SM); N_s = 2000, N_mu = 64, N_nu = 201 took 616, 596, 485,
+// 450 and 446 us per apply with 3, 4, 6, 9 and 12 tiles, N_s = 500 170, 140, 133
+// and 131 us with 3, 6, 9 and 12.  FP32: tiles are cheap, so aim
 // at about 16 warps per SM with tiles of at least 2*kRing steps.
 constexpr double kFp64OpCycles = 20.0, kFp64StepCycles = 600.0;
+constexpr int kPairRing = 4;        // prefetch depth of k_psweep (steps)
+constexpr int kPairWarps = 4;       // units per CTA of k_psweep: one per SM quarter
+constexpr int kPairResident = 16;   // units per SM at 128 registers a lane
 static int choose_tiles64(const Problem* P) {
-  const int64_t sms = P->num_sms, groups = 2LL * P->ngroups;
+  const int64_t sms = P->num_sms;
+  if (P->npair) {
+    int T = (int)std::max<int64_t>(1, std::min<int64_t>(kMaxTiles64, kPairResident * sms / P->ngroups64));
+    while (T > 1 && (P->Ns - 1 + T - 1) / T < 2 * kPairRing) --T;
+    return T;
+  }
+  const int64_t groups = 2LL * P->ngroups;
   auto kernel = [&](int64_t units, double ops) {
     return std::max((double)((units + sms - 1) / sms) * ops * kFp64OpCycles, kFp64StepCycles);
   };
   int best = 1;
   double best_cost = 1e300;
-  for (int T = 1; T <= kMaxTiles64; ++T) {
+  for (int T = 1; T <= kMaxTilesRay; ++T) {
     const int L = (P->Ns - 1 + T - 1) / T;
     if (T > 1 && L < 2 * kRing) break;
     const double maps = (double)(T - 1) * P->nray * (L + 2) * 2.0 / 32.0 / (double)sms * kFp64OpCycles;
@@ -471,15 +491,24 @@ __device__ __forceinline__ void group_ray(const FormalArgs& A, int g, int lane, 
   m = (int)(r / A.Nnu);
 }
 
-// slope of tile t's map for every ray, E = product of the e coefficients of
-// its steps in marching order: Etile[t][r], t < T-1 (setup)
-__global__ void k_etile(const double* __restrict__ ce, int Ns, int64_t nray, int64_t nd, int T, int64_t cstride,
+// the ray of lane u of the FP64 formal solver: ray u itself, or with CS_PAIR
+// the first ray of pair u (nlane pairs, the downward half first)
+__device__ __forceinline__ int64_t lane_ray(int64_t u, int64_t nlane, int Nh, int Nnu, int shared) {
+  if (shared != CS_PAIR) return u;
+  const int64_t half = nlane / 2, q = u < half ? u : u - half;
+  const int np = pair_count(Nnu);
+  return ((u < half ? 0 : Nh) + q / np) * Nnu + q % np;
+}
+
+// slope of tile t's map for every lane, E = product of the e coefficients of
+// its steps in marching order: Etile[t][u], t < T-1 (setup)
+__global__ void k_etile(const double* __restrict__ ce, int Ns, int64_t nlane, int64_t nd, int T, int64_t cstride,
                         int shared, int Nh, int Nnu, double* __restrict__ Etile) {
   const int L = (Ns - 1 + T - 1) / T;
-  const int64_t n = (int64_t)(T - 1) * nray;
+  const int64_t n = (int64_t)(T - 1) * nlane;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int t = (int)(i / nray);
-    const int64_t r = i % nray;
+    const int t = (int)(i / nlane);
+    const int64_t r = lane_ray(i % nlane, nlane, Nh, Nnu, shared);
     const bool down = r < nd;
     const int j0 = 1 + t * L, j1 = min(Ns, j0 + L);
     const int64_t col = coef_col(r, Nh, Nnu, shared);
@@ -498,35 +527,35 @@ __global__ void k_etile(const double* __restrict__ ce, int Ns, int64_t nray, int
 //     B(t, r, s) = sum_n K[t][n][r] S_s(node j0 - 1 + n, m(r)).
 // k_kmap builds K at setup (one backward pass per tile and ray); the map
 // kernel is then one independent FMA per node instead of a dependent
-// recurrence.  K[t][n][r], n < L + 2.
+// recurrence.  K[t][n][lane], n < L + 2 (lane: lane_ray).
 __global__ void k_kmap(const double* __restrict__ ce, const double* __restrict__ ca, const double* __restrict__ cb,
-                       const double* __restrict__ cg, int Ns, int64_t nray, int64_t nd, int T, int64_t cstride,
+                       const double* __restrict__ cg, int Ns, int64_t nlane, int64_t nd, int T, int64_t cstride,
                        int shared, int Nh, int Nnu, double* __restrict__ K) {
   const int L = (Ns - 1 + T - 1) / T;
-  const int64_t n = (int64_t)(T - 1) * nray;
+  const int64_t n = (int64_t)(T - 1) * nlane;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int t = (int)(i / nray);
-    const int64_t r = i % nray;
+    const int t = (int)(i / nlane);
+    const int64_t u = i % nlane, r = lane_ray(u, nlane, Nh, Nnu, shared);
     const bool down = r < nd;
     const int j0 = 1 + t * L, j1 = min(Ns, j0 + L);
-    double* __restrict__ Kt = K + (int64_t)t * (L + 2) * nray + r;
-    for (int q = 0; q < L + 2; ++q) Kt[(int64_t)q * nray] = 0.0;
+    double* __restrict__ Kt = K + (int64_t)t * (L + 2) * nlane + u;
+    for (int q = 0; q < L + 2; ++q) Kt[(int64_t)q * nlane] = 0.0;
     const int64_t col = coef_col(r, Nh, Nnu, shared);
     double Pj = 1.0;   // product of e over the steps after j
     for (int j = j1 - 1; j >= j0; --j) {
       const int64_t c = (int64_t)(down ? j - 1 : Ns - 1 - j) * cstride + col;
       const int q = j - j0 + 1;   // local index of node j
-      Kt[(int64_t)q * nray] += Pj * cb[c];
-      Kt[(int64_t)(q - 1) * nray] += Pj * ca[c];
-      if (cg) Kt[(int64_t)(q + 1) * nray] += Pj * cg[c];
+      Kt[(int64_t)q * nlane] += Pj * cb[c];
+      Kt[(int64_t)(q - 1) * nlane] += Pj * ca[c];
+      if (cg) Kt[(int64_t)(q + 1) * nlane] += Pj * cg[c];
       Pj *= ce[c];
     }
   }
 }
 
 // the map offsets B of tiles t < T-1 for both Stokes parameters, written as
-// Bmap[g * 2 + s][t][lane] for the sweep kernel.  A CTA takes 32 rays of one
-// tile (x) and splits the tile's nodes over kMapSlices thread rows (y), so
+// Bmap[g * 2 + s][t][lane] for the sweep kernel.  A CTA takes 32 lanes (rays or
+// pairs) of one tile (x) and splits the tile's nodes over kMapSlices thread rows (y), so
 // many loads are in flight; the rows' partial sums are added in a fixed order.
 constexpr int kMapSlices = 8;
 __global__ void __launch_bounds__(32 * kMapSlices) k_fmapdot(const FormalArgs A, const double* __restrict__ K,
@@ -534,20 +563,20 @@ __global__ void __launch_bounds__(32 * kMapSlices) k_fmapdot(const FormalArgs A,
   if (A.kstop && A.step >= *A.kstop) return;
   pdl_wait();   // the source values of the quadrature before
   const int Ns = A.Ns, T = A.ntile, L = (Ns - 1 + T - 1) / T;
-  const int64_t nray = A.nray;
+  const int64_t nlane = A.npair ? A.npair : A.nray, half = A.npair ? nlane / 2 : A.nd;   // lanes, downward ones
   const int t = blockIdx.y;
-  const int64_t r = (int64_t)blockIdx.x * 32 + threadIdx.x;
-  const bool valid = r < nray;
-  const int64_t rc = valid ? r : nray - 1;
+  const int64_t u = (int64_t)blockIdx.x * 32 + threadIdx.x;
+  const bool valid = u < nlane;
+  const int64_t uc = valid ? u : nlane - 1;
   const double* __restrict__ S = reinterpret_cast<const double*>(A.S);
   const int64_t sQ = (int64_t)Ns * A.Nmu;
-  const bool down = rc < A.nd;
-  const int m = (int)(rc / A.Nnu);
+  const bool down = uc < half;
+  const int m = (int)(lane_ray(uc, nlane, A.Nmu / 2, A.Nnu, A.cshare) / A.Nnu);
   const int j0 = 1 + t * L, jend = min(Ns - 1, j0 + L);   // nodes j0-1 .. jend
-  const double* __restrict__ Kt = K + (int64_t)t * (L + 2) * nray + rc;
+  const double* __restrict__ Kt = K + (int64_t)t * (L + 2) * nlane + uc;
   double bI = 0.0, bQ = 0.0;
   for (int j = j0 - 1 + (int)threadIdx.y; j <= jend; j += kMapSlices) {
-    const double k = Kt[(int64_t)(j - j0 + 1) * nray];
+    const double k = Kt[(int64_t)(j - j0 + 1) * nlane];
     const int64_t o = (int64_t)(down ? j : Ns - 1 - j) * A.Nmu + m;
     bI = fma(k, S[o], bI);
     bQ = fma(k, S[sQ + o], bQ);
@@ -560,7 +589,7 @@ __global__ void __launch_bounds__(32 * kMapSlices) k_fmapdot(const FormalArgs A,
     double b = 0.0;
 #pragma unroll
     for (int y = 0; y < kMapSlices; ++y) b += red[threadIdx.y][y][threadIdx.x];
-    const int64_t rr = down ? r : r - A.nd;
+    const int64_t rr = down ? u : u - half;
     const int g = (int)(rr / 32) + (down ? 0 : A.ngd), lane = (int)(rr % 32);
     Bmap[((size_t)(2 * g + threadIdx.y) * (T - 1) + t) * 32 + lane] = b;
   }
@@ -604,6 +633,157 @@ __global__ void __launch_bounds__(32, FS == RT_FS_DELO_PARABOLIC ? 12 : 16) k_fs
   }
 }
 
+// The same for a profile that is symmetric on the frequency grid (CS_PAIR).
+// The source functions do not depend on the frequency, so the rays p and
+// Nnu-1-p of a direction have the same step coefficients and the same I and Q:
+// one lane marches the pair once, both Stokes parameters, and writes the four
+// outputs y = z - I.  Per step that is 6 operations of the recurrence and one
+// per output, 2.5 per element instead of 4, and half of the map offsets and of
+// the tables.  The FP64 pipe bounds it; a unit is one warp (32 pairs, one tile),
+// four to a CTA, so that each quarter of an SM gets its share.
+template <int MODE>
+__global__ void __launch_bounds__(32 * kPairWarps) k_psweep(const FormalArgs A, const double* __restrict__ Bmap,
+                                                            const double* __restrict__ Etile, int units) {
+  if (A.kstop && A.step >= *A.kstop) return;
+  pdl_wait();   // as k_fsweep: a dependent of k_fmapdot that releases none of its own early
+  const int lane = threadIdx.x & 31, unit = blockIdx.x * kPairWarps + (threadIdx.x >> 5);
+  if (unit >= units) return;
+  const int Ns = A.Ns, Nh = A.Nmu / 2, Nnu = A.Nnu, np = pair_count(Nnu);
+  const int T = A.ntile, L = (Ns - 1 + T - 1) / T;
+  const int t = unit % T, g = unit / T;
+  const int64_t half = A.npair / 2;
+  const bool down = g < A.ngd;
+  const int64_t qi = (int64_t)(down ? g : g - A.ngd) * 32 + lane;
+  const bool active = qi < half;
+  const int64_t q = active ? qi : half - 1;
+  const int m = (down ? 0 : Nh) + (int)(q / np), p = (int)(q % np);
+  const bool active2 = active && p != Nnu - 1 - p;   // the middle frequency is its own mirror
+  const int64_t u = (down ? 0 : half) + q;
+  const int64_t col = (int64_t)(down ? Nh - 1 - m : m - Nh) * np + p;
+  double I = MODE == KM_RHS && !down ? A.inflow_bottom : 0.0, Q = 0.0;
+  for (int tt = 0; tt < t; ++tt) {
+    const double E = Etile[(size_t)tt * A.npair + u];
+    I = fma(E, I, Bmap[((size_t)(2 * g) * (T - 1) + tt) * 32 + lane]);
+    Q = fma(E, Q, Bmap[((size_t)(2 * g + 1) * (T - 1) + tt) * 32 + lane]);
+  }
+  const int64_t nray = A.nray, plane = (int64_t)Ns * nray;
+  const int64_t o1 = (int64_t)m * Nnu + p, o2 = (int64_t)m * Nnu + (Nnu - 1 - p);   // the pair's rays
+  const double* __restrict__ x = reinterpret_cast<const double*>(A.x);
+  double* __restrict__ y = reinterpret_cast<double*>(A.y);
+  const double* __restrict__ d = A.dinv;
+  const double* __restrict__ SI = reinterpret_cast<const double*>(A.S) + m;
+  const double* __restrict__ SQ = SI + (int64_t)Ns * A.Nmu;
+  if (t == 0 && active) {   // entry node: the inflow itself
+    const int64_t k = (int64_t)(down ? 0 : Ns - 1) * nray;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int64_t o = s * plane + k + (h ? o2 : o1);
+        if (h && !active2) continue;
+        if (MODE == KM_RHS) y[o] = s ? Q : I;
+        else if (MODE == KM_JACOBI) y[o] = x[o] * d[o];
+        else y[o] = x[o];
+      }
+    }
+  }
+  const int j0 = 1 + t * L, j1 = min(Ns, j0 + L);
+  if (j0 >= j1) return;
+  // downward: node j is height j, its step crosses interval j - 1; upward:
+  // height Ns-1-j, interval Ns-1-j
+  const int k0 = down ? j0 : Ns - 1 - j0;
+  const int64_t dk = down ? 1 : -1;
+  double spI = SI[(int64_t)(k0 - dk) * A.Nmu], spQ = SQ[(int64_t)(k0 - dk) * A.Nmu];
+  const int64_t cs = A.cstride;
+  constexpr int R = kPairRing;
+  double re[R], ra[R], rb[R], rI[R], rQ[R], rx[R][4], rd[R][4];
+  auto load = [&](int v, int j) {
+    if (j < j1) {
+      const int64_t k = k0 + dk * (j - j0);
+      const int64_t c = (down ? k - 1 : k) * cs + col;
+      re[v] = A.ce[c];
+      ra[v] = A.ca[c];
+      rb[v] = A.cb[c];
+      rI[v] = SI[k * A.Nmu];
+      rQ[v] = SQ[k * A.Nmu];
+      if (MODE != KM_RHS) {
+        const int64_t o = k * nray;
+        rx[v][0] = x[o + o1];
+        rx[v][1] = x[o + o2];
+        rx[v][2] = x[plane + o + o1];
+        rx[v][3] = x[plane + o + o2];
+        if (MODE == KM_JACOBI) {
+          rd[v][0] = d[o + o1];
+          rd[v][1] = d[o + o2];
+          rd[v][2] = d[plane + o + o1];
+          rd[v][3] = d[plane + o + o2];
+        }
+      }
+    }
+  };
+  auto step = [&](int v, int j) {
+    const double e = re[v], al = ra[v], be = rb[v], sI = rI[v], sQ = rQ[v];
+    const int64_t o = (k0 + dk * (j - j0)) * nray;
+    double vI, vQ;   // what is subtracted from z
+    if (MODE == KM_LOCAL_LAMBDA) {   // the step without its beta S_k term
+      vI = fma(e, I, al * spI);
+      vQ = fma(e, Q, al * spQ);
+      I = fma(be, sI, vI);
+      Q = fma(be, sQ, vQ);
+    } else {
+      I = fma(e, I, fma(al, spI, be * sI));
+      Q = fma(e, Q, fma(al, spQ, be * sQ));
+      vI = I;
+      vQ = Q;
+    }
+    if (active) {
+      if (MODE == KM_RHS) {
+        y[o + o1] = vI;
+        y[plane + o + o1] = vQ;
+      } else if (MODE == KM_JACOBI) {
+        y[o + o1] = fma(rx[v][0], rd[v][0], -vI);
+        y[plane + o + o1] = fma(rx[v][2], rd[v][2], -vQ);
+      } else {
+        y[o + o1] = rx[v][0] - vI;
+        y[plane + o + o1] = rx[v][2] - vQ;
+      }
+    }
+    if (active2) {
+      if (MODE == KM_RHS) {
+        y[o + o2] = vI;
+        y[plane + o + o2] = vQ;
+      } else if (MODE == KM_JACOBI) {
+        y[o + o2] = fma(rx[v][1], rd[v][1], -vI);
+        y[plane + o + o2] = fma(rx[v][3], rd[v][3], -vQ);
+      } else {
+        y[o + o2] = rx[v][1] - vI;
+        y[plane + o + o2] = rx[v][3] - vQ;
+      }
+    }
+    spI = sI;
+    spQ = sQ;
+  };
+#pragma unroll
+  for (int v = 0; v < R; ++v) load(v, j0 + v);
+  int jb = j0;
+  for (; jb + 2 * R <= j1; jb += R) {   // every step and refill in range
+#pragma unroll
+    for (int v = 0; v < R; ++v) {
+      step(v, jb + v);
+      load(v, jb + v + R);
+    }
+  }
+  for (; jb < j1; jb += R) {
+#pragma unroll
+    for (int v = 0; v < R; ++v) {
+      if (jb + v < j1) {
+        step(v, jb + v);
+        load(v, jb + v + R);
+      }
+    }
+  }
+}
+
 static int choose_tiles32(const Problem* P) {
   const int64_t want = (8LL * P->num_sms + P->ngroups - 1) / P->ngroups;
   int T = want < 1 ? 1 : (int)(want > kMaxTiles ? kMaxTiles : want);
@@ -617,6 +797,15 @@ rt_status setup_device_tables(Problem* P, cudaStream_t st) {
   P->nd = (int64_t)Nh * Nnu;
   const int ngd = (int)((P->nd + 31) / 32);
   P->ngroups = 2 * ngd;
+  // the step coefficients depend on |mu| only unless the scheme has a
+  // downwind term, and on the frequency through the profile: where that is
+  // symmetric on the grid, bit for bit, the pairs p, Nnu-1-p share them too
+  bool mirror = P->fs != RT_FS_DELO_PARABOLIC && P->N >= kPairMinN;
+  for (int p = 0; p < Nnu && mirror; ++p) mirror = P->phi_hat[p] == P->phi_hat[Nnu - 1 - p];
+  P->cshare = P->fs == RT_FS_DELO_PARABOLIC ? CS_RAY : mirror ? CS_PAIR : CS_MU;
+  P->cstride = mirror ? (int64_t)Nh * pair_count(Nnu) : P->cshare ? nray / 2 : nray;
+  P->npair = mirror ? 2 * P->cstride : 0;
+  P->ngroups64 = mirror ? 2 * (int)((P->cstride + 31) / 32) : P->ngroups;
   P->ntile64 = choose_tiles64(P);
 #ifdef RT_EXPERIMENT
   if (const char* t = std::getenv("RT_TILES64")) P->ntile64 = std::min(kMaxTiles64, std::max(1, std::atoi(t)));
@@ -655,10 +844,6 @@ rt_status setup_device_tables(Problem* P, cudaStream_t st) {
   RT_TRY(upload(P, &P->t201d, P->t201, st));
   RT_TRY(upload(P, &P->t202d, P->t202, st));
   RT_TRY(upload(P, &P->Bd, P->B, st));
-  // the step coefficients depend on |mu| only unless the scheme has a
-  // downwind term: one table column per (|mu|, p) then serves both directions
-  P->cshare = P->fs != RT_FS_DELO_PARABOLIC;
-  P->cstride = P->cshare ? nray / 2 : nray;
   const size_t nc = (size_t)(Ns - 1) * P->cstride;
   RT_TRY_CUDA(dev_alloc(P, (void**)&P->ce, nc * sizeof(double)));
   RT_TRY_CUDA(dev_alloc(P, (void**)&P->ca, nc * sizeof(double)));
@@ -673,18 +858,19 @@ rt_status setup_device_tables(Problem* P, cudaStream_t st) {
   RT_TRY_CUDA(cudaGetLastError());
   if (P->ntile64 > 1) {   // the FP64 formal solver's tile slopes and map buffer
     const int T = P->ntile64;
-    RT_TRY_CUDA(dev_alloc(P, (void**)&P->Etile, (size_t)(T - 1) * nray * sizeof(double)));
-    const size_t nb = (size_t)2 * P->ngroups * (T - 1) * 32;
+    const int64_t nlane = P->npair ? P->npair : nray;
+    RT_TRY_CUDA(dev_alloc(P, (void**)&P->Etile, (size_t)(T - 1) * nlane * sizeof(double)));
+    const size_t nb = (size_t)2 * P->ngroups64 * (T - 1) * 32;
     RT_TRY_CUDA(dev_alloc(P, (void**)&P->Bmap, nb * sizeof(double)));
     RT_TRY_CUDA(cudaMemsetAsync(P->Bmap, 0, nb * sizeof(double), st));   // lanes past a direction's last ray
     const int L = (Ns - 1 + T - 1) / T;
-    const int64_t nk = (int64_t)(T - 1) * (L + 2) * nray;
+    const int64_t nk = (int64_t)(T - 1) * (L + 2) * nlane;
     RT_TRY_CUDA(dev_alloc(P, (void**)&P->Kmap, (size_t)nk * sizeof(double)));
-    k_kmap<<<grid_for((int64_t)(T - 1) * nray, 256, 8 * P->num_sms), 256, 0, st>>>(
-        P->ce, P->ca, P->cb, P->cg, Ns, nray, P->nd, T, P->cstride, P->cshare, Nh, Nnu, P->Kmap);
+    k_kmap<<<grid_for((int64_t)(T - 1) * nlane, 256, 8 * P->num_sms), 256, 0, st>>>(
+        P->ce, P->ca, P->cb, P->cg, Ns, nlane, P->nd, T, P->cstride, P->cshare, Nh, Nnu, P->Kmap);
     RT_COUNT(1);
-    k_etile<<<grid_for((int64_t)(T - 1) * nray, 256, 8 * P->num_sms), 256, 0, st>>>(
-        P->ce, Ns, nray, P->nd, T, P->cstride, P->cshare, Nh, Nnu, P->Etile);
+    k_etile<<<grid_for((int64_t)(T - 1) * nlane, 256, 8 * P->num_sms), 256, 0, st>>>(
+        P->ce, Ns, nlane, P->nd, T, P->cstride, P->cshare, Nh, Nnu, P->Etile);
     RT_COUNT(1);
     RT_TRY_CUDA(cudaGetLastError());
   }
@@ -729,6 +915,7 @@ static FormalArgs formal_args(const Problem* P, const void* x, void* y, const vo
   A.cg = P->cg;
   A.cstride = P->cstride;
   A.cshare = P->cshare;
+  A.npair = 0;
   A.dtau32 = P->dtau32;
   A.r32 = P->r32;
   A.S = S;
@@ -747,15 +934,25 @@ static FormalArgs formal_args(const Problem* P, const void* x, void* y, const vo
 }
 
 template <int FS, int MODE>
-static void formal64_units(const Problem* P, const FormalArgs& A, cudaStream_t st) {
-  const int T = P->ntile64, groups = 2 * P->ngroups;
+static void formal64_units(const Problem* P, FormalArgs A, cudaStream_t st) {
+  const int T = P->ntile64;
+  const bool pair = FS != RT_FS_DELO_PARABOLIC && P->npair;
+  A.ngd = P->ngroups64 / 2;
+  A.npair = pair ? P->npair : 0;
   if (T > 1) {
-    launch_pdl_shape(k_fmapdot, dim3((unsigned)((P->nray + 31) / 32), (unsigned)(T - 1)), dim3(32, kMapSlices), st,
+    const int64_t nlane = pair ? P->npair : P->nray;
+    launch_pdl_shape(k_fmapdot, dim3((unsigned)((nlane + 31) / 32), (unsigned)(T - 1)), dim3(32, kMapSlices), st,
                      A, (const double*)P->Kmap, P->Bmap);
     RT_COUNT(1);
   }
-  launch_pdl_shape(k_fsweep<FS, MODE>, dim3(groups * T), dim3(32), st, A, (const double*)P->Bmap,
-                   (const double*)P->Etile);
+  if (pair) {
+    const int units = P->ngroups64 * T;
+    launch_pdl_shape(k_psweep<MODE>, dim3((units + kPairWarps - 1) / kPairWarps), dim3(32 * kPairWarps), st, A,
+                     (const double*)P->Bmap, (const double*)P->Etile, units);
+  } else {
+    launch_pdl_shape(k_fsweep<FS, MODE>, dim3(2 * P->ngroups64 * T), dim3(32), st, A, (const double*)P->Bmap,
+                     (const double*)P->Etile);
+  }
   RT_COUNT(1);
 }
 
@@ -803,23 +1000,25 @@ rt_status op_apply64(Problem* P, const double* x, double* y, int mode, cudaStrea
   }
   const double xiW2 = P->xi * P->W2;
   const int Ns = P->Ns, Nmu = P->Nmu;
+  const bool pair = P->npair > 0;
   if (nin) {   // GMRES: x = u / ||u|| formed by the quadrature kernel
     double* xw = const_cast<double*>(x);
     switch (mode) {
       case AM_PLAIN:
-        RT_TRY_CUDA(launch_pdl(k_moments64_norm<KM_PLAIN, false>, Ns + 1, kMom64Threads, st,
+        RT_TRY_CUDA(launch_pdl(pair ? k_moments64_norm<KM_PLAIN, false, true> : k_moments64_norm<KM_PLAIN, false, false>, Ns + 1, kMom64Threads, st,
             xw, nullptr, P->wray, P->t201d, P->t202d, nullptr, Ns, Nmu, P->nray, P->xi, xiW2, P->S, *nin));
         break;
       case AM_JACOBI:
         if (P->wjac)
-          RT_TRY_CUDA(launch_pdl(k_moments64_norm<KM_JACOBI, true>, Ns + 1, kMom64Threads, st,
+          RT_TRY_CUDA(launch_pdl(k_moments64_norm<KM_JACOBI, true, false>, Ns + 1, kMom64Threads, st,
               xw, nullptr, P->wjac, P->t201d, P->t202d, nullptr, Ns, Nmu, P->nray, P->xi, xiW2, P->S, *nin));
         else
-          RT_TRY_CUDA(launch_pdl(k_moments64_norm<KM_JACOBI, false>, Ns + 1, kMom64Threads, st,
+          RT_TRY_CUDA(launch_pdl(k_moments64_norm<KM_JACOBI, false, false>, Ns + 1, kMom64Threads, st,
               xw, P->dinv, P->wray, P->t201d, P->t202d, nullptr, Ns, Nmu, P->nray, P->xi, xiW2, P->S, *nin));
         break;
       case AM_LOCAL_LAMBDA:
-        RT_TRY_CUDA(launch_pdl(k_moments64_norm<KM_LOCAL_LAMBDA, false>, Ns + 1, kMom64Threads, st,
+        RT_TRY_CUDA(launch_pdl(pair ? k_moments64_norm<KM_LOCAL_LAMBDA, false, true>
+                                    : k_moments64_norm<KM_LOCAL_LAMBDA, false, false>, Ns + 1, kMom64Threads, st,
             xw, nullptr, P->wray, P->t201d, P->t202d, P->Minv, Ns, Nmu, P->nray, P->xi, xiW2, P->S, *nin));
         break;
       default:
@@ -837,7 +1036,7 @@ rt_status op_apply64(Problem* P, const double* x, double* y, int mode, cudaStrea
   }
   switch (mode) {
     case AM_PLAIN:
-      k_moments64<KM_PLAIN><<<Ns, kMom64Threads, 0, st>>>(x, nullptr, P->wray, P->t201d, P->t202d, nullptr, Ns, Nmu,
+      (pair ? k_moments64<KM_PLAIN, false, true> : k_moments64<KM_PLAIN>)<<<Ns, kMom64Threads, 0, st>>>(x, nullptr, P->wray, P->t201d, P->t202d, nullptr, Ns, Nmu,
                                                           P->nray, P->xi, xiW2, P->S, kstop, step); RT_COUNT(1);
       launch_formal64<KM_PLAIN>(P, x, y, P->S, st, kstop, step);
       break;
@@ -852,7 +1051,7 @@ rt_status op_apply64(Problem* P, const double* x, double* y, int mode, cudaStrea
       launch_formal64<KM_JACOBI>(P, x, y, P->S, st, kstop, step);
       break;
     case AM_LOCAL_LAMBDA:
-      k_moments64<KM_LOCAL_LAMBDA><<<Ns, kMom64Threads, 0, st>>>(x, nullptr, P->wray, P->t201d, P->t202d, P->Minv,
+      (pair ? k_moments64<KM_LOCAL_LAMBDA, false, true> : k_moments64<KM_LOCAL_LAMBDA>)<<<Ns, kMom64Threads, 0, st>>>(x, nullptr, P->wray, P->t201d, P->t202d, P->Minv,
                                                                  Ns, Nmu, P->nray, P->xi, xiW2, P->S, kstop, step);
       RT_COUNT(1);
       launch_formal64<KM_LOCAL_LAMBDA>(P, x, y, P->S, st, kstop, step);
@@ -971,7 +1170,7 @@ rt_status op_x0_paper(Problem* P, double* x, cudaStream_t st) {
 rt_status op_precond_ll(Problem* P, const double* v, double* z, cudaStream_t st, const int* kstop, int step) {
   if (P->form == RT_FORM_SIGMA) return op_precond_sigma(P, v, z, st, kstop, step);
   const double xiW2 = P->xi * P->W2;
-  k_moments64<KM_LOCAL_LAMBDA><<<P->Ns, kMom64Threads, 0, st>>>(v, nullptr, P->wray, P->t201d, P->t202d, P->Minv,
+  (P->npair ? k_moments64<KM_LOCAL_LAMBDA, false, true> : k_moments64<KM_LOCAL_LAMBDA>)<<<P->Ns, kMom64Threads, 0, st>>>(v, nullptr, P->wray, P->t201d, P->t202d, P->Minv,
                                                                 P->Ns, P->Nmu, P->nray, P->xi, xiW2, P->S2, kstop,
                                                                 step); RT_COUNT(1);
   k_add_local<<<grid_for(P->N, 256, 8 * P->num_sms), 256, 0, st>>>(v, P->cb, P->ce, P->cg, P->S2, P->Ns, P->Nmu,
