@@ -59,8 +59,8 @@ struct InstDev {
   int64_t cstride;   // columns of the FP64 tables (coef_col)
   int cshare;
   double xi, xiW2, inflow_bottom;
-  const double *ce, *ca, *cb, *wnu, *wmu, *wray, *t201, *t202, *Minv;
-  const float *dtau32, *r32, *wnu32, *wmu32, *t201f, *t202f;
+  const double *ce, *ca, *cb, *wray, *t201, *t202, *Minv;
+  const float *dtau32, *r32, *wray32, *t201f, *t202f;
   double *S, *S2;
   float* S32;
   double *V, *x, *b, *r, *w, *t, *tmp, *dinv, *part;
@@ -153,16 +153,14 @@ __global__ void __launch_bounds__(kMomThreads) kb_moments(const InstDev* __restr
       moments_flat64<MODE, false, NORM>(x, I.dinv, I.wray, I.t201, I.t202, I.Minv, I.Ns, I.Nmu, I.nray, I.xi,
                                         I.xiW2, useS2 ? I.S2 : I.S, it.y, inv, xo);
     } else {
-      moments_height<double, float, MODE, NORM>(x, I.dinv, I.wnu32, I.wmu32, I.t201f, I.t202f, I.Minv, I.Ns, I.Nmu,
-                                                I.Nnu, (float)I.xi, (float)I.xiW2, I.S32, it.y, inv, xo);
+      moments_flat32<double, MODE, NORM>(x, I.dinv, I.wray32, I.t201f, I.t202f, I.Minv, I.Ns, I.Nmu, I.nray,
+                                         (float)I.xi, (float)I.xiW2, I.S32, it.y, inv, xo);
     }
     __syncthreads();
   }
 }
 
-template <typename TC, int FS, int MODE, int NS>
-__device__ __forceinline__ void formal_item(const InstDev& I, int g, int s0, int src, int dst) {
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ FormalArgs item_args(const InstDev& I, int src, int dst, const void* S) {
   FormalArgs A;
   A.x = vec(I, src);
   A.dinv = I.dinv;
@@ -172,9 +170,10 @@ __device__ __forceinline__ void formal_item(const InstDev& I, int g, int s0, int
   A.cg = nullptr;
   A.cstride = I.cstride;
   A.cshare = I.cshare;
+  A.npair = 0;
   A.dtau32 = I.dtau32;
   A.r32 = I.r32;
-  A.S = sizeof(TC) == 8 ? (const void*)I.S : (const void*)I.S32;
+  A.S = S;
   A.y = vec(I, dst);
   A.Ns = I.Ns;
   A.Nmu = I.Nmu;
@@ -186,6 +185,13 @@ __device__ __forceinline__ void formal_item(const InstDev& I, int g, int s0, int
   A.inflow_bottom = I.inflow_bottom;
   A.kstop = nullptr;
   A.step = 0;
+  return A;
+}
+
+template <int FS, int MODE>
+__device__ __forceinline__ void formal_item(const InstDev& I, int g, int s0, int src, int dst) {
+  const int lane = threadIdx.x & 31;
+  const FormalArgs A = item_args(I, src, dst, I.S);
   const bool down = g < I.ngd;
   const int64_t base = down ? (int64_t)g * 32 : I.nd + (int64_t)(g - I.ngd) * 32;
   const int64_t end = down ? I.nd : I.nray;
@@ -193,42 +199,97 @@ __device__ __forceinline__ void formal_item(const InstDev& I, int g, int s0, int
   const int64_t r = active ? base + lane : end - 1;
   const int m = (int)(r / I.Nnu);
   const int Ns = I.Ns;
-  TC Iv[NS];
-#pragma unroll
-  for (int q = 0; q < NS; ++q) Iv[q] = 0;
+  double Iv[1] = {0.0};
   if (active) {
     const int k0 = down ? 0 : Ns - 1;
     const double* x = reinterpret_cast<const double*>(A.x);
     double* y = reinterpret_cast<double*>(A.y);
+    const int64_t o = (int64_t)s0 * Ns * I.nray + (int64_t)k0 * I.nray + r;
+    if (MODE == KM_JACOBI) y[o] = x[o] * I.dinv[o];
+    else y[o] = x[o];
+  }
+  double E = 1;
+  sweep<double, double, FS, MODE, 1, 1, kRing>(A, s0, down, r, m, active, 1, Ns, Iv, E);
+}
+
+// FP64: items (slot, group, Stokes), one warp each
+template <int MODE>
+__global__ void __launch_bounds__(32 * kFormalWarps) kb_formal(const InstDev* __restrict__ insts,
+                                                               const int4* __restrict__ wl, const Counts* cnt,
+                                                               int src, int dst, int step) {
+  const int n = cnt->ng64;
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  for (int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < n; w += warps) {
+    const int4 it = wl[w];
+    const InstDev& I = insts[it.x];
+    if (step_gated(I, step)) continue;
+    formal_item<0, MODE>(I, it.y, it.z, src, dst);
+  }
+}
+
+// FP32: items (slot, group), both Stokes parameters per lane.  A CTA takes a
+// ray group and splits its depth into up to kTiles32 tiles, one warp each: the
+// tile maps (phase A), their chain (phase B), the sweep with the output (phase
+// C), as k_formal does for a single problem.  With one warp marching all
+// heights of a group, 32 atmospheres put 7 warps on an SM, each waiting on its
+// own recurrence: 276 us a launch.
+constexpr int kTiles32 = 8;
+constexpr int kRingB = 8;   // prefetch depth (steps)
+
+template <int FS, int MODE>
+__device__ __forceinline__ void formal_item32(const InstDev& I, int g, int src, int dst,
+                                              float (*sh)[kTiles32][32]) {
+  const int lane = threadIdx.x & 31, t = threadIdx.x >> 5;
+  const FormalArgs A = item_args(I, src, dst, I.S32);
+  const bool down = g < I.ngd;
+  const int64_t base = down ? (int64_t)g * 32 : I.nd + (int64_t)(g - I.ngd) * 32;
+  const int64_t end = down ? I.nd : I.nray;
+  const bool active = base + lane < end;
+  const int64_t r = active ? base + lane : end - 1;
+  const int m = (int)(r / I.Nnu);
+  const int Ns = I.Ns;
+  const int T = max(1, min(kTiles32, (Ns - 1) / kRingB)), L = (Ns - 1 + T - 1) / T;
+  const int j0 = 1 + t * L, j1 = t < T ? min(Ns, j0 + L) : j0;
+  float Iv[2] = {0.f, 0.f};
+  if (t < T - 1 && j0 < j1) {
+    float E = 1.f, B[2] = {0.f, 0.f};
+    sweep<float, double, FS, MODE, 0, 2, kRingB>(A, 0, down, r, m, active, j0, j1, B, E);
+    sh[0][t][lane] = E;
+    sh[1][t][lane] = B[0];
+    sh[2][t][lane] = B[1];
+  }
+  __syncthreads();
+  for (int u = 0; u < t && t < T && 1 + u * L < Ns; ++u) {   // inflow of the tile: zero at the boundary
+    Iv[0] = fmaf(sh[0][u][lane], Iv[0], sh[1][u][lane]);
+    Iv[1] = fmaf(sh[0][u][lane], Iv[1], sh[2][u][lane]);
+  }
+  if (t == 0 && active) {
+    const int k0 = down ? 0 : Ns - 1;
+    const double* x = reinterpret_cast<const double*>(A.x);
+    double* y = reinterpret_cast<double*>(A.y);
 #pragma unroll
-    for (int q = 0; q < NS; ++q) {
-      const int64_t o = (int64_t)(s0 + q) * Ns * I.nray + (int64_t)k0 * I.nray + r;
+    for (int q = 0; q < 2; ++q) {
+      const int64_t o = (int64_t)q * Ns * I.nray + (int64_t)k0 * I.nray + r;
       if (MODE == KM_JACOBI) y[o] = x[o] * I.dinv[o];
       else y[o] = x[o];
     }
   }
-  TC E = 1;
-  if (sizeof(TC) == 8)
-    sweep<TC, double, FS, MODE, 1, NS, kRing>(A, s0, down, r, m, active, 1, Ns, Iv, E);
-  else
-    sweep<TC, double, FS, MODE, 1, NS, kRing32>(A, s0, down, r, m, active, 1, Ns, Iv, E);
+  float E = 1.f;
+  if (j0 < j1) sweep<float, double, FS, MODE, 1, 2, kRingB>(A, 0, down, r, m, active, j0, j1, Iv, E);
+  __syncthreads();   // the maps are read before the next item writes its own
 }
 
-// FP64: items (slot, group, Stokes); FP32: items (slot, group) with both
-// Stokes parameters per lane, one launch per formal solver (FS)
-template <typename TC, int FS, int MODE>
-__global__ void __launch_bounds__(32 * kFormalWarps) kb_formal(const InstDev* __restrict__ insts,
-                                                               const int4* __restrict__ wl, const Counts* cnt,
-                                                               int src, int dst, int step) {
-  const int n = sizeof(TC) == 8 ? cnt->ng64 : cnt->ng32[FS];
-  const int off = sizeof(TC) == 8 ? 0 : cnt->off32[FS];
-  const int warps = gridDim.x * (blockDim.x >> 5);
-  for (int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < n; w += warps) {
+template <int FS, int MODE>
+__global__ void __launch_bounds__(32 * kTiles32) kb_formal32(const InstDev* __restrict__ insts,
+                                                             const int4* __restrict__ wl, const Counts* cnt, int src,
+                                                             int dst, int step) {
+  __shared__ float sh[3][kTiles32][32];   // per tile: E, B of I, B of Q
+  const int n = cnt->ng32[FS], off = cnt->off32[FS];
+  for (int w = blockIdx.x; w < n; w += gridDim.x) {
     const int4 it = wl[off + w];
     const InstDev& I = insts[it.x];
     if (step_gated(I, step)) continue;
-    if (sizeof(TC) == 8) formal_item<TC, 0, MODE, 1>(I, it.y, it.z, src, dst);
-    else formal_item<TC, FS, MODE, 2>(I, it.y, 0, src, dst);
+    formal_item32<FS, MODE>(I, it.y, src, dst, sh);
   }
 }
 
@@ -652,12 +713,9 @@ static_assert(kChunk % kPassTile == 0, "a chunk starts on a tile");
 
 template <int MODE>
 void formal32(Server* S, cudaStream_t st, int src, int dst, int step) {
-  kb_formal<float, RT_FS_DELO_LINEAR, MODE><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(S->d_insts, S->d_wl_g32,
-                                                                                     S->d_counts, src, dst, step); RT_COUNT(1);
-  kb_formal<float, RT_FS_IMPLICIT_EULER, MODE><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(S->d_insts, S->d_wl_g32,
-                                                                                        S->d_counts, src, dst, step); RT_COUNT(1);
-  kb_formal<float, RT_FS_TRAPEZOIDAL, MODE><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(S->d_insts, S->d_wl_g32,
-                                                                                     S->d_counts, src, dst, step); RT_COUNT(1);
+  kb_formal32<RT_FS_DELO_LINEAR, MODE><<<S->grid_g, 32 * kTiles32, 0, st>>>(S->d_insts, S->d_wl_g32, S->d_counts, src, dst, step); RT_COUNT(1);
+  kb_formal32<RT_FS_IMPLICIT_EULER, MODE><<<S->grid_g, 32 * kTiles32, 0, st>>>(S->d_insts, S->d_wl_g32, S->d_counts, src, dst, step); RT_COUNT(1);
+  kb_formal32<RT_FS_TRAPEZOIDAL, MODE><<<S->grid_g, 32 * kTiles32, 0, st>>>(S->d_insts, S->d_wl_g32, S->d_counts, src, dst, step); RT_COUNT(1);
 }
 
 template <bool NORM>
@@ -668,16 +726,16 @@ void enqueue_apply_t(Server* S, cudaStream_t st, int src, int dst, int md, bool 
     switch (md) {
       case KM_JACOBI:
         kb_moments<double, KM_JACOBI, NORM><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, src, step, 0); RT_COUNT(1);
-        kb_formal<double, 0, KM_JACOBI><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(I, S->d_wl_g64, C, src, dst, step); RT_COUNT(1);
+        kb_formal<KM_JACOBI><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(I, S->d_wl_g64, C, src, dst, step); RT_COUNT(1);
         break;
       case KM_LOCAL_LAMBDA:
         kb_moments<double, KM_LOCAL_LAMBDA, NORM><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, src, step, 0); RT_COUNT(1);
-        kb_formal<double, 0, KM_LOCAL_LAMBDA><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(I, S->d_wl_g64, C, src, dst,
+        kb_formal<KM_LOCAL_LAMBDA><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(I, S->d_wl_g64, C, src, dst,
                                                                                      step); RT_COUNT(1);
         break;
       default:
         kb_moments<double, KM_PLAIN, NORM><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, src, step, 0); RT_COUNT(1);
-        kb_formal<double, 0, KM_PLAIN><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(I, S->d_wl_g64, C, src, dst, step); RT_COUNT(1);
+        kb_formal<KM_PLAIN><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(I, S->d_wl_g64, C, src, dst, step); RT_COUNT(1);
     }
   } else {
     switch (md) {
@@ -970,16 +1028,13 @@ rt_status make_instance(Server* S, Request* rq, Instance* in, int slot) {
   D.cb = P.cb;
   D.cstride = P.cstride;
   D.cshare = P.cshare;
-  D.wnu = P.wI2;
-  D.wmu = P.wQ2;
   D.wray = P.wray;
   D.t201 = P.t201d;
   D.t202 = P.t202d;
   D.Minv = P.Minv;
   D.dtau32 = P.dtau32;
   D.r32 = P.r32;
-  D.wnu32 = P.wI2f;
-  D.wmu32 = P.wQ2f;
+  D.wray32 = P.wray32;
   D.t201f = P.t201f;
   D.t202f = P.t202f;
   D.S = P.S;

@@ -126,7 +126,12 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cud
 }
 
 // sum of G partials in a fixed order (lane-strided, then a fixed shuffle
-// tree); every lane of the calling warp gets the result
+// tree); every lane of the calling warp gets the result.  TREE: a lane's
+// values are added as trees of 8 (the additions of a chain wait on one
+// another; GMRES's passes do this between every two kernels), else in the
+// order of their index (BiCGSTAB and CGS, whose iterates amplify a change of
+// rounding).
+template <bool TREE = true>
 __device__ __forceinline__ double partials_sum_warp(const double* __restrict__ part, int G) {
   const int lane = threadIdx.x & 31;
   constexpr int U = 8;   // loads in flight per lane
@@ -134,11 +139,18 @@ __device__ __forceinline__ double partials_sum_warp(const double* __restrict__ p
   for (int i0 = lane; i0 < G; i0 += 32 * U) {
     double v[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (i0 + 32 * u < G) v[u] = part[i0 + 32 * u];
+    for (int u = 0; u < U; ++u) v[u] = i0 + 32 * u < G ? part[i0 + 32 * u] : 0.0;
+    if (TREE) {
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (i0 + 32 * u < G) s += v[u];
+      for (int o = U / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < o; ++u) v[u] += v[u + o];
+      s += v[0];
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + 32 * u < G) s += v[u];
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -331,8 +343,6 @@ struct Problem {
   double* Kmap = nullptr;  // [ntile64-1][L+2][nray or npair] weights of the map offsets in the node source values
   double* wray = nullptr;  // [3][nray] hat-w_m * hat-w_p, the same times T201_m, times T202_m
   double* wjac = nullptr;  // [3][Ns][nray] wray times the Jacobi inverse diagonal (I, I, Q), once a solver set it
-  double* wI2 = nullptr;   // [Nnu] spectral weights hat-w_p
-  double* wQ2 = nullptr;   // [Nmu] angular weights hat-w_m = w_m / 2
   double* t201d = nullptr; // [Nmu]
   double* t202d = nullptr; // [Nmu]
   double* Bd = nullptr;    // [Ns]
@@ -344,9 +354,7 @@ struct Problem {
   // FP32 device tables
   float* dtau32 = nullptr;  // [Ns-1] tau_{k+1} - tau_k
   float* r32 = nullptr;     // [nray] phi_hat_p / |mu_m|
-  float* wray32 = nullptr;
-  float* wI2f = nullptr;
-  float* wQ2f = nullptr;
+  float* wray32 = nullptr;  // [3][nray] wray in FP32
   float* t201f = nullptr;
   float* t202f = nullptr;
   float* S32 = nullptr;     // [2][Ns][Nmu]

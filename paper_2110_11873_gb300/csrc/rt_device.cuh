@@ -8,7 +8,7 @@
 namespace rt {
 namespace {
 
-constexpr int kMomThreads = 256;
+constexpr int kMomThreads = 256;      // threads of the FP32 quadrature (and of the batch's)
 constexpr int kMaxTiles = 8;     // FP32 kernel: up to 256 threads per CTA (255 registers a lane)
 constexpr int kMaxTilesRay = 16; // FP64 formal solver on rays: depth tiles per ray group (one warp each)
 constexpr int kMaxTiles64 = 32;  // FP64 formal solver on pairs of rays: the same
@@ -22,6 +22,46 @@ __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// FP64 <-> FP32 on the integer pipe: the conversion instructions run on the
+// FP64 pipe (1.9 a clock and SM, measured), which then bounds every kernel
+// that computes in FP32 on FP64 vectors.  The same results as the conversions
+// (round to nearest even, subnormal numbers kept, NaN stays NaN).
+__device__ __forceinline__ float to_f32(double x) {
+  const uint32_t hi = __double2hiint(x), lo = __double2loint(x), ab = hi & 0x7fffffffu, sg = hi & 0x80000000u;
+  if (ab - 0x38100000u < 0x47f00000u - 0x38100000u) {   // a normal number below 2^128
+    const uint32_t t = __funnelshift_l(lo, ab - 0x38000000u, 3), rem = lo << 3;
+    return __uint_as_float((t + (uint32_t)((rem | (t & 1u)) > 0x80000000u)) | sg);
+  }
+  if (ab >= 0x47f00000u) return __uint_as_float((ab > 0x7ff00000u || (ab == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u) | sg);
+  const int s = 926 - (int)(ab >> 20);   // a multiple of 2^-149: the mantissa over 2^s
+  if (s > 54) return __uint_as_float(sg);
+  const uint64_t m = ((uint64_t)((ab & 0xfffffu) | 0x100000u) << 32) | lo;
+  const uint64_t q = m >> s, rem = m << (64 - s);
+  return __uint_as_float(((uint32_t)q + (uint32_t)((rem | (q & 1u)) > 0x8000000000000000ull)) | sg);
+}
+__device__ __forceinline__ double to_f64(float x) {
+  uint32_t u = __float_as_uint(x), ab = u & 0x7fffffffu;
+  const uint32_t sg = u & 0x80000000u;
+  uint32_t bias = 0x38000000u;
+  if (ab - 0x00800000u >= 0x7f800000u - 0x00800000u) {
+    if (ab == 0) return __hiloint2double((int)sg, 0);
+    if (ab >= 0x7f800000u) {   // an infinity or a NaN
+      bias = 0x70000000u;
+    } else {                   // subnormal: shift the leading bit to its place
+      const int z = __clz(ab) - 8;
+      ab = (ab << z) & 0x7fffffu;
+      bias = 0x38100000u - ((uint32_t)z << 20);
+    }
+  }
+  return __hiloint2double((int)(((ab >> 3) + bias) | sg), (int)(ab << 29));
+}
+template <typename To, typename From>
+__device__ __forceinline__ To vcast(From x) {
+  if constexpr (sizeof(To) == 4 && sizeof(From) == 8) return to_f32(x);
+  else if constexpr (sizeof(To) == 8 && sizeof(From) == 4) return to_f64(x);
+  else return x;
 }
 
 // beta* (coefficient of S_k in I_k) of ray r = m*Nnu + p at height k: the
@@ -46,82 +86,60 @@ __device__ __forceinline__ double beta_star(const double* __restrict__ cb, int k
 }
 
 // ----------------------------------------------------------------- K1: T∘J
-// One block per height; warp w sums the direction rows m = w, w+8, ...:
-// a_m = sum_p w_p z_I(k,m,p), b_m = sum_p w_p z_Q(k,m,p) (one multiply-add
-// per element), then J00 += w_m a_m and J20 += w_m (T201_m a_m + T202_m b_m).
-// Every lane issues the loads of a whole row before it adds.  MODE:
-// KM_PLAIN z = x; KM_JACOBI z = x * dinv; KM_LOCAL_LAMBDA z = x and
-// sigma_k <- M_k^{-1} sigma_k.  TI: input vector type, TC: arithmetic type.
-constexpr int kRowChunk = 8;   // loads per lane in flight per Stokes parameter
+// MODE: KM_PLAIN z = x; KM_JACOBI z = x * dinv; KM_LOCAL_LAMBDA z = x and
+// sigma_k <- M_k^{-1} sigma_k.
 
-// moments of height k by the whole block (all threads must call it).
+// FP32 quadrature of height k by the whole block (kMomThreads threads) as
+// flat dot products over its rays, with the per-ray weights w0 = hat-w_m
+// hat-w_p, w1 = w0 T201_m, w2 = w0 T202_m (wray, [3][nray]):
+//     J00 = sum_r w0 I_r,   J20 = sum_r (w1 I_r + w2 Q_r).
 // NORM: the input is x * inv, written to xout in the input's precision as
-// each element is read (the GMRES normalisation of the batched solver)
-template <typename TI, typename TC, int MODE, bool NORM = false>
-__device__ __forceinline__ void moments_height(
-    const TI* __restrict__ x, const double* __restrict__ dinv, const TC* __restrict__ wnu,
-    const TC* __restrict__ wmu, const TC* __restrict__ t201, const TC* __restrict__ t202,
-    const double* __restrict__ Minv, int Ns, int Nmu, int Nnu, TC xi, TC xiW2, TC* __restrict__ S, int k,
-    double inv = 1.0, TI* __restrict__ xout = nullptr) {
-  const int64_t nray = (int64_t)Nmu * Nnu;
+// each element is read (the GMRES normalisation of the batched solver).  A
+// warp per direction row, as before, left lanes idle on short rows and half
+// of its loads predicated off (32 uneven atmospheres: 139 us a launch).
+template <typename TI, int MODE, bool NORM = false>
+__device__ __forceinline__ void moments_flat32(const TI* __restrict__ x, const double* __restrict__ dinv,
+                                               const float* __restrict__ wray, const float* __restrict__ t201,
+                                               const float* __restrict__ t202, const double* __restrict__ Minv,
+                                               int Ns, int Nmu, int64_t nray, float xi, float xiW2,
+                                               float* __restrict__ S, int k, double inv = 1.0,
+                                               TI* __restrict__ xout = nullptr) {
+  constexpr int nw = kMomThreads / 32;
   const int64_t oI = (int64_t)k * nray, oQ = ((int64_t)Ns + k) * nray;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int nw = kMomThreads / 32;
-  TC j00 = 0, j20 = 0;
-  for (int m = warp; m < Nmu; m += nw) {
-    const int64_t row = (int64_t)m * Nnu;
-    TC aI = 0, aQ = 0;
-    for (int p0 = 0; p0 < Nnu; p0 += 32 * kRowChunk) {
-      TC vI[kRowChunk], vQ[kRowChunk], wv[kRowChunk];
-#pragma unroll
-      for (int c = 0; c < kRowChunk; ++c) {
-        const int p = p0 + c * 32 + lane;
-        const bool ok = p < Nnu;
-        const int64_t q = row + (ok ? p : 0);
-        if (NORM) {
-          TI a = 0, b = 0;
-          if (ok) {
-            a = (TI)(x[oI + q] * inv);
-            b = (TI)(x[oQ + q] * inv);
-            xout[oI + q] = a;
-            xout[oQ + q] = b;
-          }
-          vI[c] = (TC)a;
-          vQ[c] = (TC)b;
-        } else {
-          vI[c] = ok ? (TC)x[oI + q] : (TC)0;
-          vQ[c] = ok ? (TC)x[oQ + q] : (TC)0;
-        }
-        wv[c] = ok ? wnu[p] : (TC)0;
-        if (MODE == KM_JACOBI && ok) {
-          vI[c] *= (TC)dinv[oI + q];
-          vQ[c] *= (TC)dinv[oQ + q];
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < kRowChunk; ++c) {
-        aI = fma(wv[c], vI[c], aI);
-        aQ = fma(wv[c], vQ[c], aQ);
-      }
+  float a0 = 0.f, a1 = 0.f;
+#pragma unroll 4
+  for (int64_t r = threadIdx.x; r < nray; r += kMomThreads) {
+    TI xI = x[oI + r], xQ = x[oQ + r];
+    if (NORM) {
+      xI = (TI)(xI * inv);
+      xQ = (TI)(xQ * inv);
+      xout[oI + r] = xI;
+      xout[oQ + r] = xQ;
     }
-    aI = warp_sum(aI);
-    aQ = warp_sum(aQ);
-    const TC wm = wmu[m];
-    j00 = fma(wm, aI, j00);
-    j20 = fma(wm, fma(t201[m], aI, t202[m] * aQ), j20);
+    float vI = vcast<float>(xI), vQ = vcast<float>(xQ);
+    if (MODE == KM_JACOBI) {
+      vI *= to_f32(dinv[oI + r]);
+      vQ *= to_f32(dinv[oQ + r]);
+    }
+    a0 = fmaf(wray[r], vI, a0);
+    a1 = fmaf(wray[nray + r], vI, a1);
+    a1 = fmaf(wray[2 * nray + r], vQ, a1);
   }
-  __shared__ TC red[2][nw];
-  __shared__ TC sig[2];
-  if (lane == 0) { red[0][warp] = j00; red[1][warp] = j20; }
+  a0 = warp_sum(a0);
+  a1 = warp_sum(a1);
+  __shared__ float red[2][nw];
+  __shared__ float sig[2];
+  if (lane == 0) { red[0][warp] = a0; red[1][warp] = a1; }
   __syncthreads();
   if (threadIdx.x == 0) {
-    TC a = 0, b = 0;
+    float a = 0.f, b = 0.f;
     for (int w = 0; w < nw; ++w) { a += red[0][w]; b += red[1][w]; }
-    TC s0 = xi * a, s2 = xiW2 * b;
+    float s0 = xi * a, s2 = xiW2 * b;
     if (MODE == KM_LOCAL_LAMBDA) {
       const double* Mi = Minv + 4 * k;
-      const TC u0 = (TC)Mi[0] * s0 + (TC)Mi[1] * s2;
-      const TC u2 = (TC)Mi[2] * s0 + (TC)Mi[3] * s2;
+      const float u0 = (float)Mi[0] * s0 + (float)Mi[1] * s2;
+      const float u2 = (float)Mi[2] * s0 + (float)Mi[3] * s2;
       s0 = u0;
       s2 = u2;
     }
@@ -181,7 +199,7 @@ __device__ __forceinline__ void moments_finish64(double a0, double a1, const dou
 // threads stride over r): with the per-ray weights w0 = hat-w_m hat-w_p,
 // w1 = w0 T201_m, w2 = w0 T202_m (wray, [3][nray]),
 //     J00 = sum_r w0 I_r,   J20 = sum_r (w1 I_r + w2 Q_r),
-// then S as in moments_height.  Every FP64 operation is useful work: no
+// then S of every direction.  Every FP64 operation is useful work: no
 // lane idles on a short row and there is one reduction per height (the FP64
 // pipe bounds this kernel).  Any block size that is a multiple of 32.
 // WJ (Jacobi mode): wray holds per-element weights [3][Ns][nray], the
@@ -381,8 +399,8 @@ __device__ __forceinline__ void sweep(const FormalArgs& A, int s0, bool down, in
         rsv[u][q] = Sm[q * sstride + (int64_t)k * A.Nmu];
         if (PHASE == 1 && MODE != KM_RHS) {
           const int64_t o = q * plane + (int64_t)k * nray + r;
-          rx[u][q] = (TC)x[o];
-          if (MODE == KM_JACOBI) rd[u][q] = (TC)dinv[o];
+          rx[u][q] = vcast<TC>(x[o]);
+          if (MODE == KM_JACOBI) rd[u][q] = vcast<TC>(dinv[o]);
         }
       }
     } else if (PARA && j == j1 && j < Ns) {
@@ -419,19 +437,19 @@ __device__ __forceinline__ void sweep(const FormalArgs& A, int s0, bool down, in
         // part of I_prev): x - (e (I_prev - gamma_prev S_k) + alpha S_prev + gamma S_next)
         if (PARA) {
           const TC t = fma(e, fma(-gp, sk, I[q]), fma(al, sp[q], rg[u] * rsv[(u + 1) % RING][q]));
-          if (active) y[q * plane + o] = (TV)(rx[u][q] - t);
+          if (active) y[q * plane + o] = vcast<TV>(rx[u][q] - t);
           I[q] = fma(fma(e, gp, be), sk, t);
         } else {
           const TC t = fma(e, I[q], al * sp[q]);
-          if (active) y[q * plane + o] = (TV)(rx[u][q] - t);
+          if (active) y[q * plane + o] = vcast<TV>(rx[u][q] - t);
           I[q] = fma(be, sk, t);
         }
       } else {
         I[q] = fma(e, I[q], fma(al, sp[q], cur));
         if (active) {
-          if (MODE == KM_RHS) y[q * plane + o] = (TV)I[q];
-          else if (MODE == KM_JACOBI) y[q * plane + o] = (TV)(rx[u][q] * rd[u][q] - I[q]);
-          else y[q * plane + o] = (TV)(rx[u][q] - I[q]);
+          if (MODE == KM_RHS) y[q * plane + o] = vcast<TV>(I[q]);
+          else if (MODE == KM_JACOBI) y[q * plane + o] = vcast<TV>(rx[u][q] * rd[u][q] - I[q]);
+          else y[q * plane + o] = vcast<TV>(rx[u][q] - I[q]);
         }
       }
       sp[q] = sk;

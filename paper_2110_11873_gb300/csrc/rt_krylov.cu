@@ -64,7 +64,7 @@ __device__ __forceinline__ double block_sum(double v) {
 // sum of G partials in a fixed order (lane-strided, then a fixed shuffle tree);
 // every thread of the calling warp gets the result
 __device__ __forceinline__ double sum_partials_warp(const double* __restrict__ part, int G) {
-  return partials_sum_warp(part, G);
+  return partials_sum_warp<false>(part, G);
 }
 
 // broadcast of sum_partials to the whole block

@@ -223,14 +223,14 @@ __global__ void k_add_local(const double* __restrict__ v, const double* __restri
 }
 
 
-template <typename TI, typename TC, int MODE>
+template <typename TI, int MODE>
 __global__ void __launch_bounds__(kMomThreads) k_moments(
-    const TI* __restrict__ x, const double* __restrict__ dinv, const TC* __restrict__ wnu,
-    const TC* __restrict__ wmu, const TC* __restrict__ t201, const TC* __restrict__ t202,
-    const double* __restrict__ Minv, int Ns, int Nmu, int Nnu, TC xi, TC xiW2, TC* __restrict__ S,
-    const int* kstop, int step) {
+    const TI* __restrict__ x, const double* __restrict__ dinv, const float* __restrict__ wray,
+    const float* __restrict__ t201, const float* __restrict__ t202, const double* __restrict__ Minv, int Ns, int Nmu,
+    int64_t nray, float xi, float xiW2, float* __restrict__ S, const int* kstop, int step) {
+  pdl_wait();
   if (kstop && step >= *kstop) return;
-  moments_height<TI, TC, MODE>(x, dinv, wnu, wmu, t201, t202, Minv, Ns, Nmu, Nnu, xi, xiW2, S, blockIdx.x);
+  moments_flat32<TI, MODE>(x, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
 }
 
 // FP64 quadrature, one CTA per height (flat over the rays); WJ: Jacobi mode
@@ -242,6 +242,7 @@ __global__ void __launch_bounds__(kMom64Threads) k_moments64(
     const double* __restrict__ x, const double* __restrict__ dinv, const double* __restrict__ wray,
     const double* __restrict__ t201, const double* __restrict__ t202, const double* __restrict__ Minv, int Ns,
     int Nmu, int64_t nray, double xi, double xiW2, double* __restrict__ S, const int* kstop, int step) {
+  pdl_wait();   // x, the step counter, and S, which the formal solver before may still read
   if (kstop && step >= *kstop) return;
   if (PAIR) moments_pair64<MODE>(x, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
   else moments_flat64<MODE, WJ>(x, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
@@ -288,6 +289,7 @@ __global__ void k_jacobi_weights(const double* __restrict__ wray, const double* 
 template <typename TC, typename TV, int FS, int MODE, int NSPLIT, int RING, int MAXT>
 __global__ void __launch_bounds__(32 * MAXT) k_formal(const FormalArgs A) {
   constexpr int NS = 2 / NSPLIT;   // Stokes parameters per lane
+  pdl_wait();   // the source values of the quadrature before
   if (A.kstop && A.step >= *A.kstop) return;
   const int lane = threadIdx.x & 31, t = threadIdx.x >> 5;
   const int s0 = NSPLIT == 2 ? (blockIdx.x & 1) : 0;
@@ -347,8 +349,8 @@ __global__ void __launch_bounds__(32 * MAXT) k_formal(const FormalArgs A) {
 #pragma unroll
     for (int q = 0; q < NS; ++q) {
       const int64_t o = (int64_t)(s0 + q) * Ns * A.nray + (int64_t)k0 * A.nray + r;
-      if (MODE == KM_RHS) y[o] = (TV)I[q];
-      else if (MODE == KM_JACOBI) y[o] = (TV)((TC)x[o] * (TC)A.dinv[o]);
+      if (MODE == KM_RHS) y[o] = vcast<TV>(I[q]);
+      else if (MODE == KM_JACOBI) y[o] = vcast<TV>(vcast<TC>(x[o]) * vcast<TC>(A.dinv[o]));
       else y[o] = x[o];
     }
   }
@@ -404,15 +406,15 @@ void dev_free(Problem* P, void* p) {
 }
 
 void free_device(Problem* P) {
-  void* ptrs[] = {P->ce,     P->ca,    P->cb,     P->wray,   P->wI2,  P->wQ2,   P->t201d, P->t202d,
-                  P->Bd,     P->Minv,  P->S,      P->S2,     P->dtau32, P->r32, P->wray32, P->wI2f,
-                  P->wQ2f,   P->t201f, P->t202f,  P->S32,    P->V,    P->work,  P->dinv,  P->work32,
+  void* ptrs[] = {P->ce,     P->ca,    P->cb,     P->wray,   P->t201d, P->t202d,
+                  P->Bd,     P->Minv,  P->S,      P->S2,     P->dtau32, P->r32, P->wray32,
+                  P->t201f, P->t202f,  P->S32,    P->V,    P->work,  P->dinv,  P->work32,
                   P->partials, P->gm,  P->bc,     P->hist,  P->dev_err, P->bpart, P->qw, P->stab, P->qpart, P->qcnt, P->tile_dt, P->Mdiag, P->Ibuf, P->cg,
                   P->Etile, P->Bmap, P->Asig, P->Mpre, P->Mtri, P->Mscr, P->wjac, P->Kmap};
   for (void* p : ptrs)
     if (p) dev_free(P, p);
-  P->ce = P->ca = P->cb = P->wray = P->wI2 = P->wQ2 = P->t201d = P->t202d = P->Bd = P->Minv = P->S = P->S2 = nullptr;
-  P->dtau32 = P->r32 = P->wray32 = P->wI2f = P->wQ2f = P->t201f = P->t202f = P->S32 = nullptr;
+  P->ce = P->ca = P->cb = P->wray = P->t201d = P->t202d = P->Bd = P->Minv = P->S = P->S2 = nullptr;
+  P->dtau32 = P->r32 = P->wray32 = P->t201f = P->t202f = P->S32 = nullptr;
   P->V = P->work = P->dinv = P->partials = P->hist = P->bpart = nullptr;
   P->work32 = nullptr;
   P->gm = nullptr;
@@ -811,8 +813,7 @@ rt_status setup_device_tables(Problem* P, cudaStream_t st) {
   if (const char* t = std::getenv("RT_TILES64")) P->ntile64 = std::min(kMaxTiles64, std::max(1, std::atoi(t)));
 #endif
   P->ntile32 = choose_tiles32(P);
-  std::vector<double> dtau(Ns - 1), rscale(nray), w0(3 * nray), wnu(P->w_nu), wmu(Nmu);
-  for (int m = 0; m < Nmu; ++m) wmu[m] = 0.5 * P->w_mu[m];
+  std::vector<double> dtau(Ns - 1), rscale(nray), w0(3 * nray);
   for (int i = 0; i + 1 < Ns; ++i) dtau[i] = P->tau[i + 1] - P->tau[i];
   for (int m = 0; m < Nmu; ++m)
     for (int p = 0; p < Nnu; ++p) {
@@ -839,8 +840,6 @@ rt_status setup_device_tables(Problem* P, cudaStream_t st) {
   RT_TRY(upload(P, &d_dtau, dtau, st));
   RT_TRY(upload(P, &d_rs, rscale, st));
   RT_TRY(upload(P, &P->wray, w0, st));
-  RT_TRY(upload(P, &P->wI2, wnu, st));   // spectral weights hat-w_p
-  RT_TRY(upload(P, &P->wQ2, wmu, st));   // angular weights hat-w_m
   RT_TRY(upload(P, &P->t201d, P->t201, st));
   RT_TRY(upload(P, &P->t202d, P->t202, st));
   RT_TRY(upload(P, &P->Bd, P->B, st));
@@ -881,20 +880,16 @@ rt_status setup_device_tables(Problem* P, cudaStream_t st) {
   if (P->form == RT_FORM_SIGMA) RT_TRY_CUDA(dev_alloc(P, (void**)&P->Ibuf, (size_t)P->N * sizeof(double)));
   RT_TRY_CUDA(cudaGetLastError());
   // FP32 tables
-  std::vector<float> dtau32(Ns - 1), r32(nray), w032(nray), wI32(Nnu), wQ32(Nmu), t201f(Nmu), t202f(Nmu);
+  std::vector<float> dtau32(Ns - 1), r32(nray), w032(3 * nray), t201f(Nmu), t202f(Nmu);
   for (int i = 0; i + 1 < Ns; ++i) dtau32[i] = (float)dtau[i];
   for (int64_t r = 0; r < nray; ++r) {
     r32[r] = (float)rscale[r];
-    w032[r] = (float)w0[r];
   }
-  for (int p = 0; p < Nnu; ++p) wI32[p] = (float)wnu[p];
-  for (int m = 0; m < Nmu; ++m) wQ32[m] = (float)wmu[m];
+  for (int64_t r = 0; r < 3 * nray; ++r) w032[r] = (float)w0[r];
   for (int m = 0; m < Nmu; ++m) { t201f[m] = (float)P->t201[m]; t202f[m] = (float)P->t202[m]; }
   RT_TRY(upload(P, &P->dtau32, dtau32, st));
   RT_TRY(upload(P, &P->r32, r32, st));
   RT_TRY(upload(P, &P->wray32, w032, st));
-  RT_TRY(upload(P, &P->wI2f, wI32, st));
-  RT_TRY(upload(P, &P->wQ2f, wQ32, st));
   RT_TRY(upload(P, &P->t201f, t201f, st));
   RT_TRY(upload(P, &P->t202f, t202f, st));
   RT_TRY_CUDA(dev_alloc(P, (void**)&P->S32, (size_t)2 * Ns * Nmu * sizeof(float)));
@@ -978,13 +973,13 @@ static void launch_formal32(const Problem* P, const TV* x, TV* y, cudaStream_t s
   const int g = P->ngroups, b = 32 * P->ntile32;
   switch (P->fs) {
     case RT_FS_DELO_LINEAR:
-      k_formal<float, TV, RT_FS_DELO_LINEAR, MODE, 1, kRing32, kMaxTiles><<<g, b, 0, st>>>(A); RT_COUNT(1);
+      launch_pdl(k_formal<float, TV, RT_FS_DELO_LINEAR, MODE, 1, kRing32, kMaxTiles>, g, b, st, A); RT_COUNT(1);
       break;
     case RT_FS_IMPLICIT_EULER:
-      k_formal<float, TV, RT_FS_IMPLICIT_EULER, MODE, 1, kRing32, kMaxTiles><<<g, b, 0, st>>>(A); RT_COUNT(1);
+      launch_pdl(k_formal<float, TV, RT_FS_IMPLICIT_EULER, MODE, 1, kRing32, kMaxTiles>, g, b, st, A); RT_COUNT(1);
       break;
     default:
-      k_formal<float, TV, RT_FS_TRAPEZOIDAL, MODE, 1, kRing32, kMaxTiles><<<g, b, 0, st>>>(A); RT_COUNT(1);
+      launch_pdl(k_formal<float, TV, RT_FS_TRAPEZOIDAL, MODE, 1, kRing32, kMaxTiles>, g, b, st, A); RT_COUNT(1);
   }
 }
 
@@ -1034,26 +1029,26 @@ rt_status op_apply64(Problem* P, const double* x, double* y, int mode, cudaStrea
     RT_TRY_CUDA(cudaGetLastError());
     return RT_OK;
   }
+  // the quadrature as a programmatic dependent of whatever ran before: its
+  // launch overlaps that kernel's tail
+  auto moments = [&](auto kernel, const double* dinv, const double* w, const double* Minv) {
+    RT_COUNT(1);
+    return launch_pdl(kernel, Ns, kMom64Threads, st, x, dinv, w, (const double*)P->t201d, (const double*)P->t202d, Minv,
+                      Ns, Nmu, P->nray, P->xi, xiW2, P->S, kstop, step);
+  };
   switch (mode) {
     case AM_PLAIN:
-      (pair ? k_moments64<KM_PLAIN, false, true> : k_moments64<KM_PLAIN>)<<<Ns, kMom64Threads, 0, st>>>(x, nullptr, P->wray, P->t201d, P->t202d, nullptr, Ns, Nmu,
-                                                          P->nray, P->xi, xiW2, P->S, kstop, step); RT_COUNT(1);
+      RT_TRY_CUDA(moments(pair ? k_moments64<KM_PLAIN, false, true> : k_moments64<KM_PLAIN>, nullptr, P->wray, nullptr));
       launch_formal64<KM_PLAIN>(P, x, y, P->S, st, kstop, step);
       break;
     case AM_JACOBI:
-      if (P->wjac)
-        k_moments64<KM_JACOBI, true><<<Ns, kMom64Threads, 0, st>>>(x, nullptr, P->wjac, P->t201d, P->t202d, nullptr,
-                                                                   Ns, Nmu, P->nray, P->xi, xiW2, P->S, kstop, step);
-      else
-        k_moments64<KM_JACOBI><<<Ns, kMom64Threads, 0, st>>>(x, P->dinv, P->wray, P->t201d, P->t202d, nullptr, Ns,
-                                                             Nmu, P->nray, P->xi, xiW2, P->S, kstop, step);
-      RT_COUNT(1);
+      if (P->wjac) RT_TRY_CUDA(moments(k_moments64<KM_JACOBI, true>, nullptr, P->wjac, nullptr));
+      else RT_TRY_CUDA(moments(k_moments64<KM_JACOBI>, P->dinv, P->wray, nullptr));
       launch_formal64<KM_JACOBI>(P, x, y, P->S, st, kstop, step);
       break;
     case AM_LOCAL_LAMBDA:
-      (pair ? k_moments64<KM_LOCAL_LAMBDA, false, true> : k_moments64<KM_LOCAL_LAMBDA>)<<<Ns, kMom64Threads, 0, st>>>(x, nullptr, P->wray, P->t201d, P->t202d, P->Minv,
-                                                                 Ns, Nmu, P->nray, P->xi, xiW2, P->S, kstop, step);
-      RT_COUNT(1);
+      RT_TRY_CUDA(moments(pair ? k_moments64<KM_LOCAL_LAMBDA, false, true> : k_moments64<KM_LOCAL_LAMBDA>, nullptr,
+                          P->wray, P->Minv));
       launch_formal64<KM_LOCAL_LAMBDA>(P, x, y, P->S, st, kstop, step);
       break;
     default:
@@ -1087,24 +1082,23 @@ static rt_status apply32_impl(Problem* P, const TV* x, TV* y, int mode, cudaStre
     return RT_EINVAL;
   }
   const float xi = (float)P->xi, xiW2 = (float)(P->xi * P->W2);
-  const int Ns = P->Ns, Nmu = P->Nmu, Nnu = P->Nnu;
+  const int Ns = P->Ns, Nmu = P->Nmu;
+  auto moments = [&](auto kernel, const double* dinv, const double* Minv) {   // as in op_apply64
+    RT_COUNT(1);
+    return launch_pdl(kernel, Ns, kMomThreads, st, x, dinv, (const float*)P->wray32, (const float*)P->t201f,
+                      (const float*)P->t202f, Minv, Ns, Nmu, P->nray, xi, xiW2, P->S32, kstop, step);
+  };
   switch (mode) {
     case AM_PLAIN:
-      k_moments<TV, float, KM_PLAIN><<<Ns, kMomThreads, 0, st>>>(x, nullptr, P->wI2f, P->wQ2f, P->t201f,
-                                                                  P->t202f, nullptr, Ns, Nmu, Nnu, xi, xiW2, P->S32,
-                                                                  kstop, step); RT_COUNT(1);
+      RT_TRY_CUDA(moments(k_moments<TV, KM_PLAIN>, nullptr, nullptr));
       launch_formal32<TV, KM_PLAIN>(P, x, y, st, kstop, step);
       break;
     case AM_JACOBI:
-      k_moments<TV, float, KM_JACOBI><<<Ns, kMomThreads, 0, st>>>(x, P->dinv, P->wI2f, P->wQ2f, P->t201f,
-                                                                   P->t202f, nullptr, Ns, Nmu, Nnu, xi, xiW2, P->S32,
-                                                                   kstop, step); RT_COUNT(1);
+      RT_TRY_CUDA(moments(k_moments<TV, KM_JACOBI>, P->dinv, nullptr));
       launch_formal32<TV, KM_JACOBI>(P, x, y, st, kstop, step);
       break;
     case AM_LOCAL_LAMBDA:
-      k_moments<TV, float, KM_LOCAL_LAMBDA><<<Ns, kMomThreads, 0, st>>>(x, nullptr, P->wI2f, P->wQ2f,
-                                                                         P->t201f, P->t202f, P->Minv, Ns, Nmu, Nnu,
-                                                                         xi, xiW2, P->S32, kstop, step); RT_COUNT(1);
+      RT_TRY_CUDA(moments(k_moments<TV, KM_LOCAL_LAMBDA>, nullptr, P->Minv));
       launch_formal32<TV, KM_LOCAL_LAMBDA>(P, x, y, st, kstop, step);
       break;
     default:

@@ -196,7 +196,7 @@ __device__ __forceinline__ float4 load4<float>(const float* p) {
 template <>
 __device__ __forceinline__ float4 load4<double>(const double* p) {
   const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
-  return make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+  return make_float4(to_f32(a.x), to_f32(a.y), to_f32(b.x), to_f32(b.y));
 }
 
 // four FP64 values of u scaled by inv: stored to xo (the GMRES normalisation
@@ -209,7 +209,7 @@ __device__ __forceinline__ float4 load4_scaled(const double* u, double inv, doub
   b.y *= inv;
   reinterpret_cast<double2*>(xo)[0] = a;
   reinterpret_cast<double2*>(xo)[1] = b;
-  return make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+  return make_float4(to_f32(a.x), to_f32(a.y), to_f32(b.x), to_f32(b.y));
 }
 
 // Where the quadrature puts its result: the multipolar components of every
@@ -593,7 +593,7 @@ __device__ __forceinline__ void staged_body(const StagedArgs& A, const Maps& M, 
       if (ru == kRS - 1) pn += kRS;
       float e, al, be;
       step_coeffs<FS>(op, rsc, irsc, e, al, be);
-      const float xI = (float)xs[row * 32 + lane], xQ = (float)xs[(DK + row) * 32 + lane];
+      const float xI = vcast<float>(xs[row * 32 + lane]), xQ = vcast<float>(xs[(DK + row) * 32 + lane]);
       float yvI, yvQ;
       if (MODE == KM_LOCAL_LAMBDA) {
         // y = x - (I - beta S): the step without its beta S_k term
@@ -606,8 +606,8 @@ __device__ __forceinline__ void staged_body(const StagedArgs& A, const Maps& M, 
         U0 = fmaf(e, U0, fmaf(al, s0p, be * op.x));
         U2 = fmaf(e, U2, fmaf(al, s2p, be * op.y));
         if (MODE == KM_JACOBI) {
-          yvI = fmaf(xI, (float)ds[row * 32 + lane], -fmaf(t201, U2, U0));
-          yvQ = fmaf(xQ, (float)ds[(DK + row) * 32 + lane], -(t202 * U2));
+          yvI = fmaf(xI, to_f32(ds[row * 32 + lane]), -fmaf(t201, U2, U0));
+          yvQ = fmaf(xQ, to_f32(ds[(DK + row) * 32 + lane]), -(t202 * U2));
         } else {
           yvI = xI - fmaf(t201, U2, U0);
           yvQ = fmaf(-t202, U2, xQ);
@@ -617,8 +617,8 @@ __device__ __forceinline__ void staged_body(const StagedArgs& A, const Maps& M, 
       s2p = op.y;
       if (active) {   // evict-first stores: in a large apply, y would push out of L2 the lines of x
                       // that the quadrature left there and other warps have still to read
-        __stcs(yI, (TV)yvI);
-        __stcs(yI + plane, (TV)yvQ);
+        __stcs(yI, vcast<TV>(yvI));
+        __stcs(yI + plane, vcast<TV>(yvQ));
       }
       yI += dy;
     };
