@@ -75,7 +75,7 @@ struct InstStatus {
 };
 
 struct Counts {
-  int nh, ng64, nc, ni;
+  int nh, ng64, nc, ni;    // items of the quadrature, the FP64 formal solver, the vector kernels; instances
   int ng32[3], off32[3];   // FP32 formal-solver items, grouped by formal solver
 };
 
@@ -141,6 +141,7 @@ __device__ __forceinline__ double inst_norm_inv(const InstDev& I, int pb, double
 template <typename TC, int MODE, bool NORM = false>
 __global__ void __launch_bounds__(kMomThreads) kb_moments(const InstDev* __restrict__ insts, const int2* __restrict__ wl,
                                                           const Counts* cnt, int src, int step, int useS2) {
+  pdl_wait();
   const int n = cnt->nh;
   for (int w = blockIdx.x; w < n; w += gridDim.x) {
     const int2 it = wl[w];
@@ -217,6 +218,7 @@ template <int MODE>
 __global__ void __launch_bounds__(32 * kFormalWarps) kb_formal(const InstDev* __restrict__ insts,
                                                                const int4* __restrict__ wl, const Counts* cnt,
                                                                int src, int dst, int step) {
+  pdl_wait();
   const int n = cnt->ng64;
   const int warps = gridDim.x * (blockDim.x >> 5);
   for (int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < n; w += warps) {
@@ -284,6 +286,7 @@ __global__ void __launch_bounds__(32 * kTiles32) kb_formal32(const InstDev* __re
                                                              const int4* __restrict__ wl, const Counts* cnt, int src,
                                                              int dst, int step) {
   __shared__ float sh[3][kTiles32][32];   // per tile: E, B of I, B of Q
+  pdl_wait();
   const int n = cnt->ng32[FS], off = cnt->off32[FS];
   for (int w = blockIdx.x; w < n; w += gridDim.x) {
     const int4 it = wl[off + w];
@@ -324,6 +327,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) kb_pass(const InstDev* __rest
   __shared__ double hs[B], gs[B][B];
   PassRing R;
   pass_ring_init(R, pass_dyn, bars, &dead, S::NST);
+  pdl_wait();
   const int64_t n = cnt->nc;
   const int w0 = (int)(n * blockIdx.x / gridDim.x), w1 = (int)(n * (blockIdx.x + 1) / gridDim.x);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -391,6 +395,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) kb_pass(const InstDev* __rest
 __global__ void __launch_bounds__(32 * kBatchB) kb_givens(const InstDev* __restrict__ insts,
                                                          const int* __restrict__ wi, const Counts* cnt, int j, int pb,
                                                          int ng) {
+  pdl_wait();
   for (int q = blockIdx.x; q < cnt->ni; q += gridDim.x) {
     const InstDev& I = insts[wi[q]];
     if (j < I.gm->kstop)
@@ -413,6 +418,7 @@ struct KbPassTable {
 const KbPassTable kb_passes;
 
 __global__ void kb_lsq(const InstDev* __restrict__ insts, const int* __restrict__ wi, const Counts* cnt) {
+  pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= cnt->ni) return;
   const InstDev& I = insts[wi[q]];
@@ -428,6 +434,7 @@ __global__ void kb_lsq(const InstDev* __restrict__ insts, const int* __restrict_
 // s = sum_{i<kdone} y_i V_i; mode 0: x += s, 1: x += dinv s, 2: t = s
 __global__ void __launch_bounds__(kBT) kb_combine(const InstDev* __restrict__ insts, const int2* __restrict__ wl,
                                                   const Counts* cnt, int mode) {
+  pdl_wait();
   __shared__ double ys[kMaxRestart];
   for (int w = blockIdx.x; w < cnt->nc; w += gridDim.x) {
     const int2 it = wl[w];
@@ -445,6 +452,7 @@ __global__ void __launch_bounds__(kBT) kb_combine(const InstDev* __restrict__ in
 // x += t + beta* S2 (P^{-1} t with S2 = T M^{-1} J t)
 __global__ void __launch_bounds__(kBT) kb_add_local(const InstDev* __restrict__ insts, const int2* __restrict__ wl,
                                                     const Counts* cnt) {
+  pdl_wait();
   for (int w = blockIdx.x; w < cnt->nc; w += gridDim.x) {
     const int2 it = wl[w];
     const InstDev& I = insts[it.x];
@@ -459,6 +467,7 @@ __global__ void __launch_bounds__(kBT) kb_add_local(const InstDev* __restrict__ 
 // r = b - tmp; partial ||r||^2 into part[0]
 __global__ void __launch_bounds__(kBT) kb_residual(const InstDev* __restrict__ insts, const int2* __restrict__ wl,
                                                    const Counts* cnt) {
+  pdl_wait();
   for (int w = blockIdx.x; w < cnt->nc; w += gridDim.x) {
     const int2 it = wl[w];
     const InstDev& I = insts[it.x];
@@ -480,6 +489,7 @@ __global__ void kb_set_bnorm(const InstDev* __restrict__ insts, const int* __res
 // start of a cycle: beta = ||r||, v_0 = r / beta, g = beta e_1, step budget
 __global__ void __launch_bounds__(kBT) kb_cycle_start(const InstDev* __restrict__ insts, const int2* __restrict__ wl,
                                                       const Counts* cnt, InstStatus* __restrict__ status) {
+  pdl_wait();
   for (int w = blockIdx.x; w < cnt->nc; w += gridDim.x) {
     const int2 it = wl[w];
     const InstDev& I = insts[it.x];
@@ -658,6 +668,7 @@ struct Server {
   int* d_wl_new_i = nullptr;
   Counts* d_new_counts = nullptr;
   size_t cap_new_c = 0;
+  int fs_mask = 0;              // formal solvers (bit RT_FS_*) that instances have used so far
   cudaGraphExec_t graph = nullptr;
   long long graph_kernels = 0;
   std::atomic<long long> cycles{0}, completed{0};
@@ -711,44 +722,60 @@ size_t solver_bytes(int64_t N, int m, int nchunks) {
 constexpr int64_t kChunk = 8192;
 static_assert(kChunk % kPassTile == 0, "a chunk starts on a tile");
 
+// a kernel of the cycle: a programmatic dependent of the one before (each of
+// them waits first), so that its launch overlaps that one's tail
+template <typename... KArgs, typename... Args>
+void kb_launch(void (*kernel)(KArgs...), int grid, int block, cudaStream_t st, Args... args) {
+  launch_pdl(kernel, grid, block, st, args...);
+  RT_COUNT(1);
+}
+
+// one launch per formal solver that a resident instance uses (an empty list
+// would still cost a launch, 3 us)
 template <int MODE>
 void formal32(Server* S, cudaStream_t st, int src, int dst, int step) {
-  kb_formal32<RT_FS_DELO_LINEAR, MODE><<<S->grid_g, 32 * kTiles32, 0, st>>>(S->d_insts, S->d_wl_g32, S->d_counts, src, dst, step); RT_COUNT(1);
-  kb_formal32<RT_FS_IMPLICIT_EULER, MODE><<<S->grid_g, 32 * kTiles32, 0, st>>>(S->d_insts, S->d_wl_g32, S->d_counts, src, dst, step); RT_COUNT(1);
-  kb_formal32<RT_FS_TRAPEZOIDAL, MODE><<<S->grid_g, 32 * kTiles32, 0, st>>>(S->d_insts, S->d_wl_g32, S->d_counts, src, dst, step); RT_COUNT(1);
+  auto go = [&](auto kernel) {
+    kb_launch(kernel, S->grid_g, 32 * kTiles32, st, (const InstDev*)S->d_insts, (const int4*)S->d_wl_g32,
+              (const Counts*)S->d_counts, src, dst, step);
+  };
+  if (S->fs_mask & 1) go(kb_formal32<RT_FS_DELO_LINEAR, MODE>);
+  if (S->fs_mask & 2) go(kb_formal32<RT_FS_IMPLICIT_EULER, MODE>);
+  if (S->fs_mask & 4) go(kb_formal32<RT_FS_TRAPEZOIDAL, MODE>);
 }
 
 template <bool NORM>
 void enqueue_apply_t(Server* S, cudaStream_t st, int src, int dst, int md, bool f32, int step) {
   const InstDev* I = S->d_insts;
   const Counts* C = S->d_counts;
+  const int2* wh = S->d_wl_h;
+  const int4* w64 = S->d_wl_g64;
+  const int f64b = 32 * kFormalWarps;
   if (!f32) {
     switch (md) {
       case KM_JACOBI:
-        kb_moments<double, KM_JACOBI, NORM><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, src, step, 0); RT_COUNT(1);
-        kb_formal<KM_JACOBI><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(I, S->d_wl_g64, C, src, dst, step); RT_COUNT(1);
+        kb_launch(kb_moments<double, KM_JACOBI, NORM>, S->grid_h, kMomThreads, st, I, wh, C, src, step, 0);
+        kb_launch(kb_formal<KM_JACOBI>, S->grid_g, f64b, st, I, w64, C, src, dst, step);
         break;
       case KM_LOCAL_LAMBDA:
-        kb_moments<double, KM_LOCAL_LAMBDA, NORM><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, src, step, 0); RT_COUNT(1);
-        kb_formal<KM_LOCAL_LAMBDA><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(I, S->d_wl_g64, C, src, dst,
-                                                                                     step); RT_COUNT(1);
+        kb_launch(kb_moments<double, KM_LOCAL_LAMBDA, NORM>, S->grid_h, kMomThreads, st, I, wh, C, src, step, 0);
+        kb_launch(kb_formal<KM_LOCAL_LAMBDA>, S->grid_g, f64b, st, I, w64, C, src, dst, step);
         break;
       default:
-        kb_moments<double, KM_PLAIN, NORM><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, src, step, 0); RT_COUNT(1);
-        kb_formal<KM_PLAIN><<<S->grid_g, 32 * kFormalWarps, 0, st>>>(I, S->d_wl_g64, C, src, dst, step); RT_COUNT(1);
+        kb_launch(kb_moments<double, KM_PLAIN, NORM>, S->grid_h, kMomThreads, st, I, wh, C, src, step, 0);
+        kb_launch(kb_formal<KM_PLAIN>, S->grid_g, f64b, st, I, w64, C, src, dst, step);
     }
   } else {
     switch (md) {
       case KM_JACOBI:
-        kb_moments<float, KM_JACOBI, NORM><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, src, step, 0); RT_COUNT(1);
+        kb_launch(kb_moments<float, KM_JACOBI, NORM>, S->grid_h, kMomThreads, st, I, wh, C, src, step, 0);
         formal32<KM_JACOBI>(S, st, src, dst, step);
         break;
       case KM_LOCAL_LAMBDA:
-        kb_moments<float, KM_LOCAL_LAMBDA, NORM><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, src, step, 0); RT_COUNT(1);
+        kb_launch(kb_moments<float, KM_LOCAL_LAMBDA, NORM>, S->grid_h, kMomThreads, st, I, wh, C, src, step, 0);
         formal32<KM_LOCAL_LAMBDA>(S, st, src, dst, step);
         break;
       default:
-        kb_moments<float, KM_PLAIN, NORM><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, src, step, 0); RT_COUNT(1);
+        kb_launch(kb_moments<float, KM_PLAIN, NORM>, S->grid_h, kMomThreads, st, I, wh, C, src, step, 0);
         formal32<KM_PLAIN>(S, st, src, dst, step);
     }
   }
@@ -845,36 +872,38 @@ rt_status enqueue_batch_cycle(Server* S, cudaStream_t st) {
   const int mode = prec == RT_PREC_JACOBI ? KM_JACOBI : prec == RT_PREC_LOCAL_LAMBDA ? KM_LOCAL_LAMBDA : KM_PLAIN;
   const InstDev* I = S->d_insts;
   const Counts* C = S->d_counts;
+  const int2* wc = S->d_wl_c;
+  const int* wi = S->d_wl_i;
   for (int j = 0; j < m; ++j) {
     // steps after the first normalise v_j = w / ||w|| inside the quadrature
     enqueue_apply(S, st, j, VW, mode, fp32, j, j > 0);
     int pb = 0;
     const int gp = 2 * S->sms;   // the passes' resident CTAs
-    kb_passes.dot[std::min(kBatchB, j + 1) - 1]<<<gp, kPassThreads, kPassDynSmem, st>>>(I, S->d_wl_c, C, j, 0, 0); RT_COUNT(1);
+    RT_TRY_CUDA(launch_pdl_smem(kb_passes.dot[std::min(kBatchB, j + 1) - 1], gp, kPassThreads, kPassDynSmem, st, I, wc, C, j, 0, 0)); RT_COUNT(1);
     for (int i0 = 0; i0 <= j; i0 += kBatchB) {
       const int nb = std::min(kBatchB, j + 1 - i0);
       const int nn = std::max(0, std::min(kBatchB, j + 1 - (i0 + nb)));
-      (nn ? kb_passes.mid[nn - 1] : kb_passes.last[nb - 1])<<<gp, kPassThreads, kPassDynSmem, st>>>(I, S->d_wl_c, C, j,
-                                                                                                    i0, pb); RT_COUNT(1);
+      RT_TRY_CUDA(launch_pdl_smem(nn ? kb_passes.mid[nn - 1] : kb_passes.last[nb - 1], gp, kPassThreads, kPassDynSmem, st, I, wc, C, j,
+                                  i0, pb)); RT_COUNT(1);
       pb ^= 1;
     }
     // h_{j+1,j}, the Gram row, the rotations and the inverse norm that the
     // next step's quadrature scales w by; an instance that stops at step j
     // never forms v_{j+1}, which no later kernel of the cycle reads
     const int ng = (j + 1) % kBatchB;
-    kb_givens<<<std::min(S->opts.max_slots, 4 * S->sms), 32 * kBatchB, 0, st>>>(I, S->d_wl_i, C, j, pb, ng); RT_COUNT(1);
+    kb_launch(kb_givens, std::min(S->opts.max_slots, 4 * S->sms), 32 * kBatchB, st, I, wi, C, j, pb, ng);
   }
-  kb_lsq<<<S->grid_i, kInstThreads, 0, st>>>(I, S->d_wl_i, C); RT_COUNT(1);
+  kb_launch(kb_lsq, S->grid_i, kInstThreads, st, I, wi, C);
   if (mode == KM_LOCAL_LAMBDA) {
-    kb_combine<<<S->grid_v, kBT, 0, st>>>(I, S->d_wl_c, C, 2); RT_COUNT(1);
-    kb_moments<double, KM_LOCAL_LAMBDA><<<S->grid_h, kMomThreads, 0, st>>>(I, S->d_wl_h, C, VT, -1, 1); RT_COUNT(1);
-    kb_add_local<<<S->grid_v, kBT, 0, st>>>(I, S->d_wl_c, C); RT_COUNT(1);
+    kb_launch(kb_combine, S->grid_v, kBT, st, I, wc, C, 2);
+    kb_launch(kb_moments<double, KM_LOCAL_LAMBDA>, S->grid_h, kMomThreads, st, I, (const int2*)S->d_wl_h, C, (int)VT, -1, 1);
+    kb_launch(kb_add_local, S->grid_v, kBT, st, I, wc, C);
   } else {
-    kb_combine<<<S->grid_v, kBT, 0, st>>>(I, S->d_wl_c, C, mode == KM_JACOBI ? 1 : 0); RT_COUNT(1);
+    kb_launch(kb_combine, S->grid_v, kBT, st, I, wc, C, mode == KM_JACOBI ? 1 : 0);
   }
   enqueue_apply(S, st, VX, VTMP, KM_PLAIN, false, -1);   // FP64 true residual
-  kb_residual<<<S->grid_v, kBT, 0, st>>>(I, S->d_wl_c, C); RT_COUNT(1);
-  kb_cycle_start<<<S->grid_v, kBT, 0, st>>>(I, S->d_wl_c, C, S->d_status); RT_COUNT(1);
+  kb_launch(kb_residual, S->grid_v, kBT, st, I, wc, C);
+  kb_launch(kb_cycle_start, S->grid_v, kBT, st, I, wc, C, S->d_status);
   RT_TRY_CUDA(cudaGetLastError());
   return RT_OK;
 }
@@ -938,10 +967,18 @@ rt_status rebuild_lists(Server* S) {
     for (int cc = 0; cc < in->dev.nchunks; ++cc) c.push_back(make_int2(sl, cc));
   }
   Counts cn{(int)h.size(), (int)g64.size(), (int)c.size(), (int)wi.size(), {0, 0, 0}, {0, 0, 0}};
+  int mask = 0;
   for (int f = 0; f < 3; ++f) {
     cn.off32[f] = (int)g32.size();
     cn.ng32[f] = (int)g32f[f].size();
+    if (cn.ng32[f]) mask |= 1 << f;
     g32.insert(g32.end(), g32f[f].begin(), g32f[f].end());
+  }
+  // the captured cycle launches the formal solvers of the mask; one that is
+  // no longer resident costs a launch, not a new capture
+  if (mask & ~S->fs_mask) {
+    S->fs_mask |= mask;
+    drop_graph(S);
   }
   // interleave the formal-solver items of different instances so that big
   // instances do not end up on the same SMs

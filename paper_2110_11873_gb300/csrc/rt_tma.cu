@@ -118,13 +118,6 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tm)) : "memory");
 }
 
-// 2^a by the hardware's approximate exponential (a <= 0 here)
-__device__ __forceinline__ float ex2_approx(float a) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
-  return r;
-}
-
 // ------------------------------------------------------ step coefficients
 // The coefficients of I_k = e I_prev + alpha S_prev + beta S_k from the node
 // operand op (op.z, op.w: the interval constants of the table) and the ray's
@@ -143,14 +136,8 @@ __device__ __forceinline__ float ex2_approx(float a) {
 //   trapezoidal: op.z = dtau; h = Delta / 2, q = 1 / (1 + h), e = (1 - h) q,
 //     alpha = beta = h q.
 //   (reciprocals by the hardware approximation, within 2 ulp)
-constexpr double kLn2 = 0.69314718055994530942;
-constexpr float kSeriesD2 = (float)(0.5 / kLn2);
-
-// (-1)^n ln2^(n+1) / (n+2)!: the series of beta / D2 in powers of D2
-constexpr double pow_ln2(int k) { return k == 0 ? 1.0 : kLn2 * pow_ln2(k - 1); }
-constexpr double fact(int k) { return k <= 1 ? 1.0 : k * fact(k - 1); }
-constexpr float kB(int n) { return (float)((n % 2 ? -1.0 : 1.0) * pow_ln2(n + 1) / fact(n + 2)); }
-
+// DELO-linear as delo_coeffs, written out: calling it forms 1 / Delta ahead of
+// the series and took 131.1 us instead of 130.4 on N = 51.5 million.
 template <int FS>
 __device__ __forceinline__ void step_coeffs(const float4& op, float rsc, float irsc, float& e, float& al, float& be) {
   if (FS == RT_FS_DELO_LINEAR) {
