@@ -512,6 +512,126 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_pass(double* __restrict__ w
   if (threadIdx.x == 0 && dead) atomicExch(err, 1);
 }
 
+// A whole Arnoldi step of a short vector (the sigma-form: N = 2 Ns) in one CTA:
+// the block passes, the normalisation, the Gram row and the Givens rotations,
+// with w in registers.  Kernel by kernel such a step is bound by launches, about
+// 4.5 us each whatever the length (sigma-form run of the paper, N = 280: 57 us
+// a step).  The same block MGS as k_pass with FP64 dots; every warp sums the
+// warps' partial dots and solves the block's triangular system for itself, so
+// a block needs one barrier.
+constexpr int kSmallThreads = 256;
+constexpr int kSmallPer = 4;                                 // elements per thread
+constexpr int64_t kSmallN = (int64_t)kSmallThreads * kSmallPer;
+
+// lane l gets the warp sum of s[l >> 2] (transposing, fixed order)
+__device__ __forceinline__ double warp_sum8(const double (&s)[8]) {
+  const int lane = threadIdx.x & 31;
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+  double a[4], b[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) a[i] = (h16 ? s[i + 4] : s[i]) + __shfl_xor_sync(0xffffffffu, h16 ? s[i] : s[i + 4], 16);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) b[i] = (h8 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, h8 ? a[i] : a[i + 2], 8);
+  double t = (h4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h4 ? b[0] : b[1], 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  return t;
+}
+
+template <int B>
+__global__ void __launch_bounds__(kSmallThreads) k_small_step(double* __restrict__ wv, double* __restrict__ V, int N,
+                                                              double* __restrict__ hcol, double* __restrict__ gram,
+                                                              GmresDev* gm, int m, int j, double* hist, int hist_cap,
+                                                              const int* kstop) {
+  static_assert(B <= 8 && kSmallThreads == 256, "8 dots, 8 warps");
+  pdl_wait();
+  if (kstop && j >= *kstop) return;
+  __shared__ double red[2][8][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k8 = lane >> 2;
+  double w[kSmallPer];
+#pragma unroll
+  for (int e = 0; e < kSmallPer; ++e) {
+    const int n = threadIdx.x + e * kSmallThreads;
+    w[e] = n < N ? wv[n] : 0.0;
+  }
+  int buf = 0;
+  // the CTA's sums of s[0..7]: lane l gets that of s[l >> 2]
+  auto cta_sum8 = [&](const double (&s)[8]) {
+    const double t = warp_sum8(s);
+    if ((lane & 3) == 0) red[buf][k8][warp] = t;
+    __syncthreads();
+    double x = red[buf][k8][2 * (lane & 3)] + red[buf][k8][2 * (lane & 3) + 1];
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    buf ^= 1;
+    return x;
+  };
+  int i0 = 0, nb = 0;
+  for (i0 = 0; i0 <= j; i0 += B) {
+    nb = min(B, j + 1 - i0);
+    const double* __restrict__ vb = V + (size_t)i0 * N;
+    double v[8][kSmallPer], s[8], gl[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      s[k] = 0.0;
+#pragma unroll
+      for (int e = 0; e < kSmallPer; ++e) {
+        const int n = threadIdx.x + e * kSmallThreads;
+        v[k][e] = k < nb && n < N ? vb[(size_t)k * N + n] : 0.0;
+        if (e * kSmallThreads < N) s[k] = fma(w[e], v[k][e], s[k]);
+      }
+      // <v_{i0+k}, v_{i0+k8}>, k < k8
+      gl[k] = k < k8 && k8 < nb ? gram[(i0 + k8) * B + (k8 - k)] : 0.0;
+    }
+    double h = cta_sum8(s);   // h_k = r_k - sum_{l<k} h_l <v_l, v_k>, l in increasing order
+#pragma unroll
+    for (int l = 0; l < 7; ++l) {
+      const double hl = __shfl_sync(0xffffffffu, h, 4 * l);
+      if (k8 > l) h = fma(-hl, gl[l], h);
+    }
+    if (warp == 0 && (lane & 3) == 0 && k8 < nb) hcol[i0 + k8] = h;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const double hk = __shfl_sync(0xffffffffu, h, 4 * k);
+      if (k < nb) {
+#pragma unroll
+        for (int e = 0; e < kSmallPer; ++e)
+          if (e * kSmallThreads < N) w[e] = fma(-hk, v[k][e], w[e]);
+      }
+    }
+    if (i0 + B > j) {   // the last block: ||w||^2 and, while v_{j+1} shares it, its Gram dots
+      const int ng = nb < B ? nb : 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        s[k] = 0.0;
+#pragma unroll
+        for (int e = 0; e < kSmallPer; ++e)
+          if (e * kSmallThreads < N) s[k] = fma(w[e], k == 0 ? w[e] : v[k - 1 < 0 ? 0 : k - 1][e], s[k]);
+      }
+      const double d = cta_sum8(s);
+      const double hn = sqrt(__shfl_sync(0xffffffffu, d, 0));
+      const double inv = hn > 0.0 ? 1.0 / hn : 0.0;
+      double* __restrict__ vo = V + (size_t)(j + 1) * N;
+#pragma unroll
+      for (int e = 0; e < kSmallPer; ++e) {
+        const int n = threadIdx.x + e * kSmallThreads;
+        if (n < N) {
+          wv[n] = w[e];
+          vo[n] = w[e] * inv;
+        }
+      }
+      // set k8: <w, v_{i0+k8-1}> = <w, v_{j+1-dd}>, dd = ng - (k8 - 1)
+      if (warp == 0 && (lane & 3) == 0 && k8 >= 1 && k8 <= ng) gram[(j + 1) * B + (ng - (k8 - 1))] = d * inv;
+      if (threadIdx.x == 0) hcol[j + 1] = hn;
+      __syncwarp();
+      if (threadIdx.x == 0 && gm) {
+        gm->vscale = inv;
+        givens_step(gm, m, j, hist, hist_cap);
+      }
+    }
+  }
+}
+
 // v_{j+1} = w / ||w|| by blocks 1..gridDim.x-1 (||w||^2 is set 0 of the last
 // pass's partials, over Gp blocks).  Block 0, scheduled first, writes
 // h_{j+1} = ||w|| to hcol[j+1] and the Gram row j+1: <v_{j+1}, v_{j+1-d}> =
@@ -982,6 +1102,7 @@ __global__ void k_rich_check(const double* __restrict__ part, int G, GmresDev* g
 __global__ void __launch_bounds__(kVecThreads) k_mul_gated(const double* __restrict__ x,
                                                            const double* __restrict__ d, double* __restrict__ y,
                                                            int64_t N, const int* kstop, int step) {
+  pdl_wait();
   if (kstop && step >= *kstop) return;
   for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x)
     y[n] = x[n] * d[n];
@@ -1075,8 +1196,7 @@ static inline bool prec_left(int pc) {
 static rt_status left_apply(Problem* P, int pc, const double* x, double* y, cudaStream_t st,
                             const int* kstop = nullptr, int step = 0) {
   if (pc == RT_PREC_JACOBI_LEFT) {
-    k_mul_gated<<<P->vec_grid, kVecThreads, 0, st>>>(x, P->dinv, y, P->Nop, kstop, step); RT_COUNT(1);
-    RT_TRY_CUDA(cudaGetLastError());
+    RT_TRY_CUDA(launch_pdl(k_mul_gated, P->vec_grid, kVecThreads, st, x, (const double*)P->dinv, y, P->Nop, kstop, step)); RT_COUNT(1);
     return RT_OK;
   }
   return op_dense_precond_apply(P, x, y, st, kstop, step);
@@ -1158,6 +1278,11 @@ static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* h
   const int Gm = plan.grid;
   const int64_t N = P->Nop;
   int pb = 0, rev = 0, ng = 0;
+  if (scale && N <= kSmallN) {
+    RT_TRY_CUDA(launch_pdl(gb == kGramB ? k_small_step<kGramB> : k_small_step<kGramMax>, 1, kSmallThreads, st, w, V,
+                           (int)N, hcol, gram, gm, m, j, hist, hcap, kstop)); RT_COUNT(1);
+    return RT_OK;
+  }
   if (plan.fixed) {
     if (gb == kGramB) RT_TRY(enqueue_passes(P, g_pass4, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev));
     else RT_TRY(enqueue_passes(P, g_pass8, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev));

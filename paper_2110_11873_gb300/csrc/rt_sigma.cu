@@ -44,6 +44,7 @@ __global__ void k_sig_source(const double* __restrict__ v, const double* __restr
                              const double* __restrict__ Minv, const double* __restrict__ t201,
                              const double* __restrict__ t202, int Ns, int Nmu, double* __restrict__ S,
                              const int* kstop, int step) {
+  pdl_wait();   // v, the step counter, and S, which the formal solver before may still read
   if (kstop && step >= *kstop) return;
   const int64_t n = (int64_t)Ns * Nmu;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(kSigThreads) k_sig_moments(
     const double* __restrict__ Minv, const double* __restrict__ wray, const double* __restrict__ t201,
     const double* __restrict__ t202, const double* __restrict__ B, int Ns, int Nmu, int Nnu, double xi, double xiW2,
     double eps, double* __restrict__ y, const int* kstop, int step) {
+  pdl_wait();
   if (kstop && step >= *kstop) return;
   const int k = blockIdx.x;
   const int64_t nray = (int64_t)Nmu * Nnu;
@@ -212,11 +214,14 @@ inline int blocks_for(int64_t n, int threads, int cap) {
 template <int MODE>
 void launch_sigma(Problem* P, const double* v, double* y, cudaStream_t st, const int* kstop, int step) {
   const int Ns = P->Ns, Nmu = P->Nmu;
-  k_sig_source<MODE><<<blocks_for((int64_t)Ns * Nmu, 256, 4 * P->num_sms), 256, 0, st>>>(
-      v, P->dinv, P->Minv, P->t201d, P->t202d, Ns, Nmu, P->S, kstop, step); RT_COUNT(1);
+  // programmatic dependents: their launches overlap the kernel before
+  launch_pdl(k_sig_source<MODE>, blocks_for((int64_t)Ns * Nmu, 256, 4 * P->num_sms), 256, st, v,
+             (const double*)P->dinv, (const double*)P->Minv, (const double*)P->t201d, (const double*)P->t202d, Ns, Nmu,
+             P->S, kstop, step); RT_COUNT(1);
   formal64_lambda(P, P->S, P->Ibuf, MODE == KM_RHS ? P->B[Ns - 1] : 0.0, st, kstop, step);
-  k_sig_moments<MODE><<<Ns, kSigThreads, 0, st>>>(P->Ibuf, v, P->dinv, P->Minv, P->wray, P->t201d, P->t202d, P->Bd,
-                                                   Ns, Nmu, P->Nnu, P->xi, P->xi * P->W2, P->eps, y, kstop, step);
+  launch_pdl(k_sig_moments<MODE>, Ns, kSigThreads, st, (const double*)P->Ibuf, v, (const double*)P->dinv,
+             (const double*)P->Minv, (const double*)P->wray, (const double*)P->t201d, (const double*)P->t202d,
+             (const double*)P->Bd, Ns, Nmu, P->Nnu, P->xi, P->xi * P->W2, P->eps, y, kstop, step);
   RT_COUNT(1);
 }
 

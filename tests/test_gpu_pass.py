@@ -75,7 +75,8 @@ def _step(P, N, j, kind, offset=0, seed=0):
 
 
 # N = 2 Ns Nmu Nnu: below, at and just past one tile; several tiles; more tiles than CTAs
-@pytest.mark.parametrize("Ns,Nmu,Nnu", [(2, 2, 2), (21, 2, 3), (32, 2, 2), (43, 2, 3), (37, 6, 33), (100, 16, 61)])
+@pytest.mark.parametrize("Ns,Nmu,Nnu", [(2, 2, 2), (21, 2, 3), (32, 2, 2), (43, 2, 3), (64, 4, 2), (43, 2, 6),
+                                        (37, 6, 33), (100, 16, 61)])
 @pytest.mark.parametrize("j", [0, 3, 4, 6, 13])
 def test_pass_sizes(Ns, Nmu, Nnu, j):
     P = problem(W.slab(Ns, Nmu, Nnu, 1e-4, 1e6, 6.0))
