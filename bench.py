@@ -11,8 +11,8 @@ DELO-linear, FP64.
 
 Reported value: operator applies per second over the timed solves (whole job
 over all ranks).  Extra keys: solves/s, the standalone apply rate and its
-algorithmic HBM bandwidth, the roofline object (against the FP64 rate
-measured by a DFMA probe kernel), the small (slab70) and large (slab300,
+algorithmic HBM bandwidth, the roofline object (against the copy bandwidth,
+with the FP64 rate of a DFMA probe kernel), the small (slab70) and large (slab300,
 three methods x two formal solvers x two precisions) workloads, the
 30-case size sweep, the batched and served streams, and the oracle: timed
 on one core and on all cores, and evaluating the per-solve error of the
@@ -41,9 +41,9 @@ METRIC = "operator applies/s & HBM GB/s; batched solves/s at resid 1e-8; p50/p99
 FP64_NOMINAL_TFLOPS = 1.25   # 2 FLOP x 2 FP64 lanes/clk/SM x 152 SMs x 2.06 GHz (context only)
 # DRAM bytes (read + write) of one block-MGS step at j = 15 on slab300: the
 # sum over its six launches in one ncu capture of `bench.py --probe bmgs
-# --probe-ns 300` (k_bdot 78.7 MB, 3 x k_bmgs<4,4> 146.7-147.0 MB,
-# k_bmgs<4,0> 78.7 MB, k_bscale 15.6 MB); retaken whenever these kernels change
-MGS_STEP_DRAM_BYTES = 613.3e6
+# --probe-ns 300` (profiles/bmgs_slab300.md); retaken whenever these kernels
+# change
+MGS_STEP_DRAM_BYTES = 610.2e6
 # GMRES restart length of the batched and served solves (local-Lambda, FP32
 # operator inside FP64 refinement).  The Arnoldi step's FP64 work grows with
 # the cycle length, the step count falls with it; on the 512-atmosphere batch
@@ -627,11 +627,12 @@ def main():
     fp64_tflops = peak64["tflops"] if peak64 else FP64_NOMINAL_TFLOPS
 
     # ---- dominant kernels of the step: the block-MGS Arnoldi orthogonalisation
-    # (k_bdot + 4 x k_bmgs + k_bscale of rt_arnoldi_bmgs), at the
-    # mean Arnoldi index j = 15 of a GMRES(30) cycle; the 17-vector basis
-    # (264 MB) is larger than L2.  FP64-pipe bound on this GPU: algorithmic
-    # work per step = the MGS loop's 2(j+1) FMA + 1 FMA (norm) + 1 multiply
-    # per element, 2 FLOP per FMA.
+    # (5 x k_pass + k_bscale of rt_arnoldi_bmgs), at the mean Arnoldi index
+    # j = 15 of a GMRES(30) cycle; the 17-vector basis (264 MB) is larger than
+    # L2.  Its dots run on the integer pipe beside the FP64 updates, so the step
+    # is bound by the bytes to the SMs; the algorithmic FP64 rate beside it
+    # counts the MGS loop's 2(j+1) FMA + 1 FMA (norm) + 1 multiply per element,
+    # 2 FLOP per FMA, whichever pipe runs them.
     jm = 15
     V = torch.randn((jm + 2) * N, dtype=torch.float64, device="cuda")
     w = torch.randn(N, dtype=torch.float64, device="cuda")
@@ -831,15 +832,14 @@ def main():
             "batched": batch,
             "served": served,
             "fp64_peak": peak64,
-            "roofline": {"kernel": "block-MGS Arnoldi step (k_bdot + 4 x k_bmgs + k_bscale, j=15)",
-                         "bound": "alu", "achieved": mgs_tflops, "peak": fp64_tflops, "unit": "TFLOP/s",
-                         "frac": mgs_tflops / fp64_tflops, "traffic": MGS_STEP_DRAM_BYTES,
-                         "peak_source": "measured: rt_probe_fp64_fma (FP64 FMA-only kernel, CUDA events)"
-                         if peak64 else "nominal 1.25 TFLOP/s (probe failed)",
-                         "hbm_gbs": mgs_gbs, "hbm_frac": mgs_gbs / hbm_peak,
-                         "note": "FP64-pipe bound; algorithmic FLOP per step (2(2(j+1)+1)+1)*N of the MGS loop; "
-                                 "hbm_gbs counts (2(j+1)+2*ceil((j+1)/4)+3)*N*8 bytes against the measured copy "
-                                 "bandwidth"},
+            "roofline": {"kernel": "block-MGS Arnoldi step (5 x k_pass + k_bscale, j=15)",
+                         "bound": "hbm", "achieved": mgs_gbs, "peak": hbm_peak, "unit": "GB/s",
+                         "frac": mgs_gbs / hbm_peak, "traffic": MGS_STEP_DRAM_BYTES,
+                         "peak_source": "measured copy bandwidth",
+                         "fp64_tflops": mgs_tflops, "fp64_frac": mgs_tflops / fp64_tflops,
+                         "note": "achieved counts (2(j+1)+2*ceil((j+1)/4)+3)*N*8 bytes; fp64_tflops the MGS loop's "
+                                 "(2(2(j+1)+1)+1)*N FLOP, half of which (the dots) run as integer digit products, "
+                                 "against the measured FP64 multiply-add rate"},
             "clocks": clk.summary(),
             "e2e": {"value": e2e_value, "unit": "applies/s", "h2d_bytes_per_step": N * 8,
                     "d2h_bytes_per_step": N * 8},

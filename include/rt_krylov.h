@@ -244,13 +244,13 @@ rt_status rt_precond_stationary(rt_problem* prob, int32_t kind, double omega, co
 rt_status rt_arnoldi_mgs(rt_problem* prob, double* V_dev, int32_t j, double* w_dev, double* h_dev, void* stream);
 
 /* One Arnoldi step by block modified Gram-Schmidt, the orthogonalisation
-   inside rt_solve_gmres (Sect. 2.1; the coefficients of rt_arnoldi_mgs in
-   exact arithmetic).  The basis is taken in blocks of RT_GRAM_BLOCK vectors:
+   inside rt_solve_gmres, there in larger blocks (Sect. 2.1; the coefficients
+   of rt_arnoldi_mgs in exact arithmetic).  The basis is taken in blocks of RT_GRAM_BLOCK vectors:
    with r_k = <w, v_k> formed before a block's updates, modified Gram-Schmidt
    gives h_k = r_k - sum_{l<k} h_l <v_l, v_k> (l, k in the block), so one pass
    over the data applies a whole block and forms the dots with the next one.
    The paper has no block form; it is a reformulation of its MGS loop with the
-   same FP64 operations per element and a quarter of the passes.
+   same updates per element and a quarter of the passes.
    gram_dev: (j+2) x RT_GRAM_BLOCK doubles; row i holds <v_i, v_{i-d}> in
    column d = 1..RT_GRAM_BLOCK-1 (column 0 unused).  Rows 1..j are read (all
    zero for an exactly orthonormal basis), each only in the columns whose

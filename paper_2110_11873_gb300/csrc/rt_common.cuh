@@ -270,8 +270,7 @@ struct BicgDev {
 enum CoefShare { CS_RAY = 0, CS_MU = 1, CS_PAIR = 2 };
 // Vector length from which a symmetric profile takes the paired FP64 kernels
 // (k_psweep, moments_pair64).  Above it the FP64 pipe bounds the apply and
-// sharing the work of a pair pays (N = 51.5 million: 621 -> 446 us with the
-// paired sweep alone); below, the quarter of the units is bound by latency
+// sharing the work of a pair pays (N = 51.5 million: 621 -> 425 us); below, the quarter of the units is bound by latency
 // (N = 47,040: 17.5 -> 18.2 us; N = 1.9 million: 38.9 -> 35.5 us, not worth
 // another rounding of the operator, which BiCGSTAB and CGS amplify).
 constexpr int64_t kPairMinN = (int64_t)4 << 20;

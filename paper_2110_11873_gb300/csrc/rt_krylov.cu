@@ -11,12 +11,14 @@
 //    device memory and are updated by one thread -- of a scalar kernel, or
 //    of a dedicated CTA of the kernel that needs them next (the Givens
 //    rotations run in a CTA of the scaling kernel, or of the next step's
-//    quadrature kernel) -- so a whole GMRES restart cycle (m Arnoldi steps,
-//    the least-squares solve, the update of x and the true residual) is one
-//    CUDA graph launch followed by one host read of the convergence state;
-//  * a step index baked into each kernel of the cycle graph is compared with
+//    quadrature kernel) -- so a GMRES restart cycle runs as CUDA graphs of
+//    kSegSteps Arnoldi steps and one for its end (the least-squares solve, the
+//    update of x and the true residual), the host reading the convergence
+//    state behind each and keeping one graph ahead of the device;
+//  * a step index baked into each kernel of a cycle's graphs is compared with
 //    the device counter `kstop`: once the residual estimate passes the
-//    tolerance the remaining kernels of the cycle return at once.
+//    tolerance the remaining kernels of the graph return at once, and the
+//    graphs after it are not launched.
 #include <math.h>
 #include <string.h>
 
@@ -227,8 +229,8 @@ __global__ void __launch_bounds__(kVecThreads) k_norm_out(const double* __restri
 }
 
 // ------------------------------------------------- block MGS Arnoldi step
-// The GMRES Arnoldi step orthogonalises w against v_0..v_j in passes of
-// kGramB basis vectors.  With r_k = <w, v_k> taken before a block's updates,
+// The Arnoldi step orthogonalises w against v_0..v_j in passes of B basis
+// vectors: kGramMax inside GMRES, kGramB in rt_arnoldi_bmgs.  With r_k = <w, v_k> taken before a block's updates,
 // modified Gram-Schmidt's coefficients satisfy exactly
 //     h_k = <w - sum_{l<k} h_l v_l, v_k> = r_k - sum_{l<k} h_l <v_l, v_k>
 // (l, k in the block), so each pass sums the previous pass's dots, solves
@@ -243,10 +245,13 @@ __global__ void __launch_bounds__(kVecThreads) k_norm_out(const double* __restri
 // last CTA folds h_{j+1,j} and the Gram row and rotates the Hessenberg
 // column.
 //
-// The FP64 pipe bounds these kernels, so the reductions are kept short: one
-// CTA per resident slot (a single wave, several elements per thread) and a
-// transposing warp reduction of the four accumulators (6 FP64 additions per
-// thread instead of 20).
+// Three forms of the step (mgs_plan, enqueue_bmgs): k_pass, the dots on the
+// integer pipe and the operands streamed by bulk copies; k_small_step, short
+// vectors in one CTA; and k_bdot / k_bmgs here, for vectors that a bulk copy
+// cannot start on.  The FP64 pipe bounds these last, so their reductions are
+// kept short: one CTA per resident slot (a single wave, several elements per
+// thread) and a transposing warp reduction of the four accumulators (6 FP64
+// additions per thread instead of 20).
 constexpr int kB = kGramB;
 // shape of the block-pass kernels: one wave of kMgsCtasPerSm CTAs of
 // kMgsThreads per SM (64 registers a thread)
@@ -516,7 +521,8 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_pass(double* __restrict__ w
 // the block passes, the normalisation, the Gram row and the Givens rotations,
 // with w in registers.  Kernel by kernel such a step is bound by launches, about
 // 4.5 us each whatever the length (sigma-form run of the paper, N = 280: 57 us
-// a step).  The same block MGS as k_pass with FP64 dots; every warp sums the
+// a step with three kernels here, 54 us with one; the operator's kernels are the
+// rest).  The same block MGS as k_pass with FP64 dots; every warp sums the
 // warps' partial dots and solves the block's triangular system for itself, so
 // a block needs one barrier.
 constexpr int kSmallThreads = 256;
@@ -1438,7 +1444,7 @@ static rt_status enqueue_cycle(Problem* P, int m, int precond, int fp32, int seg
     } else {
       RT_TRY(apply_prec(P, vj, w, precond, fp32, st, kstop, j));
     }
-    // block MGS: dots with the first block, one pass per block of kGramB
+    // block MGS: dots with the first block, one pass per block of gb
     // basis vectors (the last with ||w|| and the Gram dots of v_{j+1}), then
     // (unless fused) the normalisation with the Givens rotations of column j
     RT_TRY(enqueue_bmgs(P, P->V, w, j, &gm->H[j * (m + 1)], gm->gram, gb, gm, m, hist, hcap, kstop, st, !fuse, &pb,

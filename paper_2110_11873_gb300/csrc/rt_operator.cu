@@ -13,8 +13,9 @@
 //              CTA each, so they spread evenly over the SMs -- chain the maps
 //              of the tiles before their own (the slopes E are a setup
 //              table) and sweep their tile with the output.
-//   k_psweep   the same units where the profile is symmetric on the frequency
-//              grid: a lane marches the rays p and Nnu-1-p together.
+//   k_psweep   the same units on large problems whose profile is symmetric on
+//              the frequency grid: a lane marches the rays p and Nnu-1-p
+//              together, and the quadrature (moments_pair64) adds them first.
 //   k_formal   formal solver Lambda (Eq. 9-10) along every ray, writing
 //              y_k = z_k - I_k on the fly.  A CTA owns one group of 32 rays of
 //              the same direction sign (so the 32 lanes of a warp read one
