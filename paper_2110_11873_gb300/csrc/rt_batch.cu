@@ -236,7 +236,11 @@ __global__ void __launch_bounds__(32 * kFormalWarps) kb_formal(const InstDev* __
 // heights of a group, 32 atmospheres put 7 warps on an SM, each waiting on its
 // own recurrence: 276 us a launch.
 constexpr int kTiles32 = 8;
-constexpr int kRingB = 8;   // prefetch depth (steps)
+constexpr int kTileMin32 = 8;   // shortest tile (steps)
+// Prefetch depth (steps): 4 steps of two FP64 rows on 16 warps are 32 KB in
+// flight per SM, and the ring then fits two CTAs' registers.  8 steps took 164
+// registers, one CTA.
+constexpr int kRingB = 4;
 
 template <int FS, int MODE>
 __device__ __forceinline__ void formal_item32(const InstDev& I, int g, int src, int dst,
@@ -250,7 +254,7 @@ __device__ __forceinline__ void formal_item32(const InstDev& I, int g, int src, 
   const int64_t r = active ? base + lane : end - 1;
   const int m = (int)(r / I.Nnu);
   const int Ns = I.Ns;
-  const int T = max(1, min(kTiles32, (Ns - 1) / kRingB)), L = (Ns - 1 + T - 1) / T;
+  const int T = max(1, min(kTiles32, (Ns - 1) / kTileMin32)), L = (Ns - 1 + T - 1) / T;
   const int j0 = 1 + t * L, j1 = t < T ? min(Ns, j0 + L) : j0;
   float Iv[2] = {0.f, 0.f};
   if (t < T - 1 && j0 < j1) {
@@ -282,7 +286,7 @@ __device__ __forceinline__ void formal_item32(const InstDev& I, int g, int src, 
 }
 
 template <int FS, int MODE>
-__global__ void __launch_bounds__(32 * kTiles32) kb_formal32(const InstDev* __restrict__ insts,
+__global__ void __launch_bounds__(32 * kTiles32, 2) kb_formal32(const InstDev* __restrict__ insts,
                                                              const int4* __restrict__ wl, const Counts* cnt, int src,
                                                              int dst, int step) {
   __shared__ float sh[3][kTiles32][32];   // per tile: E, B of I, B of Q

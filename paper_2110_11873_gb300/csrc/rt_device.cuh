@@ -433,7 +433,11 @@ __device__ __forceinline__ void sweep(const FormalArgs& A, int s0, bool down, in
   TC gp = 0;
   if (PARA && j0 >= 2) gp = (TC)A.cg[(int64_t)interval(j0 - 1) * cstride + col];
   // register ring of the next RING steps
-  TC re[RING], ra[RING], rb[RING], rg[RING], rsv[RING][NS], rx[RING][NS], rd[RING][NS];
+  TC re[RING], ra[RING], rb[RING], rg[RING], rsv[RING][NS];
+  // as loaded: converted on loading, an FP64 vector made the FP32 solver wait
+  // for each load at once (32 atmospheres through the batch: 141 -> 125 ms)
+  TV rx[RING][NS];
+  double rd[RING][NS];
   if (PARA) {
 #pragma unroll
     for (int u = 0; u < RING; ++u)
@@ -457,8 +461,8 @@ __device__ __forceinline__ void sweep(const FormalArgs& A, int s0, bool down, in
         rsv[u][q] = Sm[q * sstride + (int64_t)k * A.Nmu];
         if (PHASE == 1 && MODE != KM_RHS) {
           const int64_t o = q * plane + (int64_t)k * nray + r;
-          rx[u][q] = vcast<TC>(x[o]);
-          if (MODE == KM_JACOBI) rd[u][q] = vcast<TC>(dinv[o]);
+          rx[u][q] = x[o];
+          if (MODE == KM_JACOBI) rd[u][q] = dinv[o];
         }
       }
     } else if (PARA && j == j1 && j < Ns) {
@@ -496,19 +500,19 @@ __device__ __forceinline__ void sweep(const FormalArgs& A, int s0, bool down, in
         // part of I_prev): x - (e (I_prev - gamma_prev S_k) + alpha S_prev + gamma S_next)
         if (PARA) {
           const TC t = fma(e, fma(-gp, sk, I[q]), fma(al, sp[q], rg[u] * rsv[(u + 1) % RING][q]));
-          if (active) y[q * plane + o] = vcast<TV>(rx[u][q] - t);
+          if (active) y[q * plane + o] = vcast<TV>(vcast<TC>(rx[u][q]) - t);
           I[q] = fma(fma(e, gp, be), sk, t);
         } else {
           const TC t = fma(e, I[q], al * sp[q]);
-          if (active) y[q * plane + o] = vcast<TV>(rx[u][q] - t);
+          if (active) y[q * plane + o] = vcast<TV>(vcast<TC>(rx[u][q]) - t);
           I[q] = fma(be, sk, t);
         }
       } else {
         I[q] = fma(e, I[q], fma(al, sp[q], cur));
         if (active) {
           if (MODE == KM_RHS) y[q * plane + o] = vcast<TV>(I[q]);
-          else if (MODE == KM_JACOBI) y[q * plane + o] = vcast<TV>(rx[u][q] * rd[u][q] - I[q]);
-          else y[q * plane + o] = vcast<TV>(rx[u][q] - I[q]);
+          else if (MODE == KM_JACOBI) y[q * plane + o] = vcast<TV>(vcast<TC>(rx[u][q]) * vcast<TC>(rd[u][q]) - I[q]);
+          else y[q * plane + o] = vcast<TV>(vcast<TC>(rx[u][q]) - I[q]);
         }
       }
       sp[q] = sk;
