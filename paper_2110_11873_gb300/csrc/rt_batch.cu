@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) kb_pass(const InstDev* __rest
 #pragma unroll
     for (int k = 0; k < NB; ++k) h[k] = hs[k];
     const int64_t lo = (int64_t)it.y * I.chunk;
-    FixDot<S::ND, S::NF> D;
+    PassDots<B, NB, NN> D;
     D.init();
     pass_consume<B, NB, NN>(R, I.w, lo, min(I.N, lo + I.chunk), 0, h, D);
     const double s = pass_block_dots(D.finish(), S::ND);

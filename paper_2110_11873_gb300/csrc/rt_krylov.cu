@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_pass(double* __restrict__ w
   double h[NB > 0 ? NB : 1];
 #pragma unroll
   for (int k = 0; k < NB; ++k) h[k] = hs[k];
-  FixDot<S::ND, S::NF> D;
+  PassDots<B, NB, NN> D;
   D.init();
   pass_consume<B, NB, NN>(R, w, lo, hi, rev, h, D);
   const double s = pass_block_dots(D.finish(), S::ND);

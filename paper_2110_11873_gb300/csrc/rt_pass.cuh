@@ -62,10 +62,15 @@ constexpr int kFxEpoch = 62;      // additions between two scalings: 62 products
 // values and are renewed when a value does not fit and after kFxEpoch
 // additions; at each renewal the warp's integer sums are folded exactly into
 // lane d's FP64 sum.  Infinities and NaN take the FP64 products.
-template <int ND, int NF>
+//
+// SQ: dot 0 is <w, w> (v[0] is not read), from the digits of w twice and with
+// w's scale twice.  What is left of w may be far smaller than the vectors v_d:
+// on their scale its square would keep none of its digits.
+template <int ND, int NF, bool SQ>
 struct FixDot {
   static_assert(NF >= 0 && NF < ND, "at least one dot in fixed point");
   static constexpr int NI = ND - NF;
+  static constexpr int D0 = SQ ? 1 : 0;   // first dot with a vector of its own
   long long hi[NI], mid[NI], low[NI];   // sums of the digit products a1 w1, a1 w0 + a0 w1, a0 w0
   double f[NF > 0 ? NF : 1];            // the lane's FP64 sums
   int Ew, Ev;
@@ -116,16 +121,17 @@ struct FixDot {
     // (t2 2^48 + t1 2^24 + t0 + f0 2^-24) 2^58 2^(Ev - 1079) 2^(Ew - 1079)
     const long long top = ((long long)t2 << 24) + t1, bot = ((long long)t0 << 24) + f0;
     const double v = fma((double)top, 16777216.0, (double)bot * 5.9604644775390625e-08);
-    if (lane < NI) acc += v * fx_pow2(Ev - 1050) * fx_pow2(Ew - 1050);
+    const int E = SQ && lane == 0 ? Ew : Ev;
+    if (lane < NI) acc += v * fx_pow2(E - 1050) * fx_pow2(Ew - 1050);
     clear();
   }
 
   // w: the lane's element of w; v[d]: its element of vector d
   __device__ __forceinline__ void add(double w, const double (&v)[ND]) {
     const int ew = fx_exp(w);
-    int ev = fx_exp(v[0]);
+    int ev = 0;
 #pragma unroll
-    for (int d = 1; d < NI; ++d) ev = max(ev, fx_exp(v[d]));
+    for (int d = D0; d < NI; ++d) ev = max(ev, fx_exp(v[d]));
 #pragma unroll
     for (int d = 0; d < NF; ++d) f[d] = fma(w, v[NI + d], f[d]);
     if (!__all_sync(0xffffffffu, left > 0 && ew <= Ew && ev <= Ev)) {   // new scales
@@ -140,7 +146,7 @@ struct FixDot {
         Ew = 0;
 #pragma unroll
         for (int d = 0; d < NI; ++d) {
-          const double t = fx_warp_sum(w * v[d]);
+          const double t = fx_warp_sum(w * (SQ && d == 0 ? w : v[d]));
           if ((int)(threadIdx.x & 31) == d) acc += t;
         }
         return;
@@ -149,8 +155,13 @@ struct FixDot {
     --left;
     int w1, w0;
     fx_digits(__double2hiint(w), __double2loint(w), Ew, w1, w0);
+    if (SQ) {
+      hi[0] += (long long)w1 * w1;
+      mid[0] += (long long)w1 * w0 * 2;
+      low[0] += (long long)w0 * w0;
+    }
 #pragma unroll
-    for (int d = 0; d < NI; ++d) {
+    for (int d = D0; d < NI; ++d) {
       int a1, a0;
       fx_digits(__double2hiint(v[d]), __double2loint(v[d]), Ev, a1, a0);
       hi[d] += (long long)a1 * w1;
@@ -195,6 +206,7 @@ struct PassShape {
   // they fill what the NB updates leave of it (the first kernel of a step,
   // with no update, ran at half the memory rate with all its dots in integers)
   static constexpr int NF = ND > NB ? (ND - NB) / 2 : 0;
+  static constexpr bool SQ = NN == 0;                          // dot 0 is ||w||^2
   static constexpr int NV = 1 + NB + NN;                       // vectors of a stage, w first
   static constexpr int STAGE = NV * kPassTile * (int)sizeof(double);
   static constexpr int NST = kPassSmem / STAGE < kPassMaxStages ? kPassSmem / STAGE : kPassMaxStages;
@@ -305,8 +317,10 @@ __device__ __forceinline__ void pass_produce(PassRing& R, const PassSrc& S0, int
 // consumer warps: the pass over [lo, hi); h: the block's coefficients; the
 // warp's dots are added to D
 template <int B, int NB, int NN>
+using PassDots = FixDot<PassShape<B, NB, NN>::ND, PassShape<B, NB, NN>::NF, PassShape<B, NB, NN>::SQ>;
+template <int B, int NB, int NN>
 __device__ __forceinline__ void pass_consume(PassRing& R, double* __restrict__ w, int64_t lo, int64_t hi, int rev,
-                                             const double* h, FixDot<PassShape<B, NB, NN>::ND, PassShape<B, NB, NN>::NF>& D) {
+                                             const double* h, PassDots<B, NB, NN>& D) {
   using S = PassShape<B, NB, NN>;
   const int nt = pass_tiles(lo, hi);
   const int t = threadIdx.x;
@@ -334,8 +348,7 @@ __device__ __forceinline__ void pass_consume(PassRing& R, double* __restrict__ w
     for (int k = 0; k < NB; ++k) wi = fma(-h[k], b[k], wi);
     if (NB > 0 && in) w[e0 + t] = wi;
     wi = in ? wi : 0.0;
-    if (NN == 0) {
-      v[0] = wi;
+    if (NN == 0) {   // v[0] stands for w itself
 #pragma unroll
       for (int k = 0; k < S::NG; ++k) v[1 + k] = b[k];
     }

@@ -121,3 +121,59 @@ def test_gmres_blocks_of_eight(form):
         r = b - P.apply(x)
         rel = float(torch.linalg.vector_norm(r) / torch.linalg.vector_norm(b))
         assert abs(rel - info.err_est) <= 1e-11 + 1e-8 * info.err_est, (m, rel, info)
+
+
+def _basis(N, j, rng):
+    Q = []
+    for _ in range(j + 1):
+        v = rng.standard_normal(N)
+        for _ in range(2):
+            for u in Q:
+                v = v - np.dot(u, v) * u
+        Q.append(v / np.linalg.norm(v))
+    return Q
+
+
+def _normalised(P, N, j, Q, w0):
+    """h_{j+1} and v_{j+1} of one step against the w that the step left."""
+    gram = np.zeros((j + 2, 4))
+    for i in range(1, j + 1):
+        for d in range(1, min(i, 3) + 1):
+            gram[i, d] = Q[i] @ Q[i - d]
+    Vd = torch.zeros((j + 2) * N, dtype=torch.float64, device="cuda")
+    Vd[: (j + 1) * N] = to_dev(np.concatenate(Q))
+    wd = to_dev(w0)
+    h = to_host(P.arnoldi_bmgs(Vd, j, wd, to_dev(gram.reshape(-1))))
+    P.check()
+    w = to_host(wd)
+    big = np.abs(w).max()
+    left = big * np.linalg.norm(w / big)   # |w| without underflow of its square
+    v = to_host(Vd)[(j + 1) * N:]
+    return h[-1] / left - 1.0, np.linalg.norm(v) - 1.0
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-4, 1e-8, 1e-12, 1e-18, 1e-100])
+@pytest.mark.parametrize("j", range(8))
+def test_pass_norm_of_small_w(scale, j):
+    """h_{j+1} and v_{j+1} have the accuracy of FP64 relative to what is left of
+    w, whatever its size beside the unit basis.  Both sides sum N squares in
+    trees and chains of length < 1000: 1e-13 of the sum, half of it of its root;
+    the scaling of v adds three roundings."""
+    P = problem(W.slab(100, 8, 41, 1e-4, 1e6, 6.0))
+    rng = np.random.default_rng(j)
+    Q = _basis(P.N, j, rng)
+    dh, dv = _normalised(P, P.N, j, Q, scale * rng.standard_normal(P.N))
+    assert abs(dh) < 2e-13 and abs(dv) < 2e-13, (dh, dv)
+
+
+@pytest.mark.parametrize("left", [1e-6, 1e-10, 1e-14])
+@pytest.mark.parametrize("j", [0, 2, 5])
+def test_pass_norm_of_a_dependent_w(left, j):
+    """A w almost in the span of the basis: the same for what is left of it."""
+    P = problem(W.slab(100, 8, 41, 1e-4, 1e6, 6.0))
+    rng = np.random.default_rng(10 + j)
+    Q = _basis(P.N, j, rng)
+    r = rng.standard_normal(P.N)
+    w0 = sum(c * q for c, q in zip(rng.standard_normal(j + 1), Q)) + left * r / np.linalg.norm(r)
+    dh, dv = _normalised(P, P.N, j, Q, w0)
+    assert abs(dh) < 2e-13 and abs(dv) < 2e-13, (dh, dv)
