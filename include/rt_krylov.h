@@ -184,8 +184,10 @@ rt_status rt_apply_f32(rt_problem* prob, const float* x_dev, float* y_dev, void*
 /* Synchronises `stream` and reports RT_ETIMEOUT (then clears the condition)
    when a bounded device-side wait of this problem's kernels gave up since the
    last check; RT_OK otherwise.  The paper has no counterpart: it guards this
-   library's asynchronous copies.  rt_solve_gmres performs the same check
-   before it returns. */
+   library's asynchronous copies, which rt_apply_f32 and rt_arnoldi_bmgs make;
+   those calls only enqueue work, so a caller that wants to know asks here.
+   rt_solve_gmres performs the same check before it returns, and a request of
+   the batch server whose wait gave up ends with RT_ETIMEOUT. */
 rt_status rt_problem_check(rt_problem* prob, void* stream);
 
 /* Which formal-solver kernel the FP32 applies of this problem use (no
@@ -199,6 +201,10 @@ int rt_problem_formal_kernel(const rt_problem* prob);
    kernel treat the first wait of one warp as given up -- that warp flags the
    problem, waits (bounded) for its copies in flight and skips its depth
    tile, so y is invalid and the next rt_problem_check returns RT_ETIMEOUT.
+   Calls of rt_arnoldi_bmgs that stream their operands (more than 1024
+   unknowns, V_dev and w_dev 16-byte aligned) count as well: one block of
+   threads goes on without its copies, which still land before it ends, and
+   what the step wrote is invalid.
    count = 0 disarms it.  RT_EINVAL for NULL or count < 0.  Host only. */
 rt_status rt_problem_inject_wait_timeout(rt_problem* prob, int32_t count);
 
@@ -257,7 +263,8 @@ rt_status rt_arnoldi_mgs(rt_problem* prob, double* V_dev, int32_t j, double* w_d
    vectors share its block (d <= i mod RT_GRAM_BLOCK).  For the new vector,
    row j+1 gets exactly those columns, d = 1..(j+1) mod RT_GRAM_BLOCK; its
    other columns are left as they are.  V_dev, w_dev, h_dev and the limits
-   as rt_arnoldi_mgs. */
+   as rt_arnoldi_mgs.  The copies it makes are waited for with a bound:
+   rt_problem_check reports one that gave up. */
 #define RT_GRAM_BLOCK 4
 rt_status rt_arnoldi_bmgs(rt_problem* prob, double* V_dev, int32_t j, double* w_dev, double* gram_dev,
                           double* h_dev, void* stream);

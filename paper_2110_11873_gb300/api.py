@@ -278,8 +278,9 @@ class Problem:
         return self.lib.rt_problem_formal_kernel(self.handle) == 1
 
     def inject_wait_timeout(self, count: int = 1) -> None:
-        """Arm the next `count` tensor-copy FP32 applies to give up one wait
-        (failure injection; the following check() raises RT_ETIMEOUT)."""
+        """Arm the next `count` tensor-copy FP32 applies or streamed Arnoldi
+        steps (arnoldi_bmgs) to give up one wait (failure injection; the
+        following check() raises RT_ETIMEOUT)."""
         N.check(self.lib.rt_problem_inject_wait_timeout(self.handle, int(count)), "rt_problem_inject_wait_timeout")
 
     def check(self, stream=None) -> None:
@@ -333,7 +334,8 @@ class Problem:
                      h: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         """One block-MGS Arnoldi step (the GMRES orthogonalisation): as
         arnoldi_mgs, with gram ((j+2) x 4 doubles, rows 1..j read, row j+1
-        written) holding <v_i, v_{i-d}>, d = 1..3."""
+        written) holding <v_i, v_{i-d}>, d = 1..3.  Enqueued only: check()
+        reports a copy of its operands that did not arrive in time."""
         if V.dtype != torch.float64 or not V.is_contiguous() or V.numel() < (j + 2) * self.N:
             raise ValueError("V must be a contiguous float64 tensor of at least (j+2)*N values")
         if gram.dtype != torch.float64 or not gram.is_contiguous() or gram.numel() < (j + 2) * 4:

@@ -337,14 +337,16 @@ __global__ void __launch_bounds__(kPassThreads, 2) kb_pass(const InstDev* __rest
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == kPassWarps) {   // producer
     asm volatile("fence.proxy.async;" ::: "memory");   // the previous kernels' stores, before the copies
-    for (int q = w0; q < w1; ++q) {
+    bool ok = true;
+    for (int q = w0; ok && q < w1; ++q) {
       const int2 it = wl[q];
       const InstDev& I = insts[it.x];
       if (step_gated(I, j)) continue;
       const PassSrc src = pass_src<B, NB, NN>(I.w, I.V + (int64_t)i0 * I.N, I.V + (int64_t)(i0 + NB) * I.N, I.N);
       const int64_t lo = (int64_t)it.y * I.chunk;
-      pass_produce<B, NB, NN>(R, src, lo, min(I.N, lo + I.chunk), 0, 0);
+      ok = pass_produce<B, NB, NN>(R, src, lo, min(I.N, lo + I.chunk), 0, 0);
     }
+    pass_drain(R, S::NST);
     return;
   }
   int have = -1;

@@ -385,8 +385,8 @@ struct Problem {
   int* dev_err = nullptr;
   float* tile_dt = nullptr;    // [2][ntile_st] DELO-linear: the sum of dtau / ln 2 over each depth tile
   void* tma_cache = nullptr;   // host: recently encoded tensor maps of the FP32 apply (rt_tma.cu)
-  int inject_wait_fail = 0;    // standalone FP32 applies still to run with one tensor-copy wait forced to
-                               // give up (failure injection, rt_problem_inject_wait_timeout)
+  int inject_wait_fail = 0;    // standalone FP32 applies and Arnoldi steps still to run with one copy's wait
+                               // forced to give up (failure injection, rt_problem_inject_wait_timeout)
 };
 
 // operator entry points used by the solvers (all enqueue on `st`)

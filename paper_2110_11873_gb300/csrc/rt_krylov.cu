@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_pass(double* __restrict__ w
                                                           int64_t N, int i0, const double* __restrict__ part_in,
                                                           double* __restrict__ part_out, double* __restrict__ hcol,
                                                           const double* __restrict__ gram, int j, int rev,
-                                                          const int* kstop, int* err) {
+                                                          const int* kstop, int* err, int fail_wait) {
   using S = PassShape<B, NB, NN>;
   static_assert(kPassWarps >= B && kPassTile >= B * B, "one warp per set of partials");
   if (kstop && j >= *kstop) return;
@@ -477,6 +477,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_pass(double* __restrict__ w
       }
     }
     pass_produce<B, NB, NN>(R, src, lo, hi, rev, early);
+    pass_drain(R, S::NST);
     return;
   }
   if (NB > 0 && threadIdx.x < B * B) {   // the block's Gram entries <v_{i0+k-d}, v_{i0+k}>
@@ -511,6 +512,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_pass(double* __restrict__ w
   for (int k = 0; k < NB; ++k) h[k] = hs[k];
   PassDots<B, NB, NN> D;
   D.init();
+  if (fail_wait && blockIdx.x == 0 && threadIdx.x == 0) dead = 1;   // injected: a wait gave up
   pass_consume<B, NB, NN>(R, w, lo, hi, rev, h, D);
   const double s = pass_block_dots(D.finish(), S::ND);
   if ((int)threadIdx.x < S::ND) part_out[(size_t)threadIdx.x * G + blockIdx.x] = s;
@@ -1125,7 +1127,7 @@ struct Workspace {
 };
 
 using PassFn = void (*)(double*, const double*, int64_t, int, const double*, double*, double*, const double*, int, int,
-                        const int*, int*);
+                        const int*, int*, int);
 // the passes of blocks of B vectors: first dots with n + 1 vectors, a full
 // block with n + 1 look-ahead dots, a last block of n + 1 vectors
 template <int B>
@@ -1259,11 +1261,11 @@ static rt_status add_precond(Problem* P, double* x, double* t, int precond, doub
 template <int B>
 static rt_status enqueue_passes(Problem* P, const PassTable<B>& T, const double* V, double* w, int Gm, int j,
                                 double* hcol, const double* gram, const int* kstop, cudaStream_t st, int* pb, int* ng,
-                                int* rev) {
+                                int* rev, int fail_wait) {
   const int64_t N = P->Nop;
   RT_TRY_CUDA(launch_pdl_smem(T.dot[std::min(B, j + 1) - 1], Gm, kPassThreads, kPassDynSmem, st, w, V, N, 0,
                               (const double*)nullptr, bpartb(P, 0), (double*)nullptr, (const double*)nullptr, j, *rev,
-                              kstop, P->dev_err)); RT_COUNT(1);
+                              kstop, P->dev_err, fail_wait)); RT_COUNT(1);
   for (int i0 = 0; i0 <= j; i0 += B) {
     const int nb = std::min(B, j + 1 - i0);
     const int nn = std::max(0, std::min(B, j + 1 - (i0 + nb)));
@@ -1271,7 +1273,7 @@ static rt_status enqueue_passes(Problem* P, const PassTable<B>& T, const double*
     *rev ^= 1;
     RT_TRY_CUDA(launch_pdl_smem(nn ? T.mid[nn - 1] : T.last[nb - 1], Gm, kPassThreads, kPassDynSmem, st, w, V, N, i0,
                                 (const double*)bpartb(P, *pb), bpartb(P, *pb ^ 1), hcol, gram, j, *rev, kstop,
-                                P->dev_err)); RT_COUNT(1);
+                                P->dev_err, 0)); RT_COUNT(1);
     *pb ^= 1;
   }
   return RT_OK;
@@ -1279,7 +1281,7 @@ static rt_status enqueue_passes(Problem* P, const PassTable<B>& T, const double*
 
 static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* hcol, double* gram, int gb,
                               GmresDev* gm, int m, double* hist, int hcap, const int* kstop, cudaStream_t st, bool scale = true,
-                              int* pb_out = nullptr, int* ng_out = nullptr) {
+                              int* pb_out = nullptr, int* ng_out = nullptr, int fail_wait = 0) {
   const MgsPlan plan = mgs_plan(P, V, w);
   const int Gm = plan.grid;
   const int64_t N = P->Nop;
@@ -1290,8 +1292,8 @@ static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* h
     return RT_OK;
   }
   if (plan.fixed) {
-    if (gb == kGramB) RT_TRY(enqueue_passes(P, g_pass4, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev));
-    else RT_TRY(enqueue_passes(P, g_pass8, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev));
+    if (gb == kGramB) RT_TRY(enqueue_passes(P, g_pass4, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev, fail_wait));
+    else RT_TRY(enqueue_passes(P, g_pass8, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev, fail_wait));
   } else {
     using BdotFn = void (*)(const double*, const double*, int64_t, double*, int, int, const int*);
     using BmgsFn = void (*)(double*, const double*, int64_t, int, const double*, double*, double*, const double*, int,
@@ -2251,7 +2253,13 @@ rt_status rt_arnoldi_bmgs(rt_problem* prob, double* V_dev, int32_t j, double* w_
   int* always = reinterpret_cast<int*>(&P->gm->kstop);   // a gate that never stops the kernels
   const int big = 1 << 30;
   RT_TRY_CUDA(cudaMemcpyAsync(always, &big, sizeof(int), cudaMemcpyHostToDevice, st));
-  return enqueue_bmgs(P, V_dev, w_dev, j, h_dev, gram_dev, kGramB, nullptr, 0, nullptr, 0, always, st);
+  int fail = 0;
+  if (P->inject_wait_fail > 0 && P->Nop > kSmallN && mgs_plan(P, V_dev, w_dev).fixed) {   // one armed injection
+    fail = 1;
+    P->inject_wait_fail -= 1;
+  }
+  return enqueue_bmgs(P, V_dev, w_dev, j, h_dev, gram_dev, kGramB, nullptr, 0, nullptr, 0, always, st, true, nullptr,
+                      nullptr, fail);
 }
 
 rt_status rt_solve_gmres(rt_problem* prob, const rt_solver_opts* opts, const double* b_dev, double* x_dev,

@@ -291,27 +291,36 @@ __device__ __forceinline__ void pass_issue(const PassRing& R, unsigned slot, con
               S0.policy);
 }
 
-// producer warp: the tiles of [lo, hi) from tile `from` on
+// producer warp: the tiles of [lo, hi) from tile `from` on; false once a wait
+// gave up (nothing more is copied then).  R.used counts the tiles issued.
 template <int B, int NB, int NN>
-__device__ __forceinline__ void pass_produce(PassRing& R, const PassSrc& S0, int64_t lo, int64_t hi, int rev,
+__device__ __forceinline__ bool pass_produce(PassRing& R, const PassSrc& S0, int64_t lo, int64_t hi, int rev,
                                              int from) {
   using S = PassShape<B, NB, NN>;
   const int nt = pass_tiles(lo, hi);
-  for (int q = from; q < nt; ++q) {
+  int q = from;
+  for (; q < nt; ++q) {
     const unsigned u = R.used + q, slot = u % S::NST;
     if (u >= (unsigned)S::NST) pass_wait(R, &R.empty[slot], (u / S::NST - 1) & 1);
-    if (__any_sync(0xffffffffu, *R.dead)) {
-      // the copies in flight land before the CTA leaves (bounded)
-      for (unsigned p = u < (unsigned)S::NST ? 0 : u - S::NST; p < u; ++p)
-        mbar_wait(&R.full[p % S::NST], (p / S::NST) & 1);
-      break;
-    }
+    if (__any_sync(0xffffffffu, *R.dead)) break;
     int64_t e0;
     int cnt;
     pass_tile(lo, hi, q, nt, rev, e0, cnt);
     pass_issue<B, NB, NN>(R, slot, S0, e0, cnt, true, true);
   }
-  R.used += nt;
+  R.used += q;
+  return q == nt;
+}
+
+// producer warp, before it leaves: the copies it issued land (one bound for
+// all of them).  The consumers take every tile, but one that gave up a wait
+// goes on without the copies, and none may write the CTA's shared memory after
+// its end.
+__device__ __forceinline__ void pass_drain(const PassRing& R, unsigned nst) {
+  const unsigned long long t0 = gtimer();
+  for (unsigned p = R.used > nst ? R.used - nst : 0; p < R.used; ++p)
+    while (!mbar_try_wait(&R.full[p % nst], (p / nst) & 1))
+      if (gtimer() - t0 > kWaitNs) return;
 }
 
 // consumer warps: the pass over [lo, hi); h: the block's coefficients; the

@@ -1046,7 +1046,7 @@ rt_status check_device_flag(Problem* P, cudaStream_t st) {
   if (!h) return RT_OK;
   RT_TRY_CUDA(cudaMemsetAsync(P->dev_err, 0, sizeof(int), st));
   RT_TRY_CUDA(cudaStreamSynchronize(st));
-  set_error("a device-side wait for a tensor copy gave up; results of the affected applies are invalid");
+  set_error("a device-side wait for a copy into shared memory gave up; what the calls since the last check wrote is invalid");
   return RT_ETIMEOUT;
 }
 

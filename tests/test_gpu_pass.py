@@ -177,3 +177,29 @@ def test_pass_norm_of_a_dependent_w(left, j):
     w0 = sum(c * q for c, q in zip(rng.standard_normal(j + 1), Q)) + left * r / np.linalg.norm(r)
     dh, dv = _normalised(P, P.N, j, Q, w0)
     assert abs(dh) < 2e-13 and abs(dv) < 2e-13, (dh, dv)
+
+
+def test_a_copy_that_does_not_arrive_reports_timeout_and_the_problem_recovers():
+    """Failure path of the streamed passes' bounded waits, without a device
+    fault: in an armed step one CTA goes on without its copies (they land
+    before it ends).  The next check reports RT_ETIMEOUT once; later steps are
+    right again.  A step in the register kernels (8-byte aligned operands) takes
+    no armed injection."""
+    from paper_2110_11873_gb300 import _native as N
+
+    for Ns, Nmu, Nnu in ((70, 16, 21), (300, 32, 101)):   # one tile per CTA; more tiles than stages
+        P = problem(W.slab(Ns, Nmu, Nnu, 1e-4, 1e6, 6.0))
+        V = torch.zeros(3 * P.N + 2, dtype=torch.float64, device="cuda")
+        gram = torch.zeros(12, dtype=torch.float64, device="cuda")
+        for armed in (1, 2):
+            P.inject_wait_timeout(armed)
+            for _ in range(armed):
+                P.arnoldi_bmgs(V, 0, torch.ones(P.N, dtype=torch.float64, device="cuda"), gram)
+            with pytest.raises(N.RTError) as ei:
+                P.check()
+            assert ei.value.status == N.RT_ETIMEOUT
+            P.check()   # the condition was cleared by the check that reported it
+            _step(P, P.N, 2, "normal", seed=armed)
+        P.inject_wait_timeout(1)
+        _step(P, P.N, 2, "normal", offset=1)
+        P.inject_wait_timeout(0)
