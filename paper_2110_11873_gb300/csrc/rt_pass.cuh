@@ -34,9 +34,12 @@ __device__ __forceinline__ void fx_digits(uint32_t hi, uint32_t lo, int E, int& 
   const int sh = min(E + 4 - (int)((hi >> 20) & 0x7ff), 63);   // what is left past 2^-63 rounds to 0 below
   const uint64_t M = ((uint64_t)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (uint32_t)(lo << 11);
   const uint64_t G = M >> sh;   // |x| with its leading bit at 2^59 for exponent E
+  // half a unit added to what is left of |x|; for a negative x the complement
+  // (one less than -G) puts what the shift dropped on the right side of the
+  // half, so that neither sign is rounded towards zero more often
   const uint32_t sg = (uint32_t)((int)hi >> 31);
   const uint64_t s64 = ((uint64_t)sg << 32) | sg;
-  const uint64_t g = (G ^ s64) - s64 + 4;
+  const uint64_t g = (G ^ s64) + 4;
   a0 = (int)(uint32_t)g >> 3;
   a1 = (int)(g >> 32) + (int)((uint32_t)g >> 31);
 }

@@ -203,3 +203,26 @@ def test_a_copy_that_does_not_arrive_reports_timeout_and_the_problem_recovers():
         P.inject_wait_timeout(1)
         _step(P, P.N, 2, "normal", offset=1)
         P.inject_wait_timeout(0)
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_pass_digits_round_without_a_sign(sign):
+    """Entries of one sign beside large ones that the basis vector does not
+    meet (2^20, one to every 32 elements): the fixed-point unit is 2^-34 (two
+    bits of headroom, 54 below), each entry of 1..2 is rounded to it, and the
+    rounding errors average out: 0.29 units each, 0.29 * 2^-34 / sqrt(N) / 1.5
+    of the dot on the mean, 4.4e-14 for N = 65,600; six times that is allowed.
+    An eighth of a unit in one direction would be 5e-12."""
+    P = problem(W.slab(100, 8, 41, 1e-4, 1e6, 6.0))
+    N = P.N
+    rng = np.random.default_rng(5)
+    w0 = sign * rng.uniform(1.0, 2.0, N)
+    v = rng.uniform(0.5, 1.0, N)
+    w0[::32] = 2.0 ** 20
+    v[::32] = 0.0
+    v /= np.linalg.norm(v)
+    V = torch.zeros(2 * N, dtype=torch.float64, device="cuda")
+    V[:N] = to_dev(v)
+    h = to_host(P.arnoldi_bmgs(V, 0, to_dev(w0), torch.zeros(8, dtype=torch.float64, device="cuda")))
+    exact = float(np.sum(w0.astype(np.longdouble) * v.astype(np.longdouble)))
+    assert abs(h[0] / exact - 1.0) < 2.7e-13, h[0] / exact - 1.0
