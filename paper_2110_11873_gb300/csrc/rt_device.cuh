@@ -8,7 +8,8 @@
 namespace rt {
 namespace {
 
-constexpr int kMomThreads = 256;      // threads of the FP32 quadrature (and of the batch's)
+constexpr int kMomThreads = 256;      // threads of the batch's quadratures and the FP32 one on many heights
+constexpr int kMom32Threads = 512;    // threads of the FP32 quadrature on few heights
 constexpr int kMaxTiles = 8;     // FP32 kernel: up to 256 threads per CTA (255 registers a lane)
 constexpr int kMaxTilesRay = 16; // FP64 formal solver on rays: depth tiles per ray group (one warp each)
 constexpr int kMaxTiles64 = 32;  // FP64 formal solver on pairs of rays: the same
@@ -89,27 +90,27 @@ __device__ __forceinline__ double beta_star(const double* __restrict__ cb, int k
 // MODE: KM_PLAIN z = x; KM_JACOBI z = x * dinv; KM_LOCAL_LAMBDA z = x and
 // sigma_k <- M_k^{-1} sigma_k.
 
-// FP32 quadrature of height k by the whole block (kMomThreads threads) as
-// flat dot products over its rays, with the per-ray weights w0 = hat-w_m
+// FP32 quadrature of height k by the whole block (THREADS threads) as flat dot
+// products over its rays, with the per-ray weights w0 = hat-w_m
 // hat-w_p, w1 = w0 T201_m, w2 = w0 T202_m (wray, [3][nray]):
 //     J00 = sum_r w0 I_r,   J20 = sum_r (w1 I_r + w2 Q_r).
 // NORM: the input is x * inv, written to xout in the input's precision as
 // each element is read (the GMRES normalisation of the batched solver).  A
 // warp per direction row, as before, left lanes idle on short rows and half
 // of its loads predicated off (32 uneven atmospheres: 139 us a launch).
-template <typename TI, int MODE, bool NORM = false>
+template <typename TI, int MODE, int THREADS, bool NORM = false>
 __device__ __forceinline__ void moments_flat32(const TI* __restrict__ x, const double* __restrict__ dinv,
                                                const float* __restrict__ wray, const float* __restrict__ t201,
                                                const float* __restrict__ t202, const double* __restrict__ Minv,
                                                int Ns, int Nmu, int64_t nray, float xi, float xiW2,
                                                float* __restrict__ S, int k, double inv = 1.0,
                                                TI* __restrict__ xout = nullptr) {
-  constexpr int nw = kMomThreads / 32;
+  constexpr int nw = THREADS / 32;
   const int64_t oI = (int64_t)k * nray, oQ = ((int64_t)Ns + k) * nray;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float a0 = 0.f, a1 = 0.f;
 #pragma unroll 4
-  for (int64_t r = threadIdx.x; r < nray; r += kMomThreads) {
+  for (int64_t r = threadIdx.x; r < nray; r += THREADS) {
     TI xI = x[oI + r], xQ = x[oQ + r];
     if (NORM) {
       xI = (TI)(xI * inv);

@@ -224,14 +224,21 @@ __global__ void k_add_local(const double* __restrict__ v, const double* __restri
 }
 
 
-template <typename TI, int MODE>
-__global__ void __launch_bounds__(kMomThreads) k_moments(
+// FP32 quadrature, one CTA per height.  Bound by the loads in flight, which a
+// few CTAs an SM of 256 threads leave short: up to kMom32Heights heights per SM
+// a CTA has 512 threads.  Apply with 256 and 512 of them, trapezoidal: N_s = 100
+// heights of 62 x 201 rays 31.3 and 27.3 us, 316 of 58 x 138 57.2 and 50.5 us,
+// 466 of 58 x 138 70.8 and 63.7 us; but 1000 of 30 x 101 67.1 and 69.0 us, 2000
+// of 30 x 51 113.2 and 116.8 us.
+constexpr int kMom32Heights = 4;
+template <typename TI, int MODE, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_moments(
     const TI* __restrict__ x, const double* __restrict__ dinv, const float* __restrict__ wray,
     const float* __restrict__ t201, const float* __restrict__ t202, const double* __restrict__ Minv, int Ns, int Nmu,
     int64_t nray, float xi, float xiW2, float* __restrict__ S, const int* kstop, int step) {
   pdl_wait();
   if (kstop && step >= *kstop) return;
-  moments_flat32<TI, MODE>(x, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
+  moments_flat32<TI, MODE, THREADS>(x, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
 }
 
 // FP64 quadrature, one CTA per height (flat over the rays); WJ: Jacobi mode
@@ -1060,6 +1067,18 @@ rt_status op_apply64(Problem* P, const double* x, double* y, int mode, cudaStrea
   return RT_OK;
 }
 
+// the quadrature as in op_apply64: a programmatic dependent of whatever ran before
+template <typename TV, int MODE>
+static cudaError_t launch_moments32(const Problem* P, const TV* x, const double* dinv, const double* Minv,
+                                    cudaStream_t st, const int* kstop, int step) {
+  const bool few = P->Ns <= kMom32Heights * P->num_sms;
+  RT_COUNT(1);
+  return launch_pdl(few ? k_moments<TV, MODE, kMom32Threads> : k_moments<TV, MODE, kMomThreads>, P->Ns,
+                    few ? kMom32Threads : kMomThreads, st, x, dinv, (const float*)P->wray32, (const float*)P->t201f,
+                    (const float*)P->t202f, Minv, P->Ns, P->Nmu, P->nray, (float)P->xi, (float)(P->xi * P->W2),
+                    P->S32, kstop, step);
+}
+
 template <typename TV>
 static rt_status apply32_impl(Problem* P, const TV* x, TV* y, int mode, cudaStream_t st, const int* kstop, int step,
                               const NormIn* nin = nullptr) {
@@ -1082,24 +1101,17 @@ static rt_status apply32_impl(Problem* P, const TV* x, TV* y, int mode, cudaStre
     set_error("internal: the fused GMRES normalisation needs the staged FP32 apply");
     return RT_EINVAL;
   }
-  const float xi = (float)P->xi, xiW2 = (float)(P->xi * P->W2);
-  const int Ns = P->Ns, Nmu = P->Nmu;
-  auto moments = [&](auto kernel, const double* dinv, const double* Minv) {   // as in op_apply64
-    RT_COUNT(1);
-    return launch_pdl(kernel, Ns, kMomThreads, st, x, dinv, (const float*)P->wray32, (const float*)P->t201f,
-                      (const float*)P->t202f, Minv, Ns, Nmu, P->nray, xi, xiW2, P->S32, kstop, step);
-  };
   switch (mode) {
     case AM_PLAIN:
-      RT_TRY_CUDA(moments(k_moments<TV, KM_PLAIN>, nullptr, nullptr));
+      RT_TRY_CUDA((launch_moments32<TV, KM_PLAIN>(P, x, nullptr, nullptr, st, kstop, step)));
       launch_formal32<TV, KM_PLAIN>(P, x, y, st, kstop, step);
       break;
     case AM_JACOBI:
-      RT_TRY_CUDA(moments(k_moments<TV, KM_JACOBI>, P->dinv, nullptr));
+      RT_TRY_CUDA((launch_moments32<TV, KM_JACOBI>(P, x, P->dinv, nullptr, st, kstop, step)));
       launch_formal32<TV, KM_JACOBI>(P, x, y, st, kstop, step);
       break;
     case AM_LOCAL_LAMBDA:
-      RT_TRY_CUDA(moments(k_moments<TV, KM_LOCAL_LAMBDA>, nullptr, P->Minv));
+      RT_TRY_CUDA((launch_moments32<TV, KM_LOCAL_LAMBDA>(P, x, nullptr, P->Minv, st, kstop, step)));
       launch_formal32<TV, KM_LOCAL_LAMBDA>(P, x, y, st, kstop, step);
       break;
     default:
