@@ -14,7 +14,9 @@ constexpr int kMaxTiles = 8;     // FP32 kernel: up to 256 threads per CTA (255 
 constexpr int kMaxTilesRay = 16; // FP64 formal solver on rays: depth tiles per ray group (one warp each)
 constexpr int kMaxTiles64 = 32;  // FP64 formal solver on pairs of rays: the same
 constexpr int kRing = 8;         // prefetch depth of the FP64 formal-solver kernel (steps)
-constexpr int kRing32 = 16;      // prefetch depth of the FP32 kernel (one lane carries I and Q)
+constexpr int kRing32 = 8;       // the same of the FP32 kernel (one lane carries I and Q), FP32 vectors
+constexpr int kRing32D = 4;      // ... and FP64 vectors
+constexpr int kMinSteps32 = 32;  // shortest depth tile of the FP32 kernel (steps)
 
 enum KMode { KM_PLAIN = 0, KM_JACOBI = 1, KM_LOCAL_LAMBDA = 2, KM_RHS = 3 };
 

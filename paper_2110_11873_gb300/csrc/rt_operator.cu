@@ -294,8 +294,13 @@ __global__ void k_jacobi_weights(const double* __restrict__ wray, const double* 
 // grid: NSPLIT * ngroups CTAs (ray group g, and with NSPLIT = 2 the Stokes
 // parameter s = blockIdx.x % 2 -- with NSPLIT = 1 one lane carries I and Q);
 // block: 32 * ntile threads (warp t = depth tile t)
+//
+// Two CTAs to an SM (128 registers a lane): with a ring of 16 steps, which FP64
+// vectors hold unconverted, a lane took 138 to 226 registers, so that more ray
+// groups than SMs ran in two waves and fewer had half the warps to hide their
+// recurrences.
 template <typename TC, typename TV, int FS, int MODE, int NSPLIT, int RING, int MAXT>
-__global__ void __launch_bounds__(32 * MAXT) k_formal(const FormalArgs A) {
+__global__ void __launch_bounds__(32 * MAXT, 2) k_formal(const FormalArgs A) {
   constexpr int NS = 2 / NSPLIT;   // Stokes parameters per lane
   pdl_wait();   // the source values of the quadrature before
   if (A.kstop && A.step >= *A.kstop) return;
@@ -458,7 +463,7 @@ static rt_status upload(Problem* P, T** dst, const std::vector<T>& src, cudaStre
 // (kPairResident per SM); N_s = 2000, N_mu = 64, N_nu = 201 took 616, 596, 485,
 // 450 and 446 us per apply with 3, 4, 6, 9 and 12 tiles, N_s = 500 170, 140, 133
 // and 131 us with 3, 6, 9 and 12.  FP32: tiles are cheap, so aim
-// at about 16 warps per SM with tiles of at least 2*kRing steps.
+// at about 8 warps per SM with tiles of at least kMinSteps32 steps.
 constexpr double kFp64OpCycles = 20.0, kFp64StepCycles = 600.0;
 constexpr int kPairRing = 4;        // prefetch depth of k_psweep (steps)
 constexpr int kPairWarps = 4;       // units per CTA of k_psweep: one per SM quarter
@@ -797,7 +802,7 @@ __global__ void __launch_bounds__(32 * kPairWarps) k_psweep(const FormalArgs A, 
 static int choose_tiles32(const Problem* P) {
   const int64_t want = (8LL * P->num_sms + P->ngroups - 1) / P->ngroups;
   int T = want < 1 ? 1 : (int)(want > kMaxTiles ? kMaxTiles : want);
-  while (T > 1 && (P->Ns - 1) / T < 2 * kRing32) --T;
+  while (T > 1 && (P->Ns - 1) / T < kMinSteps32) --T;
   return T;
 }
 
@@ -979,15 +984,16 @@ template <typename TV, int MODE>
 static void launch_formal32(const Problem* P, const TV* x, TV* y, cudaStream_t st, const int* kstop, int step) {
   const FormalArgs A = formal_args(P, x, y, P->S32, P->ntile32, kstop, step);
   const int g = P->ngroups, b = 32 * P->ntile32;
+  constexpr int RING = sizeof(TV) == 8 ? kRing32D : kRing32;
   switch (P->fs) {
     case RT_FS_DELO_LINEAR:
-      launch_pdl(k_formal<float, TV, RT_FS_DELO_LINEAR, MODE, 1, kRing32, kMaxTiles>, g, b, st, A); RT_COUNT(1);
+      launch_pdl(k_formal<float, TV, RT_FS_DELO_LINEAR, MODE, 1, RING, kMaxTiles>, g, b, st, A); RT_COUNT(1);
       break;
     case RT_FS_IMPLICIT_EULER:
-      launch_pdl(k_formal<float, TV, RT_FS_IMPLICIT_EULER, MODE, 1, kRing32, kMaxTiles>, g, b, st, A); RT_COUNT(1);
+      launch_pdl(k_formal<float, TV, RT_FS_IMPLICIT_EULER, MODE, 1, RING, kMaxTiles>, g, b, st, A); RT_COUNT(1);
       break;
     default:
-      launch_pdl(k_formal<float, TV, RT_FS_TRAPEZOIDAL, MODE, 1, kRing32, kMaxTiles>, g, b, st, A); RT_COUNT(1);
+      launch_pdl(k_formal<float, TV, RT_FS_TRAPEZOIDAL, MODE, 1, RING, kMaxTiles>, g, b, st, A); RT_COUNT(1);
   }
 }
 
