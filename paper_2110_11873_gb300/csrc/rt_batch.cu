@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kMomThreads) kb_moments(const InstDev* __restr
       moments_flat64<MODE, false, NORM>(x, I.dinv, I.wray, I.t201, I.t202, I.Minv, I.Ns, I.Nmu, I.nray, I.xi,
                                         I.xiW2, useS2 ? I.S2 : I.S, it.y, inv, xo);
     } else {
-      moments_flat32<double, MODE, kMomThreads, NORM>(x, I.dinv, I.wray32, I.t201f, I.t202f, I.Minv, I.Ns, I.Nmu, I.nray,
+      moments_flat32<double, MODE, kMomThreads, 1, NORM>(x, I.dinv, I.wray32, I.t201f, I.t202f, I.Minv, I.Ns, I.Nmu, I.nray,
                                          (float)I.xi, (float)I.xiW2, I.S32, it.y, inv, xo);
     }
     __syncthreads();

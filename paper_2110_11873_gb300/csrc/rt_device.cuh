@@ -99,8 +99,9 @@ __device__ __forceinline__ double beta_star(const double* __restrict__ cb, int k
 // NORM: the input is x * inv, written to xout in the input's precision as
 // each element is read (the GMRES normalisation of the batched solver).  A
 // warp per direction row, as before, left lanes idle on short rows and half
-// of its loads predicated off (32 uneven atmospheres: 139 us a launch).
-template <typename TI, int MODE, int THREADS, bool NORM = false>
+// of its loads predicated off (32 uneven atmospheres: 139 us a launch).  U: rays
+// whose loads are issued before their sums.
+template <typename TI, int MODE, int THREADS, int U, bool NORM = false>
 __device__ __forceinline__ void moments_flat32(const TI* __restrict__ x, const double* __restrict__ dinv,
                                                const float* __restrict__ wray, const float* __restrict__ t201,
                                                const float* __restrict__ t202, const double* __restrict__ Minv,
@@ -111,23 +112,43 @@ __device__ __forceinline__ void moments_flat32(const TI* __restrict__ x, const d
   const int64_t oI = (int64_t)k * nray, oQ = ((int64_t)Ns + k) * nray;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float a0 = 0.f, a1 = 0.f;
-#pragma unroll 4
-  for (int64_t r = threadIdx.x; r < nray; r += THREADS) {
-    TI xI = x[oI + r], xQ = x[oQ + r];
-    if (NORM) {
-      xI = (TI)(xI * inv);
-      xQ = (TI)(xQ * inv);
-      xout[oI + r] = xI;
-      xout[oQ + r] = xQ;
+#pragma unroll (U == 1 ? 4 : 1)
+  for (int64_t r0 = threadIdx.x; r0 < nray; r0 += U * THREADS) {
+    TI xI[U], xQ[U];
+    double dI[U], dQ[U];
+    float w0[U], w1[U], w2[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t r = r0 + u * THREADS < nray ? r0 + u * THREADS : r0;
+      xI[u] = x[oI + r];
+      xQ[u] = x[oQ + r];
+      if (MODE == KM_JACOBI) {
+        dI[u] = dinv[oI + r];
+        dQ[u] = dinv[oQ + r];
+      }
+      w0[u] = wray[r];
+      w1[u] = wray[nray + r];
+      w2[u] = wray[2 * nray + r];
     }
-    float vI = vcast<float>(xI), vQ = vcast<float>(xQ);
-    if (MODE == KM_JACOBI) {
-      vI *= to_f32(dinv[oI + r]);
-      vQ *= to_f32(dinv[oQ + r]);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t r = r0 + u * THREADS;
+      if (u > 0 && r >= nray) continue;
+      if (NORM) {
+        xI[u] = (TI)(xI[u] * inv);
+        xQ[u] = (TI)(xQ[u] * inv);
+        xout[oI + r] = xI[u];
+        xout[oQ + r] = xQ[u];
+      }
+      float vI = vcast<float>(xI[u]), vQ = vcast<float>(xQ[u]);
+      if (MODE == KM_JACOBI) {
+        vI *= to_f32(dI[u]);
+        vQ *= to_f32(dQ[u]);
+      }
+      a0 = fmaf(w0[u], vI, a0);
+      a1 = fmaf(w1[u], vI, a1);
+      a1 = fmaf(w2[u], vQ, a1);
     }
-    a0 = fmaf(wray[r], vI, a0);
-    a1 = fmaf(wray[nray + r], vI, a1);
-    a1 = fmaf(wray[2 * nray + r], vQ, a1);
   }
   a0 = warp_sum(a0);
   a1 = warp_sum(a1);

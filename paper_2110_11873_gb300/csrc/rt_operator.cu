@@ -224,13 +224,14 @@ __global__ void k_add_local(const double* __restrict__ v, const double* __restri
 }
 
 
-// FP32 quadrature, one CTA per height.  Bound by the loads in flight, which a
-// few CTAs an SM of 256 threads leave short: up to kMom32Heights heights per SM
-// a CTA has 512 threads.  Apply with 256 and 512 of them, trapezoidal: N_s = 100
-// heights of 62 x 201 rays 31.3 and 27.3 us, 316 of 58 x 138 57.2 and 50.5 us,
-// 466 of 58 x 138 70.8 and 63.7 us; but 1000 of 30 x 101 67.1 and 69.0 us, 2000
-// of 30 x 51 113.2 and 116.8 us.
-constexpr int kMom32Heights = 4;
+// FP32 quadrature, one CTA per height.  Bound by the loads in flight: a thread
+// issues those of kMom32Rays rays before it adds (apply with 256 threads a CTA,
+// trapezoidal, N_s = 1000 heights of 30 x 101 rays 52.1 -> 48.2 us, 2000 of 30 x
+// 51 86.2 -> 81.7 us), and on few heights, up to kMom32Heights per SM, a CTA has
+// 512 threads where that many rays are left: 256 and 512 threads took 37.6 and
+// 33.3 us on 316 heights of 58 x 138 rays, 20.3 and 18.0 us on 100 of 62 x 201,
+// but 47.1 and 47.8 us on 466 of 58 x 138 and 48.2 and 52.4 us on 1000 of 30 x 101.
+constexpr int kMom32Rays = 4, kMom32Heights = 3;
 template <typename TI, int MODE, int THREADS>
 __global__ void __launch_bounds__(THREADS) k_moments(
     const TI* __restrict__ x, const double* __restrict__ dinv, const float* __restrict__ wray,
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(THREADS) k_moments(
     int64_t nray, float xi, float xiW2, float* __restrict__ S, const int* kstop, int step) {
   pdl_wait();
   if (kstop && step >= *kstop) return;
-  moments_flat32<TI, MODE, THREADS>(x, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
+  moments_flat32<TI, MODE, THREADS, kMom32Rays>(x, dinv, wray, t201, t202, Minv, Ns, Nmu, nray, xi, xiW2, S, blockIdx.x);
 }
 
 // FP64 quadrature, one CTA per height (flat over the rays); WJ: Jacobi mode
@@ -1077,7 +1078,7 @@ rt_status op_apply64(Problem* P, const double* x, double* y, int mode, cudaStrea
 template <typename TV, int MODE>
 static cudaError_t launch_moments32(const Problem* P, const TV* x, const double* dinv, const double* Minv,
                                     cudaStream_t st, const int* kstop, int step) {
-  const bool few = P->Ns <= kMom32Heights * P->num_sms;
+  const bool few = P->Ns <= kMom32Heights * P->num_sms && P->nray > kMom32Rays * kMomThreads;
   RT_COUNT(1);
   return launch_pdl(few ? k_moments<TV, MODE, kMom32Threads> : k_moments<TV, MODE, kMomThreads>, P->Ns,
                     few ? kMom32Threads : kMomThreads, st, x, dinv, (const float*)P->wray32, (const float*)P->t201f,

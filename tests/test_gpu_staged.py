@@ -202,11 +202,12 @@ def test_chained_applies_back_to_back_equal_synchronised_ones(name, at):
         np.testing.assert_array_equal(chained, to_host(ref), err_msg=f"{name} {dt}")
 
 
-@pytest.mark.parametrize("Ns,Nmu,Nnu", [(5, 2, 2), (9, 2, 255), (9, 2, 256), (9, 2, 257), (7, 6, 171), (3, 30, 101), (608, 2, 3),
-                                        (609, 2, 3), (640, 2, 129)])
+@pytest.mark.parametrize("Ns,Nmu,Nnu", [(5, 2, 2), (9, 2, 255), (9, 2, 256), (9, 2, 257), (7, 6, 171), (3, 30, 101), (456, 2, 3),
+                                        (457, 2, 3), (3, 2, 1024), (3, 2, 1025), (460, 2, 511), (460, 2, 513)])
 def test_register_path_ray_counts_around_the_quadrature_block(Ns, Nmu, Nnu, monkeypatch):
     """The flat FP32 quadrature with less than a warp of rays, and below, at and
-    past one and two rounds of its threads, on few and on many heights."""
+    past one and two rounds of its threads and four rays of each, on few and on
+    many heights."""
     at = W.slab(Ns, Nmu, Nnu, 1e-3, 1e4, 5.0, eps=1e-2)
     monkeypatch.setenv("RT_NO_TMA", "1")
     P = problem(at)
