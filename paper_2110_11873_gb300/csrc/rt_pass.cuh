@@ -57,6 +57,7 @@ __device__ __forceinline__ double fx_warp_sum(double t) {
 
 constexpr int kFxHead = 2;        // headroom (bits) over the first values' largest exponent
 constexpr int kFxHeadMore = 3;    // the same when a later value did not fit
+constexpr int kFxMinExp = 64;     // smallest scale: zeros and subnormal numbers shift out from 59 on
 constexpr int kFxEpoch = 62;      // additions between two scalings: 62 products a lane fit the 64-bit sums
 
 // ND dot products <w, v_d> of one warp, one element per lane and add(); the
@@ -64,7 +65,9 @@ constexpr int kFxEpoch = 62;      // additions between two scalings: 62 products
 // scales (one exponent for w, one for the v_d) come from the warp's first
 // values and are renewed when a value does not fit and after kFxEpoch
 // additions; at each renewal the warp's integer sums are folded exactly into
-// lane d's FP64 sum.  Infinities and NaN take the FP64 products.
+// lane d's FP64 sum.  Infinities, NaN and values whose largest is below 2^-961
+// (the scales end there) take the FP64 products; zeros and subnormal numbers
+// have digits of value zero.
 //
 // SQ: dot 0 is <w, w> (v[0] is not read), from the digits of w twice and with
 // w's scale twice.  What is left of w may be far smaller than the vectors v_d:
@@ -124,8 +127,9 @@ struct FixDot {
     // (t2 2^48 + t1 2^24 + t0 + f0 2^-24) 2^58 2^(Ev - 1079) 2^(Ew - 1079)
     const long long top = ((long long)t2 << 24) + t1, bot = ((long long)t0 << 24) + f0;
     const double v = fma((double)top, 16777216.0, (double)bot * 5.9604644775390625e-08);
-    const int E = SQ && lane == 0 ? Ew : Ev;
-    if (lane < NI) acc += v * fx_pow2(E - 1050) * fx_pow2(Ew - 1050);
+    // the power of two in two halves, so that neither overflows or underflows before the product does
+    const int E = (SQ && lane == 0 ? Ew : Ev) + Ew - 2100;
+    if (lane < NI) acc += v * fx_pow2(E >> 1) * fx_pow2(E - (E >> 1));
     clear();
   }
 
@@ -141,10 +145,11 @@ struct FixDot {
       const int head = left > 0 ? kFxHeadMore : kFxHead;
       if (Ew) fold();
       const int mw = __reduce_max_sync(0xffffffffu, ew), mv = __reduce_max_sync(0xffffffffu, ev);
-      Ew = min(max(mw + head, 64), 2046);
-      Ev = min(max(mv + head, 64), 2046);
+      Ew = min(max(mw + head, kFxMinExp), 2046);
+      Ev = min(max(mv + head, kFxMinExp), 2046);
       left = kFxEpoch;
-      if (max(mw, mv) == 2047) {   // an infinity or a NaN: these elements in FP64
+      const bool f64 = max(mw, mv) == 2047 || (mw > 0 && mw + head < kFxMinExp) || (mv > 0 && mv + head < kFxMinExp);
+      if (f64) {   // these elements in FP64
         left = 0;
         Ew = 0;
 #pragma unroll

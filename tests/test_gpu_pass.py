@@ -226,3 +226,43 @@ def test_pass_digits_round_without_a_sign(sign):
     h = to_host(P.arnoldi_bmgs(V, 0, to_dev(w0), torch.zeros(8, dtype=torch.float64, device="cuda")))
     exact = float(np.sum(w0.astype(np.longdouble) * v.astype(np.longdouble)))
     assert abs(h[0] / exact - 1.0) < 2.7e-13, h[0] / exact - 1.0
+
+
+@pytest.mark.parametrize("scale", [1e-290, 1e-300, 1e-306])
+@pytest.mark.parametrize("j", [0, 2, 3, 9])
+def test_pass_of_a_w_near_the_smallest_numbers(scale, j):
+    """Entries below 2^-961, where the fixed-point scales end: the coefficients
+    and what is left of w keep the accuracy of the other cases, 1e-12 and 1e-11
+    of |w| (the products with the basis round to multiples of 5e-324, 65,600 of
+    them to 2e-319 at most)."""
+    P = problem(W.slab(100, 8, 41, 1e-4, 1e6, 6.0))
+    N = P.N
+    rng = np.random.default_rng(j)
+    Q = _basis(N, j, rng)
+    u0 = rng.standard_normal(N)
+    gram = np.zeros((j + 2, 4))
+    for i in range(1, j + 1):
+        for d in range(1, min(i, 3) + 1):
+            gram[i, d] = Q[i] @ Q[i - d]
+    V = torch.zeros((j + 2) * N, dtype=torch.float64, device="cuda")
+    V[: (j + 1) * N] = to_dev(np.concatenate(Q))
+    wd = to_dev(scale * u0)
+    h = to_host(P.arnoldi_bmgs(V, j, wd, to_dev(gram.reshape(-1))))
+    P.check()
+    href, w = _mgs(Q, u0)
+    s = np.linalg.norm(u0)
+    np.testing.assert_allclose(h[: j + 1] / scale, href[: j + 1], rtol=0, atol=1e-12 * s)
+    np.testing.assert_allclose(to_host(wd) / scale, w, rtol=0, atol=1e-11 * s)
+
+
+def test_pass_of_large_vectors_and_a_small_w():
+    """A dot whose factors are far apart but whose value is ordinary: 1e300 and
+    1e-300 (the basis of a caller need not be normalised for it)."""
+    P = problem(W.slab(100, 8, 41, 1e-4, 1e6, 6.0))
+    N = P.N
+    rng = np.random.default_rng(2)
+    v, w0 = rng.standard_normal(N), rng.standard_normal(N)
+    V = torch.zeros(2 * N, dtype=torch.float64, device="cuda")
+    V[:N] = to_dev(1e300 * v)
+    h = to_host(P.arnoldi_bmgs(V, 0, to_dev(1e-300 * w0), torch.zeros(8, dtype=torch.float64, device="cuda")))
+    assert abs(h[0] - v @ w0) < 1e-12 * np.linalg.norm(v) * np.linalg.norm(w0), h[0]
