@@ -248,7 +248,8 @@ __global__ void __launch_bounds__(kVecThreads) k_norm_out(const double* __restri
 // Three forms of the step (mgs_plan, enqueue_bmgs): k_pass, the dots on the
 // integer pipe and the operands streamed by bulk copies; k_small_step, short
 // vectors in one CTA; and k_bdot / k_bmgs here, for vectors that a bulk copy
-// cannot start on.  The FP64 pipe bounds these last, so their reductions are
+// cannot start on (k_bdot also for the first dots of the first steps, kRegDots).
+// The FP64 pipe bounds these last, so their reductions are
 // kept short: one CTA per resident slot (a single wave, several elements per
 // thread) and a transposing warp reduction of the four accumulators (6 FP64
 // additions per thread instead of 20).
@@ -1128,14 +1129,24 @@ struct Workspace {
 
 using PassFn = void (*)(double*, const double*, int64_t, int, const double*, double*, double*, const double*, int, int,
                         const int*, int*, int);
+// The first dots of a step with up to kRegDots vectors run in k_bdot: with
+// nothing to update, the FP64 pipe holds that many dots beside the loads (slab of
+// 1,939,200 unknowns, k_bdot and k_pass: 8.7 and 14.8 us for one vector, 13.1
+// and 16.6 for two, 16.5 and 18.8 for three).
+constexpr int kRegDots = 3;
 // the passes of blocks of B vectors: first dots with n + 1 vectors, a full
 // block with n + 1 look-ahead dots, a last block of n + 1 vectors
 template <int B>
 struct PassTable {
   PassFn dot[B], mid[B], last[B];
+  template <int n>
+  static constexpr PassFn first_dots() {
+    if constexpr (n <= kRegDots) return nullptr;
+    else return k_pass<B, 0, n>;
+  }
   template <int... n>
   constexpr explicit PassTable(std::integer_sequence<int, n...>)
-      : dot{k_pass<B, 0, n + 1>...}, mid{k_pass<B, B, n + 1>...}, last{k_pass<B, n + 1, 0>...} {}
+      : dot{first_dots<n + 1>()...}, mid{k_pass<B, B, n + 1>...}, last{k_pass<B, n + 1, 0>...} {}
   PassTable() : PassTable(std::make_integer_sequence<int, B>()) {}
 };
 static const PassTable<kGramB> g_pass4;      // rt_arnoldi_bmgs (RT_GRAM_BLOCK)
@@ -1146,9 +1157,13 @@ static cudaError_t pass_smem_attr(const PassTable<B>& T) {
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < B; ++i)
     for (PassFn f : {T.dot[i], T.mid[i], T.last[i]})
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassDynSmem);
+      if (e == cudaSuccess && f) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassDynSmem);
   return e;
 }
+
+using BdotFn = void (*)(const double*, const double*, int64_t, double*, int, int, const int*);
+static_assert(kGramB == 4 && kRegDots <= kGramB, "kernel tables");
+static const BdotFn g_bdot[kGramB] = {k_bdot<1>, k_bdot<2>, k_bdot<3>, k_bdot<4>};
 
 static rt_status ensure_workspace(Problem* P, int restart, cudaStream_t st) {
   {
@@ -1263,9 +1278,13 @@ static rt_status enqueue_passes(Problem* P, const PassTable<B>& T, const double*
                                 double* hcol, const double* gram, const int* kstop, cudaStream_t st, int* pb, int* ng,
                                 int* rev, int fail_wait) {
   const int64_t N = P->Nop;
-  RT_TRY_CUDA(launch_pdl_smem(T.dot[std::min(B, j + 1) - 1], Gm, kPassThreads, kPassDynSmem, st, w, V, N, 0,
-                              (const double*)nullptr, bpartb(P, 0), (double*)nullptr, (const double*)nullptr, j, *rev,
-                              kstop, P->dev_err, fail_wait)); RT_COUNT(1);
+  if (j < kRegDots)
+    RT_TRY_CUDA(launch_pdl(g_bdot[j], Gm, kMgsThreads, st, (const double*)w, V, N, bpartb(P, 0), j, *rev, kstop));
+  else
+    RT_TRY_CUDA(launch_pdl_smem(T.dot[std::min(B, j + 1) - 1], Gm, kPassThreads, kPassDynSmem, st, w, V, N, 0,
+                                (const double*)nullptr, bpartb(P, 0), (double*)nullptr, (const double*)nullptr, j,
+                                *rev, kstop, P->dev_err, 0));
+  RT_COUNT(1);
   for (int i0 = 0; i0 <= j; i0 += B) {
     const int nb = std::min(B, j + 1 - i0);
     const int nn = std::max(0, std::min(B, j + 1 - (i0 + nb)));
@@ -1273,7 +1292,7 @@ static rt_status enqueue_passes(Problem* P, const PassTable<B>& T, const double*
     *rev ^= 1;
     RT_TRY_CUDA(launch_pdl_smem(nn ? T.mid[nn - 1] : T.last[nb - 1], Gm, kPassThreads, kPassDynSmem, st, w, V, N, i0,
                                 (const double*)bpartb(P, *pb), bpartb(P, *pb ^ 1), hcol, gram, j, *rev, kstop,
-                                P->dev_err, 0)); RT_COUNT(1);
+                                P->dev_err, i0 == 0 ? fail_wait : 0)); RT_COUNT(1);
     *pb ^= 1;
   }
   return RT_OK;
@@ -1295,10 +1314,8 @@ static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* h
     if (gb == kGramB) RT_TRY(enqueue_passes(P, g_pass4, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev, fail_wait));
     else RT_TRY(enqueue_passes(P, g_pass8, V, w, Gm, j, hcol, gram, kstop, st, &pb, &ng, &rev, fail_wait));
   } else {
-    using BdotFn = void (*)(const double*, const double*, int64_t, double*, int, int, const int*);
     using BmgsFn = void (*)(double*, const double*, int64_t, int, const double*, double*, double*, const double*, int,
                             int, const int*);
-    static const BdotFn bdot[kGramB] = {k_bdot<1>, k_bdot<2>, k_bdot<3>, k_bdot<4>};
     static const BmgsFn pass[kGramB] = {k_bmgs<4, 1>, k_bmgs<4, 2>, k_bmgs<4, 3>, k_bmgs<4, 4>};
     static const BmgsFn last[kGramB] = {k_bmgs<1, 0>, k_bmgs<2, 0>, k_bmgs<3, 0>, k_bmgs<4, 0>};
     static_assert(kGramB == 4, "kernel tables");
@@ -1306,7 +1323,7 @@ static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* h
       set_error("internal: these block passes take blocks of %d vectors", kGramB);
       return RT_EINVAL;
     }
-    RT_TRY_CUDA(launch_pdl(bdot[std::min(kGramB, j + 1) - 1], Gm, kMgsThreads, st, (const double*)w, (const double*)V,
+    RT_TRY_CUDA(launch_pdl(g_bdot[std::min(kGramB, j + 1) - 1], Gm, kMgsThreads, st, (const double*)w, (const double*)V,
                            N, bpartb(P, 0), j, rev, kstop)); RT_COUNT(1);
     for (int i0 = 0; i0 <= j; i0 += kGramB) {
       const int nb = std::min(kGramB, j + 1 - i0);

@@ -221,9 +221,9 @@ def test_pass_digits_round_without_a_sign(sign):
     w0[::32] = 2.0 ** 20
     v[::32] = 0.0
     v /= np.linalg.norm(v)
-    V = torch.zeros(2 * N, dtype=torch.float64, device="cuda")
+    V = torch.zeros(5 * N, dtype=torch.float64, device="cuda")   # a step that forms the first dot on the integer pipe
     V[:N] = to_dev(v)
-    h = to_host(P.arnoldi_bmgs(V, 0, to_dev(w0), torch.zeros(8, dtype=torch.float64, device="cuda")))
+    h = to_host(P.arnoldi_bmgs(V, 3, to_dev(w0), torch.zeros(20, dtype=torch.float64, device="cuda")))
     exact = float(np.sum(w0.astype(np.longdouble) * v.astype(np.longdouble)))
     assert abs(h[0] / exact - 1.0) < 2.7e-13, h[0] / exact - 1.0
 
@@ -262,7 +262,7 @@ def test_pass_of_large_vectors_and_a_small_w():
     N = P.N
     rng = np.random.default_rng(2)
     v, w0 = rng.standard_normal(N), rng.standard_normal(N)
-    V = torch.zeros(2 * N, dtype=torch.float64, device="cuda")
+    V = torch.zeros(5 * N, dtype=torch.float64, device="cuda")
     V[:N] = to_dev(1e300 * v)
-    h = to_host(P.arnoldi_bmgs(V, 0, to_dev(1e-300 * w0), torch.zeros(8, dtype=torch.float64, device="cuda")))
+    h = to_host(P.arnoldi_bmgs(V, 3, to_dev(1e-300 * w0), torch.zeros(20, dtype=torch.float64, device="cuda")))
     assert abs(h[0] - v @ w0) < 1e-12 * np.linalg.norm(v) * np.linalg.norm(w0), h[0]
