@@ -12,9 +12,10 @@
 //    of a dedicated CTA of the kernel that needs them next (the Givens
 //    rotations run in a CTA of the scaling kernel, or of the next step's
 //    quadrature kernel) -- so a GMRES restart cycle runs as CUDA graphs of
-//    kSegSteps Arnoldi steps and one for its end (the least-squares solve, the
-//    update of x and the true residual), the host reading the convergence
-//    state behind each and keeping one graph ahead of the device;
+//    kSegSteps Arnoldi steps, the last with the end of the cycle (the
+//    least-squares solve, the update of x and the true residual), the host
+//    reading the convergence state behind each and keeping one graph ahead of
+//    the device;
 //  * a step index baked into each kernel of a cycle's graphs is compared with
 //    the device counter `kstop`: once the residual estimate passes the
 //    tolerance the remaining kernels of the graph return at once, and the
@@ -1350,16 +1351,19 @@ static rt_status enqueue_bmgs(Problem* P, double* V, double* w, int j, double* h
 }
 
 // --------------------------------------------------------------- GMRES
-// A restart cycle is launched as graphs of kSegSteps Arnoldi steps and a last
-// one with the end of the cycle.  One graph of the whole cycle (as the cycle
-// was launched before) ran its kernels past convergence as gated launches,
+// A restart cycle is launched as graphs of kSegSteps Arnoldi steps, the last of
+// which also holds the end of the cycle and up to kSegSteps / 2 steps more.  One
+// graph of the whole cycle ran its kernels past convergence as gated launches,
 // about 1.3 us each: an unrestarted sigma-form run of 41 steps spent two thirds
 // of its time in them, and the launch queued ahead of the host's check cost a
-// cycle of 30 steps 5%.
+// cycle of 30 steps 5%.  A graph of its own for the end of every cycle, on the
+// other hand, cost short cycles 7% (70 x 16 x 21, restarts of 5).
 constexpr int kSegSteps = 8;
-inline int cycle_segments(int m) { return (m + kSegSteps - 1) / kSegSteps; }
+inline int cycle_segments(int m) { return std::max(1, (m + kSegSteps / 2 - 1) / kSegSteps); }
+inline int segment_end(int m, int seg) { return seg + 1 >= cycle_segments(m) ? m : (seg + 1) * kSegSteps; }
 
-// seg: steps seg * kSegSteps .. of the cycle, or cycle_segments(m) for its end
+// seg: steps seg * kSegSteps .. of the cycle, the last of cycle_segments(m) with
+// its end; or cycle_segments(m) for the end alone, after a stop in an earlier one
 struct GmresGraphKey {
   int m, precond, fp32, seg;
   bool operator<(const GmresGraphKey& o) const {
@@ -1423,8 +1427,8 @@ void release_graphs(Problem* P) {
   }
 }
 
-// Enqueue segment seg of a restart cycle: Arnoldi steps of 0..m-1 or, for seg
-// = cycle_segments(m), the least squares, x update, true residual and the
+// Enqueue segment seg of a restart cycle (GmresGraphKey): Arnoldi steps of
+// 0..m-1 and, at the end, the least squares, x update, true residual and the
 // start of the next cycle.  Vectors: x = wk(0), b = wk(1), r = wk(2), w =
 // wk(3), t = wk(4), Ax = wk(5), tmp = wk(6).
 static rt_status enqueue_cycle(Problem* P, int m, int precond, int fp32, int seg, cudaStream_t st) {
@@ -1446,8 +1450,9 @@ static rt_status enqueue_cycle(Problem* P, int m, int precond, int fp32, int seg
   const MgsPlan plan = mgs_plan(P, P->V, w);
   const int Gm = plan.grid;                          // partials per reduction of the block passes
   const int gb = plan.fixed ? kGramMax : kGramB;     // their block size
-  const bool end = seg == cycle_segments(m);
-  const int j0 = end ? m : seg * kSegSteps, j1 = end ? m : std::min(m, j0 + kSegSteps);
+  const int nseg = cycle_segments(m);
+  const bool end = seg + 1 >= nseg;
+  const int j0 = seg == nseg ? m : seg * kSegSteps, j1 = segment_end(m, seg);
   // where the step before the segment left its last partials (enqueue_bmgs)
   int pb = 0, ng = 0;
   if (j0 > 0) {
@@ -1684,6 +1689,7 @@ static rt_status gmres_core(Problem* P, const rt_solver_opts* o, int fp32, doubl
   // the first kernel after it, so a stop at that end still needs the next
   // segment), the end of the cycle comes next.
   const int nseg = cycle_segments(m);
+  auto ends = [&](int seg) { return seg + 1 >= nseg; };   // the end of the cycle is in it
   HeaderQueue<GmresDev> Q{gc, P->gm, kGmresHeader, st};
   RT_TRY(Q.init());
   auto launch = [&](int seg, int slot) -> rt_status {
@@ -1691,19 +1697,19 @@ static rt_status gmres_core(Problem* P, const rt_solver_opts* o, int fp32, doubl
     RT_TRY(get_graph(P, gc, m, o->precond, fp32, seg, &ex));
     return Q.launch(ex, slot);
   };
-  int cur = 0, next = 1, slot = 0;
+  int cur = 0, next = ends(0) ? 0 : 1, slot = 0;
   rt_status s = launch(cur, slot);
   while (s == RT_OK) {
     s = launch(next, slot ^ 1);
     if (s == RT_OK) s = Q.read(slot, hs);
     if (s != RT_OK) break;
-    int after = next == nseg ? 0 : next + 1;
-    if (cur == nseg) {
+    int after = ends(next) ? 0 : next + 1;
+    if (ends(cur)) {
       *cycles += 1;
       const GmresDev& h = *hs;
       if (h.rel != h.rel || !(h.rel >= tol) || h.iters >= maxit || (h.breakdown && h.kdone == 0) || h.kstop == 0)
         break;
-    } else if (next != nseg && hs->kstop < std::min(m, (cur + 1) * kSegSteps)) {
+    } else if (!ends(next) && hs->kstop < segment_end(m, cur)) {
       after = nseg;
     }
     cur = next;
