@@ -159,6 +159,11 @@ struct FixDot {
         }
         return;
       }
+      if (mw == 0 || (!SQ && mv == 0)) {   // nothing to add, and no scale for what follows
+        left = 0;
+        Ew = 0;
+        return;
+      }
     }
     --left;
     int w1, w0;

@@ -266,3 +266,25 @@ def test_pass_of_large_vectors_and_a_small_w():
     V[:N] = to_dev(1e300 * v)
     h = to_host(P.arnoldi_bmgs(V, 3, to_dev(1e-300 * w0), torch.zeros(20, dtype=torch.float64, device="cuda")))
     assert abs(h[0] - v @ w0) < 1e-12 * np.linalg.norm(v) * np.linalg.norm(w0), h[0]
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-300])
+def test_pass_of_zero_tiles_before_others(scale):
+    """Every other tile of w, or of the basis vectors, is zero: a warp that meets
+    the zeros first takes no scale from them."""
+    P = problem(W.slab(300, 32, 32, 1e-4, 1e6, 6.0))   # 2400 tiles, 8 to a CTA
+    N, j = P.N, 6
+    rng = np.random.default_rng(1)
+    zero = np.arange(N) // 256 % 2 == 0
+    u0 = np.where(zero, 0.0, rng.standard_normal(N))
+    Q = np.where(zero[None] == (np.arange(j + 1) % 3 == 2)[:, None], rng.standard_normal((j + 1, N)), 0.0) / np.sqrt(N / 2)
+    V = torch.zeros((j + 2) * N, dtype=torch.float64, device="cuda")
+    V[: (j + 1) * N] = to_dev(Q.reshape(-1))
+    gram = np.zeros((j + 2, 4))
+    for i in range(1, j + 1):
+        for d in range(1, min(i, 3) + 1):
+            gram[i, d] = Q[i] @ Q[i - d]
+    h = to_host(P.arnoldi_bmgs(V, j, to_dev(scale * u0), to_dev(gram.reshape(-1))))
+    P.check()
+    href, w = _mgs(Q, u0)
+    np.testing.assert_allclose(h[: j + 1] / scale, href[: j + 1], rtol=0, atol=1e-12 * np.linalg.norm(u0))
