@@ -707,18 +707,25 @@ inline int cdiv(int a, int b) { return (a + b - 1) / b; }
 // also the number of partials per reduction.  k_pass is the faster one at
 // every size measured: a step at j = 29 took 273.8 us with k_bdot / k_bmgs and
 // 213.2 us with k_pass at N = 1,939,200, 87.6 and 68.5 us at N = 195,200, 64.0
-// and 52.8 us at N = 69,440 (blocks of 4).
+// and 52.8 us at N = 69,440 (blocks of 4).  Grid: the resident CTAs, but one per
+// SM up to kPassFewTiles tiles for each: more of them cost more in starting and
+// in partials (every CTA of the next pass sums them) than they gain.  GMRES
+// cycles of 12 and 60 steps, 2 and 1 per SM: N = 47,040 (184 tiles) 624 and 609,
+// 3848 and 3673 us; N = 65,600 644 and 610, 4163 and 3705 us; N = 99,200 674 and
+// 639, 4642 and 4091 us; N = 196,800 (769 tiles) no difference.
 struct MgsPlan {
   bool fixed;
   int grid;
 };
-constexpr int kPassCtasPerSm = 2;   // resident at once (the ring's size): 1 per SM took 1.25 times as long
+constexpr int kPassCtasPerSm = 2;   // resident at once (the ring's size); on long vectors 1 per SM took 1.25 times as long
+constexpr int kPassFewTiles = 4;
 inline MgsPlan mgs_plan(const Problem* P, const double* V, const double* w) {
   const int64_t N = P->Nop;
   if ((N & 1) || !P->dev_err || (reinterpret_cast<uintptr_t>(V) & 15) || (reinterpret_cast<uintptr_t>(w) & 15))
     return {false, mgs_grid(P)};
   const int64_t tiles = (N + kPassTile - 1) / kPassTile;
-  return {true, (int)std::min<int64_t>(tiles, std::min(kPassCtasPerSm * P->num_sms, kMaxPartials))};
+  const int ctas = (tiles < kPassFewTiles * P->num_sms ? 1 : kPassCtasPerSm) * P->num_sms;
+  return {true, (int)std::min<int64_t>(tiles, std::min(ctas, kMaxPartials))};
 }
 
 // back substitution H(0:k,0:k) y = g(0:k) in the textbook order: row k-1

@@ -288,3 +288,11 @@ def test_pass_of_zero_tiles_before_others(scale):
     P.check()
     href, w = _mgs(Q, u0)
     np.testing.assert_allclose(h[: j + 1] / scale, href[: j + 1], rtol=0, atol=1e-12 * np.linalg.norm(u0))
+
+@pytest.mark.parametrize("Nnu", [95, 152, 153, 456, 607, 608, 609])
+def test_pass_grid_around_one_cta_per_sm(Nnu):
+    """Vectors of 95 to 609 tiles: fewer than one per SM, one, and up to and past
+    the length from which two CTAs share an SM."""
+    P = problem(W.slab(8, 8, Nnu * 2, 1e-4, 1e6, 6.0))   # N = 256 * Nnu
+    assert P.N == 256 * Nnu
+    _step(P, P.N, 6, "normal", seed=Nnu)
