@@ -315,6 +315,7 @@ struct Problem {
   int tau_kind = 0, mu_quad = 0, fs = 0, freq_norm = 0;
   // host grids
   std::vector<double> tau, B, mu, w_mu, x, phi, w_nu, phi_hat, t201, t202;
+  bool even_phi = false;   // the profile is even about the middle of the frequency grid, but for rounding
   // ray groups of the formal-solver kernel: 32 consecutive rays of one
   // direction sign; the nd = Nh*Nnu downward rays come first
   int64_t nd = 0;
@@ -364,7 +365,7 @@ struct Problem {
   double* dinv = nullptr;     // N, Jacobi inverse diagonal
   float* work32 = nullptr;    // 2 vectors of N (FP32 operator)
   double* partials = nullptr; // 2 x kMaxPartials x 8
-  double* bpart = nullptr;    // 2 x kGramMax x kMaxPartials: block-pass partials (two ping-pong buffers, Gram)
+  double* bpart = nullptr;    // 2 x kGramMax x kMaxPartials: block-pass partials (two buffers in turn)
   GmresDev* gm = nullptr;
   BicgDev* bc = nullptr;
   double* hist = nullptr;     // device history

@@ -815,9 +815,18 @@ rt_status setup_device_tables(Problem* P, cudaStream_t st) {
   P->ngroups = 2 * ngd;
   // the step coefficients depend on |mu| only unless the scheme has a
   // downwind term, and on the frequency through the profile: where that is
-  // symmetric on the grid, bit for bit, the pairs p, Nnu-1-p share them too
+  // symmetric on the grid (the internal one on symmetric limits, or a caller's,
+  // bit for bit) the pairs p, Nnu-1-p share them too.  The grids that a caller
+  // sees are the same whichever kernels run: x_p = x_min + p h is symmetric but
+  // for its rounding, and the tables here take the values of the lower half for
+  // both halves.
   bool mirror = P->fs != RT_FS_DELO_PARABOLIC && P->N >= kPairMinN;
-  for (int p = 0; p < Nnu && mirror; ++p) mirror = P->phi_hat[p] == P->phi_hat[Nnu - 1 - p];
+  for (int p = 0; p < Nnu && mirror && !P->even_phi; ++p) mirror = P->phi_hat[p] == P->phi_hat[Nnu - 1 - p];
+  std::vector<double> phi_hat(P->phi_hat), w_nu(P->w_nu);
+  for (int p = 0; mirror && p < Nnu / 2; ++p) {
+    phi_hat[Nnu - 1 - p] = phi_hat[p];
+    w_nu[Nnu - 1 - p] = w_nu[p];
+  }
   P->cshare = P->fs == RT_FS_DELO_PARABOLIC ? CS_RAY : mirror ? CS_PAIR : CS_MU;
   P->cstride = mirror ? (int64_t)Nh * pair_count(Nnu) : P->cshare ? nray / 2 : nray;
   P->npair = mirror ? 2 * P->cstride : 0;
@@ -832,8 +841,8 @@ rt_status setup_device_tables(Problem* P, cudaStream_t st) {
   for (int m = 0; m < Nmu; ++m)
     for (int p = 0; p < Nnu; ++p) {
       const size_t r = (size_t)m * Nnu + p;
-      rscale[r] = P->phi_hat[p] / fabs(P->mu[m]);
-      w0[r] = 0.5 * P->w_mu[m] * P->w_nu[p];
+      rscale[r] = phi_hat[p] / fabs(P->mu[m]);
+      w0[r] = 0.5 * P->w_mu[m] * w_nu[p];
       w0[nray + r] = w0[r] * P->t201[m];       // the J20 weights of I and Q
       w0[2 * nray + r] = w0[r] * P->t202[m];
     }

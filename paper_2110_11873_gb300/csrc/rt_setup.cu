@@ -207,15 +207,14 @@ void host_grids(const rt_problem_desc* d, Problem& P) {
   P.w_nu.resize(Nnu);
   P.phi_hat.resize(Nnu);
   for (int p = 0; p < Nnu; ++p) P.x[p] = (p == Nnu - 1) ? d->x_max : d->x_min + p * h;
-  if (d->x_min == -d->x_max && P.N >= kPairMinN)   // symmetric about the line centre to the last bit
-    for (int p = 0; 2 * p + 1 <= Nnu; ++p) P.x[Nnu - 1 - p] = 2 * p + 1 == Nnu ? 0.0 : -P.x[p];
+  P.even_phi = !d->phi && d->x_min == -d->x_max;
   double phi_c;
   if (d->phi) {
     for (int p = 0; p < Nnu; ++p) P.phi[p] = d->phi[p];
     phi_c = d->phi_center;
   } else {
     const double rsp = 1.0 / sqrt(M_PI);
-    for (int p = 0; p < Nnu; ++p) P.phi[p] = voigt_H(d->a, fabs(P.x[p])) * rsp;   // H is even in x
+    for (int p = 0; p < Nnu; ++p) P.phi[p] = voigt_H(d->a, P.x[p]) * rsp;
     phi_c = voigt_H(d->a, 0.0) * rsp;
   }
   double wsum = 0.0;

@@ -62,3 +62,21 @@ def test_pairs_against_the_oracle():
     assert_close_scaled(to_host(P.apply(to_dev(x))), tr.apply_I(x), 1e-10)
     assert_close_scaled(to_host(P.rhs()), tr.rhs_I(), 1e-10)
     assert_close_scaled(to_host(P.jacobi_diag()), tr.jacobi_I(), 1e-10)
+
+
+@pytest.mark.parametrize("x_max,Nnu", [(8.0, 201), (6.0, 100), (4.0, 57)])
+def test_grids_do_not_depend_on_the_kernels(x_max, Nnu):
+    """The same frequencies, profile and weights to the bit on both sides of the
+    size from which pairs are solved together; above it a symmetric x gives a
+    symmetric A x to the bit, which only the pairs do (x_p = x_min + p h rounds
+    differently in the two halves)."""
+    Ns = (4 << 20) // (2 * 64 * Nnu)
+    small, large = (problem(W.slab(n, 64, Nnu, 1e-4, 1e8, x_max)) for n in (Ns - 8, Ns + 8))
+    assert small.N < 4 << 20 <= large.N
+    a, b = small.grids(), large.grids()
+    for k in a:
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    x = to_dev(W.random_vector(large.N, 7)).reshape(-1, Nnu)
+    x = x + x.flip(1)
+    y = large.apply(x.reshape(-1)).reshape(-1, Nnu)
+    assert torch.equal(y, y.flip(1))
