@@ -139,6 +139,31 @@ def probe_main(args):
     P.close()
 
 
+# ------------------------------------------------------------ the result line
+# keys that the line gives as they are; of the others it gives the numbers
+CONTRACT = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "roofline", "clocks", "e2e", "gpu_launches", "cpu_baseline")
+
+def result_line(rec):
+    """The record as one line of at most a few KB (a reader that keeps only the
+    end of the output lost the beginning of a line of 30 KB): the other
+    sections without their texts, a list of results as how many there are and how
+    many of them converged, numbers to 5 digits."""
+    def short(v):
+        if isinstance(v, float):
+            return float(f"{v:.5g}")
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items() if not (isinstance(x, str) or k == "per_solve")}
+        if isinstance(v, list) and v and isinstance(v[0], dict):
+            return {"results": len(v), "converged": sum(r.get("status") == 0 for r in v)}
+        return v
+
+    out = {k: v if k in CONTRACT else short(v) for k, v in rec.items() if k in CONTRACT or not isinstance(v, str)}
+    if "roofline" in out:
+        out["roofline"] = {k: v for k, v in out["roofline"].items() if k != "note"}
+    return out
+
+
 # ----------------------------------------------------------------- clocks
 class ClockSampler:
     """nvidia-smi clock / throttle-reason sampling during the timed region."""
@@ -861,7 +886,8 @@ def main():
                         served.setdefault("vs_oracle", {})[kind[len("served"):]] = rows
                 if "error" in errs:
                     out["oracle_errors_failed"] = errs["error"]
-        print(json.dumps(out))
+        print(json.dumps(out), file=sys.stderr)   # the whole record
+        print(json.dumps(result_line(out)), flush=True)
     P.close()
     if dist is not None:
         dist.destroy_process_group()

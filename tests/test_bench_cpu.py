@@ -100,3 +100,24 @@ def test_oracle_per_solve_check_of_saved_solutions(tmp_path):
     assert "error" not in out, out
     assert out["batched"]["true_resid_max"] < 1e-12 and out["batched"]["err_vs_lu_max"] < 1e-12
     assert 5e-7 < out["served200"]["err_vs_lu_max"] < 2e-6
+
+
+def test_result_line_is_short_and_keeps_the_contract():
+    """Long lists and texts stay in the record on stderr; the keys that a reader
+    of the line relies on are unchanged."""
+    sys.path.insert(0, ROOT)
+    import bench
+    case = {"Ns": 300, "precond": "jacobi", "iters": 1000, "status": 0, "solve_ms": 123.456789012345}
+    solves = [{"index": i, "true_resid": 1.23456789e-9, "err_vs_lu": None} for i in range(50)]
+    rec = {k: 1.23456789012345 for k in bench.CONTRACT}
+    rec.update(metric=bench.METRIC, config={"workload": "x" * 300}, roofline={"frac": 0.5, "note": "n" * 400},
+               size_sweep={"apply": {str(n): {"apply_fp32_ms": 0.123456789} for n in range(5)}, "cases": [case] * 49 + [dict(case, status=4)]},
+               large_matrix=[case] * 24, batched={"workload": "w" * 300, "solves_per_s": 377.82819, "vs_oracle": {"per_solve": solves}},
+               solve_alg_gbs_note="n" * 400)
+    line = bench.result_line(rec)
+    assert len(json.dumps(line)) < 4000 < len(json.dumps(rec))
+    for k in bench.CONTRACT:
+        assert line[k] == (rec[k] if k != "roofline" else {"frac": 0.5}), k
+    assert line["size_sweep"]["cases"] == {"results": 50, "converged": 49}
+    assert line["large_matrix"] == {"results": 24, "converged": 24}
+    assert line["batched"] == {"solves_per_s": 377.83, "vs_oracle": {}}
