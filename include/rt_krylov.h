@@ -263,7 +263,14 @@ rt_status rt_arnoldi_mgs(rt_problem* prob, double* V_dev, int32_t j, double* w_d
    vectors share its block (d <= i mod RT_GRAM_BLOCK).  For the new vector,
    row j+1 gets exactly those columns, d = 1..(j+1) mod RT_GRAM_BLOCK; its
    other columns are left as they are.  V_dev, w_dev, h_dev and the limits
-   as rt_arnoldi_mgs.  The copies it makes are waited for with a bound:
+   as rt_arnoldi_mgs.
+   Accuracy: h_{j+1} and v_{j+1} to FP64 rounding relative to what is left of
+   w, however small that is.  h_0..h_j to FP64 rounding of |w| |v_i|: some of the
+   dots are summed exactly over products of 58-bit fixed-point numbers, scaled
+   by the largest of 1984 entries of w and of the basis at most, so that a dot
+   loses accuracy relative to the sum of |w_n v_n| (as each update of w does)
+   where w is large only where v_i is small.  Numbers below 2^-1022 count as
+   zeros there.  The copies it makes are waited for with a bound:
    rt_problem_check reports one that gave up. */
 #define RT_GRAM_BLOCK 4
 rt_status rt_arnoldi_bmgs(rt_problem* prob, double* V_dev, int32_t j, double* w_dev, double* gram_dev,

@@ -278,10 +278,15 @@ struct BicgDev {
 //             column per |mu| and pair of frequencies p, Nnu-1-p
 enum CoefShare { CS_RAY = 0, CS_MU = 1, CS_PAIR = 2 };
 // Vector length from which a symmetric profile takes the paired FP64 kernels
-// (k_psweep, moments_pair64).  Above it the FP64 pipe bounds the apply and
-// sharing the work of a pair pays (N = 51.5 million: 621 -> 425 us); below, the quarter of the units is bound by latency
-// (N = 47,040: 17.5 -> 18.2 us; N = 1.9 million: 38.9 -> 35.5 us, not worth
-// another rounding of the operator, which BiCGSTAB and CGS amplify).
+// (k_psweep, moments_pair64), DELO-parabolic excepted (its steps differ between
+// the directions).  They are the faster ones at every length measured
+// (back-to-back applies, general and paired kernels: N = 0.25 million 14.6 and
+// 13.0 us, 1.0 million 24.3 and 23.2, 1.9 million 32.7 and 32.0, 2.9 million 46.8
+// and 41.5, 4.2 million 68.5 and 56.7, 8.4 million 125 and 99, 16.7 million 215
+// and 152).  The line is not where they cross: it keeps the operator of shorter
+// vectors to the bit what it was, at a cost of up to 11% of an apply, because
+// BiCGSTAB and CGS turn a last-bit change of it into 2e-8 of a solution to 1e-8
+// (N = 1.9 million; 4e-8 at 8.4 million, where the gain of a quarter counts more).
 constexpr int64_t kPairMinN = (int64_t)4 << 20;
 __host__ __device__ __forceinline__ int pair_count(int Nnu) { return (Nnu + 1) / 2; }
 __host__ __device__ __forceinline__ int64_t coef_col(int64_t r, int Nh, int Nnu, int shared) {

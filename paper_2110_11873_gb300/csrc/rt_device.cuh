@@ -325,34 +325,13 @@ constexpr double pow_ln2(int k) { return k == 0 ? 1.0 : kLn2 * pow_ln2(k - 1); }
 constexpr double fact(int k) { return k <= 1 ? 1.0 : k * fact(k - 1); }
 constexpr float kB(int n) { return (float)((n % 2 ? -1.0 : 1.0) * pow_ln2(n + 1) / fact(n + 2)); }
 
-// DELO-linear coefficients in FP32 from D2 = Delta / ln 2 and iD = 1 / Delta:
-// one series where Delta < 1/2 (h = beta / Delta, from which alpha follows with
-// its relative accuracy), the closed forms above; both are evaluated and one
-// is selected.
-__device__ __forceinline__ void delo_coeffs(float D2, float iD, float& e, float& al, float& be) {
-  e = ex2_approx(-D2);
-  float hb = kB(7);
-  hb = fmaf(hb, D2, kB(6));
-  hb = fmaf(hb, D2, kB(5));
-  hb = fmaf(hb, D2, kB(4));
-  hb = fmaf(hb, D2, kB(3));
-  hb = fmaf(hb, D2, kB(2));
-  hb = fmaf(hb, D2, kB(1));
-  hb = fmaf(hb, D2, kB(0));
-  const float bs = hb * D2;
-  const float onep = fmaf(D2, (float)kLn2, 1.0f);
-  const float as = D2 * fmaf(-onep, hb, (float)kLn2);
-  const float q = fmaf(-e, iD, iD);
-  const bool thin = D2 < kSeriesD2;
-  be = thin ? bs : 1.0f - q;
-  al = thin ? as : q - e;
-}
-
-// The same for two steps at once, one in each half of the packed FP32
-// instructions, with the same operations and rounding: half of a step's
-// instructions are its coefficients.  The register-ring solver (sweep) gains
-// (N_s = 333, 10 x 55 rays: 20.5 -> 17.1 us an apply); the staged one
-// (rt_tma.cu), which waits on memory, does not.
+// DELO-linear coefficients of two steps in FP32 from D2 = Delta / ln 2 and iD = 1
+// / Delta, one step in each half of the packed FP32 instructions: one series where
+// Delta < 1/2 (h = beta / Delta, from which alpha follows with its relative
+// accuracy), the closed forms above; both are evaluated and one is selected.  Half
+// of a step's instructions are its coefficients.  The register-ring solver (sweep)
+// gains over one step at a time (N_s = 333, 10 x 55 rays: 20.5 -> 17.1 us an
+// apply); the staged one (rt_tma.cu), which waits on memory, does not.
 __device__ __forceinline__ void delo_coeffs2(float2 D2, float2 iD, float2& e, float2& al, float2& be) {
   auto two = [](float c) { return make_float2(c, c); };
   e = make_float2(ex2_approx(-D2.x), ex2_approx(-D2.y));
@@ -373,13 +352,10 @@ __device__ __forceinline__ void delo_coeffs2(float2 D2, float2 iD, float2& e, fl
   al = make_float2(D2.x < kSeriesD2 ? as.x : at.x, D2.y < kSeriesD2 ? as.y : at.y);
 }
 
-// FP32 step coefficients from Delta.  DELO-linear with a series of its own for
-// alpha and beta behind a branch took about twice the instructions.
+// FP32 step coefficients from Delta, implicit Euler and trapezoidal
 template <int FS>
 __device__ __forceinline__ void coeffs32(float D, float& e, float& al, float& be) {
-  if (FS == RT_FS_DELO_LINEAR) {
-    delo_coeffs(D * (float)(1.0 / kLn2), __fdividef(1.0f, D), e, al, be);
-  } else if (FS == RT_FS_IMPLICIT_EULER) {
+  if (FS == RT_FS_IMPLICIT_EULER) {
     e = __frcp_rn(1.0f + D);
     al = 0.0f;
     be = D * e;
@@ -394,7 +370,7 @@ __device__ __forceinline__ void coeffs32(float D, float& e, float& al, float& be
 // coefficients of two steps from their Delta
 template <int FS>
 __device__ __forceinline__ void coeffs32x2(float D0, float D1, float2& e, float2& al, float2& be) {
-  if (FS == RT_FS_DELO_LINEAR) {
+  if constexpr (FS == RT_FS_DELO_LINEAR) {
     constexpr float c = (float)(1.0 / kLn2);
     delo_coeffs2(make_float2(D0 * c, D1 * c), make_float2(__fdividef(1.0f, D0), __fdividef(1.0f, D1)), e, al, be);
   } else {

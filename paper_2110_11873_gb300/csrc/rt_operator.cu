@@ -299,7 +299,8 @@ __global__ void k_jacobi_weights(const double* __restrict__ wray, const double* 
 // Two CTAs to an SM (128 registers a lane): with a ring of 16 steps, which FP64
 // vectors hold unconverted, a lane took 138 to 226 registers, so that more ray
 // groups than SMs ran in two waves and fewer had half the warps to hide their
-// recurrences.
+// recurrences (apply of 466 heights of 58 x 138 rays, trapezoidal: 63.7 -> 49.7 us;
+// FP32-refinement Jacobi-GMRES on 100 x 62 x 201: 20.3 -> 14.5 ms).
 template <typename TC, typename TV, int FS, int MODE, int NSPLIT, int RING, int MAXT>
 __global__ void __launch_bounds__(32 * MAXT, 2) k_formal(const FormalArgs A) {
   constexpr int NS = 2 / NSPLIT;   // Stokes parameters per lane

@@ -136,8 +136,9 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* tm) {
 //   trapezoidal: op.z = dtau; h = Delta / 2, q = 1 / (1 + h), e = (1 - h) q,
 //     alpha = beta = h q.
 //   (reciprocals by the hardware approximation, within 2 ulp)
-// DELO-linear as delo_coeffs, written out: calling it forms 1 / Delta ahead of
-// the series and took 131.1 us instead of 130.4 on N = 51.5 million.
+// DELO-linear as delo_coeffs2, one step at a time and written out: a function of
+// D2 and 1 / Delta forms 1 / Delta ahead of the series and took 131.1 us instead
+// of 130.4 on N = 51.5 million.
 template <int FS>
 __device__ __forceinline__ void step_coeffs(const float4& op, float rsc, float irsc, float& e, float& al, float& be) {
   if (FS == RT_FS_DELO_LINEAR) {
